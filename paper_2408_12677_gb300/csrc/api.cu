@@ -72,7 +72,7 @@ struct gs_ctx {
   float* loss_partials = nullptr;
   float* tune_img = nullptr;  // zero image gradients for the autotuner
   float* dl_img = nullptr;    // per pixel: dL/dcolor (3 planes) and the depth residual sign (fused loss)
-  float* tile_loss = nullptr;  // per (tile, 8 x 8 block): fused-loss partial sums (3 floats)
+  float* tile_loss = nullptr;  // per warp job of the forward raster pass: fused-loss partial sums (3 floats)
   float* d_dscale = nullptr;   // per view: depth-gradient scale of the fused loss
   uint32_t* d_nvalid = nullptr;  // per view: target depths > 0 seen by the fused-loss forward pass
   // per-frame seeding scratch
@@ -297,7 +297,7 @@ gs_status ensure_tiles(gs_ctx* c, int64_t t) {
   GS_GROW(c, cap_t, regrow(&c->tcursor, cap));
   GS_GROW(c, cap_t, regrow(&c->torder, cap));
   GS_GROW(c, cap_t, regrow(&c->scan_aux, tile_scan_aux_size(cap)));
-  GS_GROW(c, cap_t, regrow(&c->tile_loss, 12 * cap));
+  GS_GROW(c, cap_t, regrow(&c->tile_loss, 3 * kMaxTileJobs * cap));
   c->cap_t = cap;
   c->have_state = false;
   return GS_OK;
@@ -1230,7 +1230,8 @@ gs_status render_bwd_adam_views(gs_ctx* c, const gs_gaussians* g, int32_t V, con
       ad.step_dev = c->d_step;
     }
     LossFoldArgs L{};
-    if (lf) {  // the forward pass's loss partials (per tile and 8 x 8 block)
+    if (lf) {  // the forward pass's loss partials (per tile and warp job)
+      const int64_t jobs = raster_jobs_per_tile((uint32_t)c->st_tiles, c->num_sms);
       L.partials = c->tile_loss;
       L.blk = c->loss_partials;
       L.out = lf->loss;
@@ -1243,10 +1244,10 @@ gs_status render_bwd_adam_views(gs_ctx* c, const gs_gaussians* g, int32_t V, con
       for (int k = 0; k < c->st_views; ++k) {
         const int64_t t1 = k + 1 < c->st_views ? (int64_t)c->st_map.tile_base[k + 1] : c->st_tiles;
         L.block_base[k] = blocks;
-        L.job_base[k] = 4u * c->st_map.tile_base[k];
-        L.job_base[k + 1] = (uint32_t)(4 * t1);
+        L.job_base[k] = (uint32_t)(jobs * c->st_map.tile_base[k]);
+        L.job_base[k + 1] = (uint32_t)(jobs * t1);
         L.npix[k] = (float)c->st_w[k] * (float)c->st_h[k];
-        blocks += (int)((4 * (t1 - (int64_t)c->st_map.tile_base[k]) + kLossChunk - 1) / kLossChunk);
+        blocks += (int)((jobs * (t1 - (int64_t)c->st_map.tile_base[k]) + kLossChunk - 1) / kLossChunk);
       }
       L.block_base[c->st_views] = blocks;
       L.blocks = blocks;

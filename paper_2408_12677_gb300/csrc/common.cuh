@@ -49,6 +49,7 @@ struct RasterParams {
   float log2_alpha_min;  // log2(alpha_min)
   float qmax_s;          // 9 * 0.5 log2(e): the 3-sigma bound on q'
   float t_eps;
+  float log2_clamp;      // an entry whose log2 opacity is not above this never reaches alpha_max
 };
 
 // ---------------------------------------------------------------------------

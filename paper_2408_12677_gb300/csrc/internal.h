@@ -88,7 +88,7 @@ struct AdamArgs {
 // The training step's loss reduction, done by the fused backward + Adam
 // kernel's first blocks before their own work (out nullable): reduction
 // block b (of `blocks`; view v's from block_base[v]) sums kLossChunk
-// consecutive (tile, 8 x 8 block) partials {|colour residual|, |depth
+// consecutive warp job partials {|colour residual|, |depth
 // residual| over valid targets, valid count} of one view, starting at
 // job_base[v] + (b - block_base[v]) kLossChunk, into blk[3 b + k] in a fixed
 // order; the block completing the last one (ticket: 0 between launches)
@@ -259,9 +259,9 @@ struct RasterArgs {
   uint32_t* work;         // nullable: job counter of the persistent form
   bool zero_work;         // the launcher zeroes *work first (it is not known to be 0)
   int num_sms;
-  // fused loss (forward): per (tile, 8 x 8 block) partial sums {|colour
-  // residual|, |depth residual| over valid targets, valid count} at
-  // loss_partials[3 (4 tile + block) + i]; null = no loss
+  // fused loss (forward): per warp job partial sums {|colour residual|,
+  // |depth residual| over valid targets, valid count} at
+  // loss_partials[3 (raster_jobs_per_tile tile + job) + i]; null = no loss
   float* loss_partials;
   float w_color;
   // backward: dL/dD = dLdd * depth_scale[v] when non-null (the scale the
@@ -285,6 +285,11 @@ struct RasterArgs {
   RasterView v[kMaxViews];
 };
 bool raster_shape_supported(int tw, int th);
+// pixels per lane of the raster passes (4, 2 or 1) and the warp jobs (regions
+// of 32 px per lane pixels, one loss partial each) that a tile then has
+int raster_px_per_lane(uint32_t n_tiles, int num_sms);
+inline int raster_jobs_per_tile(uint32_t n_tiles, int num_sms) { return 8 / raster_px_per_lane(n_tiles, num_sms); }
+constexpr int kMaxTileJobs = 8;
 // bounds-checked build: point the translation unit's kernels at the
 // context's bounds word (no-op in the normal build)
 cudaError_t raster_bind_bounds(uint32_t* word);
@@ -294,7 +299,7 @@ void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsig
 // loss from the forward pass's per-block partials: loss = sum over views of
 // w_color sum|rc| / (3 npix_v) + w_depth sum|rd| / nvalid_v; depth_scale[v] =
 // w_depth / nvalid_v (fixed summation order)
-// partials: scratch of >= 3 * (4 n_tiles / 2048 + views) floats; ticket: a
+// partials: scratch of >= 3 * (kMaxTileJobs n_tiles / 2048 + views) floats; ticket: a
 // device word that is 0 between launches (one launch; its last block
 // finalises and resets it); step (nullable): the device Adam step counter,
 // advanced by one after the loss is final

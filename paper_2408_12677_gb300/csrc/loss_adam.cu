@@ -141,10 +141,10 @@ __global__ void __launch_bounds__(kLossThreads) scale_kernel(const __grid_consta
 }
 
 // Loss of the fused forward pass, phase 1: block b sums, in a fixed order,
-// the (tile, 8 x 8 block) partials [lo, lo + kTileLossChunk) of one view
+// the warp job partials [lo, lo + kTileLossChunk) of one view
 // into partials[3 b ..] (the layout of loss_partials_kernel's output, so
 // loss_finalize_kernel finishes the job).  View v owns blocks
-// [block_base[v], block_base[v + 1]) and job partials [4 tile_base[v], 4 tile_base[v + 1]).
+// [block_base[v], block_base[v + 1]) and the job partials of its tiles.
 constexpr int kTileLossChunk = kLossThreads * kLossItems;
 
 struct TileLossArgs {
@@ -154,7 +154,7 @@ struct TileLossArgs {
   const float* jobs;
 };
 
-// One launch: every block sums its chunk of the per-(tile, block) partials;
+// One launch: every block sums its chunk of the warp job partials;
 // the last block to finish (a ticket counter, reset by that block) then
 // finalises the loss and the depth scales over all blocks' partials in block
 // order (so the result does not depend on which block is last), and, given
@@ -343,9 +343,10 @@ void launch_loss_tiles_finalize(const RasterArgs& a, float w_depth, float* loss,
   la.w_depth = w_depth;
   la.loss = loss;
   int blocks = 0;
+  const uint32_t jobs = (uint32_t)raster_jobs_per_tile(a.n_tiles, a.num_sms);
   for (int v = 0; v < a.views; ++v) {
-    const uint32_t j0 = 4 * a.v[v].tile_base;
-    const uint32_t j1 = 4 * (v + 1 < a.views ? a.v[v + 1].tile_base : a.n_tiles);
+    const uint32_t j0 = jobs * a.v[v].tile_base;
+    const uint32_t j1 = jobs * (v + 1 < a.views ? a.v[v + 1].tile_base : a.n_tiles);
     t.block_base[v] = blocks;
     t.job_base[v] = j0;
     t.job_base[v + 1] = j1;

@@ -2,16 +2,24 @@
 // transmittance) and backward (back to front from the stored last
 // contributor, transmittance recomputed from the stored final T).
 //
-// One CTA of 128 threads per tile; each warp owns an 8 x 8 pixel block of it,
-// each thread two pixels (rows y and y + 4), and the four warps run
-// independently (no block barriers).  A warp walks the tile's depth-sorted
-// list in chunks of 32 entries with the next chunk's 48 B records already in
-// flight, converts the records to tile-local coordinates (so per-pixel offsets
-// keep float32 precision), keeps the entries whose support bounding box meets
-// its block (ballot) and evaluates only those.  The backward pass adds each
-// Gaussian's gradient to its global record with per-lane vector atomics when
-// few lanes contribute, else after a transposed shuffle reduction over the
-// warp with one warp-wide atomic.
+// A warp owns a region of a tile's 256 pixels and its lanes form groups, each
+// with a small block of the region (WarpMap).  The warp walks the tile's
+// depth-sorted list with the records of the next 32 entries already in flight,
+// converts them to tile-local coordinates (so per-pixel offsets keep float32
+// precision) and finds which entries' support boxes meet which group's block;
+// every group then takes its own next entry, so one warp iteration evaluates
+// up to 32 (forward) or 16 (backward) different Gaussians, each on a block of
+// the size of a small splat.  The backward pass sums a Gaussian's gradient over
+// the group with shuffles and adds it to the global record with vector atomics.
+//
+// Both passes are bound by instruction issue (70% and 66% of cycles issue, the
+// ALU and FMA pipes 41% and 50% busy, DRAM 7%).  With one 8 x 8 block per warp
+// and one list for all 32 lanes, a splat of 4-5 px met 2.95 evaluated pixels
+// per blended one and each (warp, entry) hit paid its list handling and its
+// reduction for 16 blended pixels; lists per group evaluate 1.76 (forward) and
+// 1.96 (backward), and one reduction serves 16 Gaussians: 85 -> 64 us and
+// 168 -> 100 us at 1200 x 680 with 300k Gaussians, 811 -> 654 us and 1759 ->
+// 1110 us for five such views.
 #include <algorithm>
 
 #include "common.cuh"
@@ -21,19 +29,50 @@ namespace gs {
 
 namespace {
 
-constexpr int kThreads = 128;  // 4 independent warps per CTA, one 8 x 8 pixel block each
-// Backward pass: when at most this many lanes contribute to a Gaussian, each
-// adds its ten values with three 16-byte vector atomics (3 issue slots)
-// instead of the warp reduction (about 45); the kernel is issue-bound, and
-// up to this many lanes the L2 atomic units keep up (at 32 they saturate).
-constexpr int kAtomicLanes = 16;
+constexpr int kThreads = 128;  // 4 independent warps per CTA
 constexpr unsigned kFull = 0xFFFFFFFFu;
+// Lanes per group (see WarpMap).  Forward: each lane by itself, its 1 x PPL
+// pixels need no sums over lanes (65.3 -> 64.0 us at 1200 x 680, 675 -> 654 us
+// for five such views with longer lists, against groups of two).  Backward:
+// smaller blocks evaluate fewer pixels that take no part, larger ones make
+// fewer atomics: 2 lanes x 4 pixels (104 us; 4 lanes 112, 1 lane 121 us), and
+// 4 lanes x 2 or 1 pixels (2 x 2 would make too many: 92 us instead of 59 us
+// on a map of large splats, 28.0 instead of 29.9 us on one of small ones).
+constexpr int kFwdLanes = 1;
+template <int PPL>
+constexpr int kBwdLanes = PPL == 4 ? 2 : 4;
+// CTAs per SM (registers: 80 and 96 per thread)
+constexpr int kFwdCtas = 6, kBwdCtas = 5;
+
+// Pixels of a warp: a region of RW x RH pixels, lane l with the PPL pixels of
+// column l % RW from row PPL (l / RW) on (one column: dx, t0 and the column's
+// constants are computed once per entry for PPL pixels).  LPG neighbouring
+// lanes are a group, its LPG x PPL pixels a block.  A tile has JOBS regions
+// (warp jobs).
+template <int TW, int TH, int PPL, int LPG_>
+struct WarpMap {
+  static constexpr int LPG = LPG_;
+  static constexpr int ROWS = PPL;  // rows of a block
+  static constexpr int RW = PPL == 4 && TW >= 16 ? 16 : 8;
+  static constexpr int RH = 32 * PPL / RW;
+  static constexpr int JOBS = TW * TH / (RW * RH);
+  static_assert(TW * TH == 256 && TW % RW == 0 && TH % RH == 0 && JOBS == 8 / PPL, "regions tile the tile");
+};
 
 // One list entry in tile-local coordinates:
-//   a = {mu_x, mu_y, i0, k}, b = {i1, log2 opacity, z, support radius r2},
-//   c = {r, g, b, mask of the warp block's halves the support box meets}
+//   a = {mu_x, mu_y, i0, -k}, b = {i1, log2 opacity, z, support radius r2},
+//   c = {r, g, b, item id}
 struct Entry {
   float4 a, b, c;
+};
+
+// Shared memory of a warp: the converted entries of four chunks of 32 (slot
+// kRing is an entry that no pixel accepts, read by groups that have none), and
+// the raw records of the next chunk.
+constexpr int kRing = 128;
+struct WarpSmem {
+  Entry e[kRing + 1];
+  float4 raw[32][3];
 };
 
 // A list entry's item id; the checked build redirects an id beyond the
@@ -50,39 +89,177 @@ __device__ __forceinline__ void cp_record(float4* dst, const float4* __restrict_
   for (int k = 0; k < 3; ++k)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d + 16u * k), "l"(src + k) : "memory");
 }
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // Converts a gathered record to tile-local coordinates and tests the splat's
-// support bounding box against the two halves of the warp's 8 x 8 block:
-// rows [by, by + 4) (bit 0, the lanes' first pixels) and [by + 4, by + 8)
-// (bit 1, their second pixels), columns [bx, bx + 8).  The box holds every
-// pixel the per-pixel test can accept: q' <= min(qmax, log2 o - log2 alpha_min)
-// is the ellipse (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents
-// sqrt(R2) / i0 and sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2); the widening covers
-// float32 rounding of the test.  Returns the mask of halves hit (0 = none);
-// the mask is warp-uniform per entry, so a half it excludes costs the warp
-// nothing.
+// support bounding box against the blocks of the warp's region, whose first
+// pixel is (bx, by): bit l of the result is set when the box meets the pixel
+// centres of lane l's block.  The box holds every pixel the per-pixel test can
+// accept: q' <= min(qmax, log2 o - log2 alpha_min) is the ellipse
+// (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents sqrt(R2) / i0 and
+// sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2); the widening covers float32 rounding
+// of the test and of the hardware square roots and reciprocals.
+template <class M>
 __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, float ox, float oy, float bx, float by,
-                                               const RasterParams& rp, Entry& e) {
+                                               const RasterParams& rp, uint32_t id, Entry& e) {
   const float mlx = __fadd_rn(__fsub_rn(f0.x, ox), f0.z);
   const float mly = __fadd_rn(__fsub_rn(f0.y, oy), f0.w);
   const float R2 = fminf(rp.qmax_s, __fsub_rn(f1.w, rp.log2_alpha_min));
-  e.a = make_float4(mlx, mly, f1.x, f1.y);
+  e.a = make_float4(mlx, mly, f1.x, -f1.y);
   e.b = make_float4(f1.z, f1.w, f2.w, R2);
+  e.c = make_float4(f2.x, f2.y, f2.z, __uint_as_float(id));
+  if (!(R2 > 0.f && f1.x > 0.f && f1.z > 0.f)) return 0u;
+  const float Rr = sqrt_approx(R2) * 1.0001f + 1e-4f;
+  const float inv0 = rcp_approx(f1.x), inv1 = rcp_approx(f1.z);
+  const float ex = Rr * inv0 + 1e-3f;
+  const float ey = Rr * sqrt_approx(f1.y * f1.y * inv0 * inv0 + inv1 * inv1) + 1e-3f;
+  // first and last block column and row whose centres lie within the box
+  constexpr float BW = M::LPG, BH = M::ROWS, NC = M::RW / M::LPG, NR = M::RH / M::ROWS;
+  const float rx = mlx - bx, ry = mly - by;
+  const int c0 = __float2int_ru(fmaxf((rx - ex + 0.5f) / BW - 1.f, 0.f));
+  const int c1 = __float2int_rd(fminf((rx + ex - 0.5f) / BW, NC - 1.f));
+  const int r0 = __float2int_ru(fmaxf((ry - ey + 0.5f) / BH - 1.f, 0.f));
+  const int r1 = __float2int_rd(fminf((ry + ey - 0.5f) / BH, NR - 1.f));
+  if (c1 < c0 || r1 < r0) return 0u;
+  constexpr unsigned kRow = M::RW == 32 ? kFull : (1u << M::RW) - 1u;
+  const unsigned xm = (kRow >> (M::RW - M::LPG * (c1 - c0 + 1))) << (M::LPG * c0);
   unsigned m = 0u;
-  if (R2 > 0.f && f1.x > 0.f && f1.z > 0.f) {
-    const float Rr = sqrtf(R2) * 1.0001f + 1e-4f;
-    const float inv0 = rcp_approx(f1.x), inv1 = rcp_approx(f1.z);
-    const float ex = Rr * inv0 + 1e-3f;
-    const float ey = Rr * sqrtf(f1.y * f1.y * inv0 * inv0 + inv1 * inv1) + 1e-3f;
-    if (mlx + ex >= bx + 0.5f && mlx - ex <= bx + 7.5f) {
-      const float y0 = mly - ey, y1 = mly + ey;
-      m = ((y1 >= by + 0.5f && y0 <= by + 3.5f) ? 1u : 0u) | ((y1 >= by + 4.5f && y0 <= by + 7.5f) ? 2u : 0u);
+#pragma unroll
+  for (int r = 0; r < M::RH / M::ROWS; ++r) m |= r0 <= r && r <= r1 ? xm << (M::RW * r) : 0u;
+  return m;
+}
+
+// Transposes the 32 x 32 bit matrix whose row l is lane l's x: bit i of lane
+// l's result is bit l of lane i's x (32 ballots' worth in five exchanges).
+__device__ __forceinline__ unsigned warp_transpose(unsigned x, int lane) {
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const unsigned m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+    const unsigned y = __shfl_xor_sync(kFull, x, s);
+    x = lane & s ? (x & ~m) | ((y >> s) & m) : (x & m) | ((y << s) & ~m);
+  }
+  return x;
+}
+
+// The walk of a tile's list, DIR = 1 from its front, DIR = -1 from its entry
+// n - 1 backwards, in aligned chunks of 32 entries.  Offsets count entries of
+// whole chunks from the walk's first chunk on.  Up to four chunks are held
+// converted in shared memory (a ring), [base, top); each group has a bit per
+// held entry that meets its block, and takes its own next one whatever the
+// others do, up to four chunks ahead of the slowest: the groups of a warp meet
+// different numbers of entries per chunk, and these even out over the window
+// (with every group waiting at each chunk's end, a third of them idled).  A
+// chunk is converted when a group runs dry; its records are in flight
+// (cp.async) since the chunk before, the ids of one more in a register.
+template <class M, int DIR>
+struct Walk {
+  const uint32_t* __restrict__ ids;  // of the list's entry 0
+  const float4* __restrict__ feat;
+  WarpSmem* sm;
+  int n, lane;
+  uint32_t n_items;
+  float ox, oy, bx, by;
+  uint32_t g_raw, g_next;     // ids of the chunk in flight and of the one after
+  int first;                  // first entry of the walk's first chunk
+  int end;                    // offset behind the last chunk
+  int base, top;              // held chunks
+  int off;                    // the group's chunk; off = top: waiting for the next one
+  unsigned cur, w1, w2, w3;   // its remaining entries there and in the three chunks after (first one highest)
+  int met = 0;                // one past the last entry met so far (DIR > 0)
+
+  __device__ __forceinline__ int chunk(int o) const { return DIR > 0 ? o : first - o; }
+  __device__ __forceinline__ uint32_t id_at(int o) const {
+    const int i = chunk(o) + lane;
+    return o < end && i < n ? checked_id(__ldg(&ids[i]), n_items) : 0u;
+  }
+  __device__ __forceinline__ void fetch(int o) {  // the chunk at o into flight
+    g_raw = g_next;
+    if (o < end && chunk(o) + lane < n) cp_record(sm->raw[lane], feat, g_raw);
+    g_next = id_at(o + 32);
+  }
+  __device__ __forceinline__ void begin() {
+    first = DIR > 0 ? 0 : ((n - 1) >> 5) << 5;
+    end = (n + 31) & ~31;
+    base = top = off = 0;
+    cur = w1 = w2 = w3 = 0u;
+    g_next = id_at(0);
+    fetch(0);
+  }
+  // Converts the chunk at `top` and puts the following one into flight;
+  // returns its entries that meet the lane's group (bit i: entry i).
+  __device__ __forceinline__ unsigned stage(const RasterParams& rp) {
+    cp_wait_all();
+    Entry e;
+    unsigned m = 0u;
+    if (chunk(top) + lane < n) {
+      const float4* raw = sm->raw[lane];
+      m = make_entry<M>(raw[0], raw[1], raw[2], ox, oy, bx, by, rp, g_raw, e);
+    }
+    __syncwarp();  // every lane has read its last entry of the chunk that is overwritten
+    if (m) sm->e[(top & (kRing - 1)) + lane] = e;
+    fetch(top + 32);
+    __syncwarp();  // the entries are stored before any lane reads them
+    return warp_transpose(m, lane);
+  }
+  __device__ __forceinline__ void push(unsigned mine) {  // the staged chunk's entries
+    if (DIR > 0) {
+      if (mine) met = top + 32 - __clz(mine);
+      mine = __brev(mine);
+    }
+    const int r = top - off;
+    cur = r == 0 ? mine : cur;
+    w1 = r == 32 ? mine : w1;
+    w2 = r == 64 ? mine : w2;
+    w3 = r == 96 ? mine : w3;
+    top += 32;
+  }
+  __device__ __forceinline__ bool can_stage() const { return top < end && top - base < kRing; }
+  __device__ __forceinline__ bool any_up_to(int lim) const { return __any_sync(kFull, cur != 0u && off <= lim); }
+  // What the warp does next when no group is dry or no chunk can be staged
+  // (`can`): >= 0: take entries, without `can` while a group has one at an
+  // offset up to the result (everything is staged: anywhere; the ring is full:
+  // in the oldest chunk); kAgain: the oldest chunk was given up, kEnd: done.
+  static constexpr int kAgain = -1, kEnd = -2;
+  __device__ __forceinline__ int limit(bool can) {
+    if (can) return 0;
+    if (top >= end) return __any_sync(kFull, cur != 0u) ? end : kEnd;
+    if (any_up_to(base)) return base;
+    base += 32;
+    return kAgain;
+  }
+  __device__ __forceinline__ void drop() {  // the group takes no more entries
+    cur = w1 = w2 = w3 = 0u;
+    off = top;
+  }
+  __device__ __forceinline__ void step() {  // to the group's next chunk when it is done with this one
+    if (cur == 0u && off < top) {
+      cur = w1;
+      w1 = w2;
+      w2 = w3;
+      w3 = 0u;
+      off += 32;
     }
   }
-  e.c = make_float4(f2.x, f2.y, f2.z, __uint_as_float(m));
-  return m;
+  // The group's next entry: its slot in sm->e (kRing: none), idx = its place in the list.
+  __device__ __forceinline__ int take(int& idx) {
+    const int z = __clz(cur);  // 32: none
+    const int j = DIR > 0 ? z : 31 - z;
+    const int slot = cur ? (off & (kRing - 1)) + j : kRing;
+    idx = chunk(off) + j;
+    cur &= ~(0x80000000u >> (z & 31));
+    step();
+    return slot;
+  }
+};
+
+// Slot kRing of a warp's entries: support radius -1, accepted by no pixel.
+__device__ __forceinline__ void init_warp_smem(WarpSmem& sm) {
+  if ((threadIdx.x & 31) == 0) {
+    sm.e[kRing].a = make_float4(0.f, 0.f, 1.f, 0.f);
+    sm.e[kRing].b = make_float4(1.f, -126.f, 0.f, -1.f);
+    sm.e[kRing].c = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __syncwarp();
 }
 
 // Tile, view and pixel origin of visit k: k indexes the tile visit order (or
@@ -147,38 +324,6 @@ __device__ __forceinline__ uint32_t class_visit_tile(const RasterArgs& a, const 
   return __ldg(&a.cls_tiles[(size_t)c * a.cls_stride + (k - s_start[c + 1])]);
 }
 
-// Front-to-back step of one pixel for one list entry (Eq. 11 with the skip
-// and stop rules), without branches: a pixel that is done, outside the
-// support or would drop T below t_eps adds a weight of exactly 0.
-template <bool COUNT>
-__device__ __forceinline__ void blend_slot(const float4& a, const float4& bb, const float4& c, float plx, float ply,
-                                           const RasterParams& rp, int idx1, bool on, float& T, float& R, float& G,
-                                           float& B, float& D, int& last, bool& done, uint32_t& n_visit,
-                                           uint32_t& n_blend) {
-  const float dx = __fsub_rn(plx, a.x);
-  const float dy = __fsub_rn(ply, a.y);
-  const float t0 = __fmul_rn(a.z, dx);
-  const float t1 = __fmul_rn(bb.x, __fmaf_rn(-a.w, dx, dy));
-  const float q = __fmaf_rn(t0, t0, __fmul_rn(t1, t1));
-  const bool pass = on && !done && q <= bb.w;
-  const float al = fminf(rp.alpha_max, ex2_approx(__fsub_rn(bb.y, q)));
-  const float test_T = __fmul_rn(T, __fsub_rn(1.f, al));
-  const bool stop = pass && test_T < rp.t_eps;
-  const bool add = pass && !stop;
-  const float w = add ? al * T : 0.f;
-  R = fmaf(w, c.x, R);
-  G = fmaf(w, c.y, G);
-  B = fmaf(w, c.z, B);
-  D = fmaf(w, bb.z, D);
-  T = add ? test_T : T;
-  last = add ? idx1 : last;
-  if (COUNT) {
-    n_visit += (on && !done) ? 1u : 0u;
-    n_blend += add ? 1u : 0u;
-  }
-  done = done || stop;
-}
-
 // Two floats in one 64-bit register pair, for the packed FP32 instructions
 // add / sub / mul / fma .rn.f32x2: each rounds both halves exactly as the
 // scalar instruction would, and takes one issue slot for two operations per
@@ -191,8 +336,29 @@ __device__ __forceinline__ f2x f2_pack(float lo, float hi) {
   return r;
 }
 __device__ __forceinline__ f2x f2_bcast(float x) { return f2_pack(x, x); }
+// 1 if a <= b, else 0 (also for NaN)
+__device__ __forceinline__ float one_if_le(float a, float b) {
+  float d;
+  asm("set.le.f32.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+// 1 if a <= b and i < n, else 0
+__device__ __forceinline__ float one_if_le_and(float a, float b, int i, int n) {
+  float d;
+  asm("{\n .reg .pred p;\n setp.lt.s32 p, %3, %4;\n set.le.and.f32.f32 %0, %1, %2, p;\n}" : "=f"(d) : "f"(a), "f"(b), "r"(i), "r"(n));
+  return d;
+}
 __device__ __forceinline__ float f2_lo(f2x r) { return __uint_as_float((unsigned)(r & 0xFFFFFFFFull)); }
 __device__ __forceinline__ float f2_hi(f2x r) { return __uint_as_float((unsigned)(r >> 32)); }
+template <int N>
+__device__ __forceinline__ float f2_at(const f2x (&x)[N], int s) {
+  return s & 1 ? f2_hi(x[s / 2]) : f2_lo(x[s / 2]);
+}
+__device__ __forceinline__ f2x f2_add(f2x a, f2x b) {
+  f2x d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 __device__ __forceinline__ f2x f2_sub(f2x a, f2x b) {
   f2x d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -209,120 +375,153 @@ __device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
   return d;
 }
 
-// Forward pass of one 8 x 8 pixel block (quadrant `quad` of global tile
-// `tile`) by one warp; buf is the warp's shared staging buffer, s_raw the
-// two shared slots per lane that its Gaussians' records land in (cp.async).
-template <int TW, int TH, bool COUNT, bool LOSS>
+// x * s + y with the scalar s on both halves, as two scalar FMAs: they take the
+// FMA pipe as long as the packed one does, which would need s in both halves of
+// a register pair (raster_fwd 70.7 -> 65.3 us at 1200 x 680; the exponent's
+// scalars are better broadcast, since each serves two pairs).
+__device__ __forceinline__ f2x f2_fma_s(f2x x, float s, f2x y) {
+  return f2_pack(__fmaf_rn(f2_lo(x), s, f2_lo(y)), __fmaf_rn(f2_hi(x), s, f2_hi(y)));
+}
+
+// Forward pass of region `quad` of global tile `tile` by one warp.  Every
+// pixel's arithmetic is the scalar definition's, element for element (packed
+// f32x2 instructions on pairs of a lane's pixels).  The ALU pipe (compares,
+// selects, minima) has half the FMA pipe's rate, so per pixel it gets one
+// compare whose 0 / 1 result multiplies alpha: alpha = 0 leaves T and the sums
+// unchanged bit for bit.  A pixel that is done (or outside the image) has its
+// row coordinate set to infinity, so that no entry accepts it; the clamp and
+// the stop of a pixel are branches that most entries do not take.  Stored per
+// pixel: the final T and the number of list entries in front of the one that
+// it stopped at (of the last entry that meets its block if it did not stop).
+template <int TW, int TH, int PPL, bool COUNT, bool LOSS>
 __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams& rp, uint32_t tile, int quad,
-                                        Entry* __restrict__ buf, float4 (*__restrict__ s_raw)[32][3],
-                                        float* __restrict__ T_final_all,
+                                        WarpSmem& sm, float* __restrict__ T_final_all,
                                         int32_t* __restrict__ last_all, unsigned long long* __restrict__ counters) {
-  constexpr int WX = TW / 8;
+  using M = WarpMap<TW, TH, PPL, kFwdLanes>;
+  constexpr int NP = (PPL + 1) / 2;  // pairs of pixels per lane
   const TileJob job = tile_job_of<TW, TH>(a, tile);
   const RasterView& vw = a.v[job.v];
   const int width = vw.width, height = vw.height;
-  const uint32_t* __restrict__ ids = a.ids;
-  const float4* __restrict__ feat = a.feat;
   const int lane = threadIdx.x & 31;
-  const int bxi = (quad % WX) * 8, byi = (quad / WX) * 8;
-  const int lx = bxi + (lane & 7), ly0 = byi + (lane >> 3), ly1 = ly0 + 4;
-  const int px = job.ox + lx, py0 = job.oy + ly0, py1 = job.oy + ly1;
-  const bool in0 = px < width && py0 < height, in1 = px < width && py1 < height;
-  const float plx = (float)lx + 0.5f, ply0 = (float)ly0 + 0.5f, ply1 = (float)ly1 + 0.5f;
-  const float ox = (float)job.ox, oy = (float)job.oy, bx = (float)bxi, by = (float)byi;
-  const uint2 r = job.range;
-  const int n = (int)(r.y - r.x);
-  __syncwarp();  // the warp's previous job is done with buf
+  const int bxi = (quad % (TW / M::RW)) * M::RW, byi = (quad / (TW / M::RW)) * M::RH;
+  const int lx = bxi + lane % M::RW, ly = byi + PPL * (lane / M::RW);
+  const int px = job.ox + lx, py = job.oy + ly;
+  const float plx = (float)lx + 0.5f;
+  const float kInf = __int_as_float(0x7f800000);
+  __syncwarp();  // the warp's previous job is done with sm
 
-  float T0 = 1.f, R0 = 0.f, G0 = 0.f, B0 = 0.f, D0 = 0.f;
-  float T1 = 1.f, R1 = 0.f, G1 = 0.f, B1 = 0.f, D1 = 0.f;
-  int last0 = 0, last1 = 0;
-  uint32_t n_blend = 0, n_visit = 0;
-  bool done0 = !in0, done1 = !in1;
-  const f2x PLY = f2_pack(ply0, ply1), ONE2 = f2_pack(1.f, 1.f);
+  Walk<M, 1> walk;
+  walk.ids = a.ids + job.range.x;
+  walk.feat = a.feat;
+  walk.sm = &sm;
+  walk.n = (int)(job.range.y - job.range.x);
+  walk.lane = lane;
+  walk.n_items = a.n_items;
+  walk.ox = (float)job.ox;
+  walk.oy = (float)job.oy;
+  walk.bx = (float)bxi;
+  walk.by = (float)byi;
 
-  // software pipeline: chunk c's records in shared memory, chunk c + 32's in
-  // flight (cp.async), the ids of chunk c + 64 in a register
-  int cur = 0;
-  if (lane < n) cp_record(s_raw[0][lane], feat, checked_id(__ldg(&ids[r.x + lane]), a.n_items));
-  cp_commit();
-  uint32_t g2 = 32 + lane < n ? checked_id(__ldg(&ids[r.x + 32 + lane]), a.n_items) : 0u;
-  for (int c0 = 0; c0 < n; c0 += 32, cur ^= 1) {
-    if (__all_sync(kFull, done0 && done1)) break;
-    if (c0 + 32 + lane < n) cp_record(s_raw[cur ^ 1][lane], feat, g2);
-    cp_commit();
-    if (c0 + 64 + lane < n) g2 = checked_id(__ldg(&ids[r.x + c0 + 64 + lane]), a.n_items);
-    cp_wait_prev();
-    const bool have = c0 + lane < n;
-    Entry e;
-    const float4* raw = s_raw[cur][lane];
-    const bool hit = have && make_entry(raw[0], raw[1], raw[2], ox, oy, bx, by, rp, e) != 0u;
-    __syncwarp();
-    if (hit) buf[lane] = e;
-    unsigned bal = __ballot_sync(kFull, hit);
-    __syncwarp();
-    while (bal) {
-      const int j = __ffs(bal) - 1;
-      bal &= bal - 1;
-      const float4 a = buf[j].a;
-      const float4 bb = buf[j].b;
-      const float4 c = buf[j].c;
-      const unsigned halves = __float_as_uint(c.w);
-      // branch-free per pixel: every lane evaluates, predicates decide
-      // (a blend of weight 0 leaves R, G, B, D unchanged)
-      // both rows as straight-line code (independent chains; a row outside the
-      // support box runs with weight 0)
-      // a half the support box misses (warp-uniform) is skipped
-      if (halves == 3u) {
-        // blend_slot for both rows at once, element for element the same
-        // operations (packed f32x2)
-        const float dx = __fsub_rn(plx, a.x);
-        const float t0 = __fmul_rn(a.z, dx);
-        const f2x DY = f2_sub(PLY, f2_bcast(a.y));
-        const f2x WQ = f2_fma(f2_bcast(-a.w), f2_bcast(dx), DY);
-        const f2x TQ = f2_mul(f2_bcast(bb.x), WQ);
-        const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ, TQ));
-        const bool pass0 = !done0 && f2_lo(Q) <= bb.w, pass1 = !done1 && f2_hi(Q) <= bb.w;
-        const f2x ARG = f2_sub(f2_bcast(bb.y), Q);
-        const f2x AL = f2_pack(fminf(rp.alpha_max, ex2_approx(f2_lo(ARG))), fminf(rp.alpha_max, ex2_approx(f2_hi(ARG))));
-        const f2x TT = f2_pack(T0, T1);
-        const f2x TEST = f2_mul(TT, f2_sub(ONE2, AL));
-        const bool stop0 = pass0 && f2_lo(TEST) < rp.t_eps, stop1 = pass1 && f2_hi(TEST) < rp.t_eps;
-        const bool add0 = pass0 && !stop0, add1 = pass1 && !stop1;
-        const f2x WW = f2_mul(AL, TT);
-        const f2x W = f2_pack(add0 ? f2_lo(WW) : 0.f, add1 ? f2_hi(WW) : 0.f);
-        const f2x RR = f2_fma(W, f2_bcast(c.x), f2_pack(R0, R1));
-        const f2x GG = f2_fma(W, f2_bcast(c.y), f2_pack(G0, G1));
-        const f2x BB = f2_fma(W, f2_bcast(c.z), f2_pack(B0, B1));
-        const f2x DZ = f2_fma(W, f2_bcast(bb.z), f2_pack(D0, D1));
-        R0 = f2_lo(RR);
-        R1 = f2_hi(RR);
-        G0 = f2_lo(GG);
-        G1 = f2_hi(GG);
-        B0 = f2_lo(BB);
-        B1 = f2_hi(BB);
-        D0 = f2_lo(DZ);
-        D1 = f2_hi(DZ);
-        T0 = add0 ? f2_lo(TEST) : T0;
-        T1 = add1 ? f2_hi(TEST) : T1;
-        last0 = add0 ? c0 + j + 1 : last0;
-        last1 = add1 ? c0 + j + 1 : last1;
-        if (COUNT) {
-          n_visit += (done0 ? 0u : 1u) + (done1 ? 0u : 1u);
-          n_blend += (add0 ? 1u : 0u) + (add1 ? 1u : 0u);
-        }
-        done0 = done0 || stop0;
-        done1 = done1 || stop1;
-      } else if (halves == 1u) {
-        blend_slot<COUNT>(a, bb, c, plx, ply0, rp, c0 + j + 1, true, T0, R0, G0, B0, D0, last0, done0, n_visit,
-                          n_blend);
-      } else {
-        blend_slot<COUNT>(a, bb, c, plx, ply1, rp, c0 + j + 1, true, T1, R1, G1, B1, D1, last1, done1, n_visit,
-                          n_blend);
-      }
-    }
+  float ply[2 * NP];
+  f2x T[NP], R[NP], G[NP], B[NP], D[NP];
+  int stop[2 * NP];  // list entries in front of the one that the pixel stopped at
+#pragma unroll
+  for (int s = 0; s < 2 * NP; ++s) {
+    ply[s] = s < PPL && px < width && py + s < height ? (float)(ly + s) + 0.5f : kInf;
+    stop[s] = 0x7fffffff;
   }
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  const f2x ONE2 = f2_pack(1.f, 1.f);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    T[p] = ONE2;
+    R[p] = G[p] = B[p] = D[p] = 0;
+  }
+  uint32_t n_blend = 0, n_visit = 0;
+
+  if (walk.n > 0) {
+    walk.begin();
+    unsigned gone = 0u;  // 1: every pixel of the lane is done
+    for (;;) {
+      while (__any_sync(kFull, walk.cur == 0u && walk.off < walk.top)) walk.step();
+      const bool can = walk.can_stage();
+      if (can && __any_sync(kFull, (walk.cur | gone) == 0u)) {  // a lane is dry
+        bool out = true;
+#pragma unroll
+        for (int s = 0; s < PPL; ++s) out = out && ply[s] == kInf;
+        if (__all_sync(kFull, out)) break;
+        static_assert(M::LPG == 1, "a lane by itself");
+        gone = out ? 1u : 0u;
+        walk.push(walk.stage(rp));
+        if (out) walk.drop();
+        continue;
+      }
+      const int lim = walk.limit(can);
+      if (lim == walk.kEnd) break;
+      if (lim == walk.kAgain) continue;
+      do {
+        int idx;
+        const Entry& en = sm.e[walk.take(idx)];
+        const float4 ea = en.a, eb = en.b, ec = en.c;
+        const float dx = __fsub_rn(plx, ea.x);
+        const float t0 = __fmul_rn(ea.z, dx);
+        float al[2 * NP], in[2 * NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const f2x DY = f2_sub(f2_pack(ply[2 * p], ply[2 * p + 1]), f2_bcast(ea.y));
+          const f2x WQ = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
+          const f2x TQ = f2_mul(WQ, f2_bcast(eb.x));
+          const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ, TQ));
+          const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
+          al[2 * p] = ex2_approx(f2_lo(ARG));
+          al[2 * p + 1] = ex2_approx(f2_hi(ARG));
+          in[2 * p] = one_if_le(f2_lo(Q), eb.w);
+          in[2 * p + 1] = one_if_le(f2_hi(Q), eb.w);
+        }
+        if (eb.y > rp.log2_clamp) {
+#pragma unroll
+          for (int s = 0; s < 2 * NP; ++s) al[s] = fminf(rp.alpha_max, al[s]);
+        }
+        f2x AL[NP], TEST[NP];
+        float low = 1.f;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          // alpha, exactly 0 (so that T, R, G, B and D stay as they are) outside the support
+          AL[p] = f2_mul(f2_pack(al[2 * p], al[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
+          TEST[p] = f2_mul(T[p], f2_sub(ONE2, AL[p]));
+          low = fminf(low, fminf(f2_lo(TEST[p]), f2_hi(TEST[p])));
+        }
+        if (COUNT) {
+#pragma unroll
+          for (int s = 0; s < PPL; ++s) {
+            n_visit += eb.w > 0.f && ply[s] != kInf ? 1u : 0u;
+            n_blend += in[s] > 0.f && (s & 1 ? f2_hi(TEST[s / 2]) : f2_lo(TEST[s / 2])) >= rp.t_eps ? 1u : 0u;
+          }
+        }
+        if (low < rp.t_eps) {  // a pixel stops in front of this entry
+#pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const bool s0 = f2_lo(TEST[p]) < rp.t_eps, s1 = f2_hi(TEST[p]) < rp.t_eps;
+            AL[p] = f2_pack(s0 ? 0.f : f2_lo(AL[p]), s1 ? 0.f : f2_hi(AL[p]));
+            TEST[p] = f2_pack(s0 ? f2_lo(T[p]) : f2_lo(TEST[p]), s1 ? f2_hi(T[p]) : f2_hi(TEST[p]));
+            ply[2 * p] = s0 ? kInf : ply[2 * p];
+            ply[2 * p + 1] = s1 ? kInf : ply[2 * p + 1];
+            stop[2 * p] = s0 ? idx : stop[2 * p];
+            stop[2 * p + 1] = s1 ? idx : stop[2 * p + 1];
+          }
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const f2x W = f2_mul(AL[p], T[p]);
+          T[p] = TEST[p];
+          R[p] = f2_fma_s(W, ec.x, R[p]);
+          G[p] = f2_fma_s(W, ec.y, G[p]);
+          B[p] = f2_fma_s(W, ec.z, B[p]);
+          D[p] = f2_fma_s(W, eb.z, D[p]);
+        }
+      } while (can ? !__any_sync(kFull, (walk.cur | gone) == 0u) : walk.any_up_to(lim));
+    }
+    cp_wait_all();
+  }
   if (COUNT) {
     unsigned long long vb = n_blend, vv = n_visit;
 #pragma unroll
@@ -341,56 +540,40 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
   float* __restrict__ alpha = vw.alpha;
   float* __restrict__ T_final = T_final_all + vw.pix_base;
   int32_t* __restrict__ last_out = last_all + vw.pix_base;
-  if (in0) {
-    const size_t p = (size_t)py0 * width + px;
+  // L1 loss epilogue (Eq. 12 plus the depth term): the same residuals,
+  // signs and colour scale as the separate loss kernels, per-region sums
+  const float gscale_c = LOSS ? a.w_color / (3.f * (float)HW) : 0.f;
+  float sc = 0.f, sd = 0.f, nv = 0.f;
+#pragma unroll
+  for (int s = 0; s < PPL; ++s) {
+    if (!(px < width && py + s < height)) continue;
+    const size_t p = (size_t)(py + s) * width + px;
+    const float Tf = f2_at(T, s), Df = f2_at(D, s);
+    const float col[3] = {f2_at(R, s) + Tf * rp.bg[0], f2_at(G, s) + Tf * rp.bg[1], f2_at(B, s) + Tf * rp.bg[2]};
     if (color) {
-      color[p] = R0 + T0 * rp.bg[0];
-      color[HW + p] = G0 + T0 * rp.bg[1];
-      color[2 * HW + p] = B0 + T0 * rp.bg[2];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) color[(size_t)c * HW + p] = col[c];
     }
-    if (depth) depth[p] = D0;
-    if (alpha) alpha[p] = 1.f - T0;
-    T_final[p] = T0;
-    last_out[p] = last0;
-  }
-  if (in1) {
-    const size_t p = (size_t)py1 * width + px;
-    if (color) {
-      color[p] = R1 + T1 * rp.bg[0];
-      color[HW + p] = G1 + T1 * rp.bg[1];
-      color[2 * HW + p] = B1 + T1 * rp.bg[2];
-    }
-    if (depth) depth[p] = D1;
-    if (alpha) alpha[p] = 1.f - T1;
-    T_final[p] = T1;
-    last_out[p] = last1;
-  }
-  if constexpr (LOSS) {
-    // L1 loss epilogue (Eq. 12 plus the depth term): the same residuals,
-    // signs and colour scale as the separate loss kernels, per-block sums
-    const float gscale_c = a.w_color / (3.f * (float)HW);
-    float sc = 0.f, sd = 0.f, nv = 0.f;
-    const float* __restrict__ trgb = vw.trgb;
-    const float* __restrict__ tdep = vw.tdep;
-    float* __restrict__ ldc = vw.loss_dc;
-    float* __restrict__ ldd = vw.loss_dd;
-    auto score = [&](size_t p, float T, float Rc, float Gc, float Bc, float D) {
-      const float col[3] = {Rc + T * rp.bg[0], Gc + T * rp.bg[1], Bc + T * rp.bg[2]};
+    if (depth) depth[p] = Df;
+    if (alpha) alpha[p] = 1.f - Tf;
+    T_final[p] = Tf;
+    last_out[p] = min(stop[s], walk.met);
+    if constexpr (LOSS) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const float r = col[c] - __ldg(&trgb[(size_t)c * HW + p]);
+        const float r = col[c] - __ldg(&vw.trgb[(size_t)c * HW + p]);
         sc += fabsf(r);
-        ldc[(size_t)c * HW + p] = gscale_c * (float)((r > 0.f) - (r < 0.f));
+        vw.loss_dc[(size_t)c * HW + p] = gscale_c * (float)((r > 0.f) - (r < 0.f));
       }
-      const float td = __ldg(&tdep[p]);
+      const float td = __ldg(&vw.tdep[p]);
       const bool valid = td > 0.f;
-      const float rd = D - td;
+      const float rd = Df - td;
       sd += valid ? fabsf(rd) : 0.f;
       nv += valid ? 1.f : 0.f;
-      ldd[p] = valid ? (float)((rd > 0.f) - (rd < 0.f)) : 0.f;
-    };
-    if (in0) score((size_t)py0 * width + px, T0, R0, G0, B0, D0);
-    if (in1) score((size_t)py1 * width + px, T1, R1, G1, B1, D1);
+      vw.loss_dd[p] = valid ? (float)((rd > 0.f) - (rd < 0.f)) : 0.f;
+    }
+  }
+  if constexpr (LOSS) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       sc += __shfl_xor_sync(kFull, sc, off);
@@ -398,7 +581,7 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
       nv += __shfl_xor_sync(kFull, nv, off);
     }
     if (lane == 0) {
-      float* part = a.loss_partials + 3 * (4 * (size_t)job.tile + quad);
+      float* part = a.loss_partials + 3 * (M::JOBS * (size_t)job.tile + quad);
       part[0] = sc;
       part[1] = sd;
       part[2] = nv;
@@ -407,11 +590,11 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
   }
 }
 
-// Pulls the next (tile visit, quadrant) job for the calling warp from the
-// device counter `work`: jobs 4k .. 4k + 3 are the four quadrants of visit
-// k, so warps take the tiles in visit order (longest lists first) and a warp
-// that finishes early takes new work instead of waiting for the other
-// quadrants of its tile.  Returns false when all jobs are taken.
+// Pulls the next (tile visit, region) job for the calling warp from the
+// device counter `work`: a visit's JOBS regions are consecutive jobs, so warps
+// take the tiles in visit order (longest lists first) and a warp that
+// finishes early takes new work instead of waiting for the other regions of
+// its tile.  Returns false when all jobs are taken.
 __device__ __forceinline__ bool next_job(uint32_t* __restrict__ work, uint32_t n_jobs, uint32_t& job) {
   uint32_t j = 0;
   if ((threadIdx.x & 31) == 0) j = atomicAdd(work, 1u);
@@ -430,157 +613,93 @@ __device__ __forceinline__ uint32_t fwd_visit_tile(const RasterArgs& a, const ui
   return tile;
 }
 
-// PERSIST = false: one CTA per tile visit, warp w on quadrant w.  Otherwise
-// a persistent grid whose warps pull jobs from `work` with next_job.
-template <int TW, int TH, bool COUNT, bool LOSS, bool PERSIST>
-__global__ void __launch_bounds__(kThreads, 7) raster_fwd_kernel(const __grid_constant__ RasterArgs a, RasterParams rp,
+// `work` null: warp w of the grid on job w.  Otherwise a persistent grid whose
+// warps pull jobs from `work` with next_job.
+template <int TW, int TH, int PPL, bool COUNT, bool LOSS>
+__global__ void __launch_bounds__(kThreads, kFwdCtas) raster_fwd_kernel(const __grid_constant__ RasterArgs a, RasterParams rp,
                                                               float* __restrict__ T_final_all,
                                                               int32_t* __restrict__ last_all,
                                                               unsigned long long* __restrict__ counters,
                                                               uint32_t* __restrict__ work) {
   pdl_enter();
-  static_assert((TW / 8) * (TH / 8) == kThreads / 32, "four 8x8 warp blocks per tile");
-  __shared__ Entry s_e[kThreads / 32][32];
-  __shared__ __align__(16) float4 s_rawf[kThreads / 32][2][32][3];
+  constexpr uint32_t JOBS = 8 / PPL;
+  __shared__ __align__(16) WarpSmem s_w[kThreads / 32];
   __shared__ uint32_t s_start[kLenClasses + 1];  // bucket mode: tiles of class c or longer
   const int warp = threadIdx.x >> 5;
   if (a.cls_count) load_class_starts(a, s_start);  // CTA-uniform
-  if constexpr (!PERSIST) {
-    fwd_job<TW, TH, COUNT, LOSS>(a, rp, fwd_visit_tile(a, s_start, blockIdx.x, warp), warp, s_e[warp], s_rawf[warp],
-                                 T_final_all, last_all, counters);
+  init_warp_smem(s_w[warp]);
+  const uint32_t n_jobs = JOBS * a.n_tiles;
+  uint32_t job = blockIdx.x * (kThreads / 32) + warp;
+  while (work ? next_job(work, n_jobs, job) : job < n_jobs) {
+    const int quad = (int)(job % JOBS);
+    fwd_job<TW, TH, PPL, COUNT, LOSS>(a, rp, fwd_visit_tile(a, s_start, job / JOBS, quad), quad, s_w[warp], T_final_all,
+                                      last_all, counters);
+    if (!work) break;
+  }
+}
+
+// Adds x to the record's float4 `part` unless it is all zeros (a group without
+// a contribution, or without an entry).
+__device__ __forceinline__ void add_part(float* __restrict__ rec, int part, float a, float b, float c, float d) {
+  const unsigned bits = (__float_as_uint(a) | __float_as_uint(b) | __float_as_uint(c) | __float_as_uint(d)) & 0x7fffffffu;
+  if (bits) atomicAdd(reinterpret_cast<float4*>(rec) + part, make_float4(a, b, c, d));
+}
+
+// Sums the ten values v over the lanes of each group and adds the totals to
+// the group's record (12 floats: {s0 .. s3}, {s4, s5, depth, -}, {r, g, b, -})
+// with 16-byte vector atomics: four lanes exchange at distance 2 (v[0..6] to
+// the lower two, v[7..9] to the upper) and 1, after which lane l has float4 l
+// (11 shuffles for all groups of the warp at once); two lanes at distance 1
+// (float4 0 to the first lane, 1 and 2 to the second).
+template <int LPG>
+__device__ __forceinline__ void group_reduce_add10(const float (&v)[10], int lane, float* __restrict__ rec) {
+  if constexpr (LPG == 4) {
+    const bool b1 = lane & 2, l0 = (lane & 3) == 0, l1 = (lane & 3) == 1;
+    float u[7];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i] = (b1 ? v[7 + i] : v[i]) + __shfl_xor_sync(kFull, b1 ? v[i] : v[7 + i], 2);
+#pragma unroll
+    for (int i = 3; i < 7; ++i) u[i] = v[i] + __shfl_xor_sync(kFull, v[i], 2);
+    float x[4];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) x[i] = (l1 ? u[4 + i] : u[i]) + __shfl_xor_sync(kFull, l0 ? u[4 + i] : u[i], 1);
+    x[3] = u[3] + __shfl_xor_sync(kFull, u[3], 1);
+    if ((lane & 3) < 3) add_part(rec, lane & 3, x[0], x[1], x[2], l0 ? x[3] : 0.f);
   } else {
-    const uint32_t n_jobs = 4u * a.n_tiles;
-    uint32_t job;
-    while (next_job(work, n_jobs, job)) {
-      const int quad = (int)(job & 3u);
-      fwd_job<TW, TH, COUNT, LOSS>(a, rp, fwd_visit_tile(a, s_start, job >> 2, quad), quad, s_e[warp], s_rawf[warp],
-                                   T_final_all, last_all, counters);
-    }
+    static_assert(LPG == 2, "groups of 4 or 2 lanes");
+    const bool l1 = lane & 1;
+    float x[6];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = (l1 ? v[4 + i] : v[i]) + __shfl_xor_sync(kFull, l1 ? v[i] : v[4 + i], 1);
+    x[4] = v[8] + __shfl_xor_sync(kFull, v[8], 1);
+    x[5] = v[9] + __shfl_xor_sync(kFull, v[9], 1);
+    add_part(rec, l1 ? 1 : 0, x[0], x[1], x[2], l1 ? 0.f : x[3]);
+    if (l1) add_part(rec, 2, x[3], x[4], x[5], 0.f);
   }
 }
 
-// float offset of gradient value k (the six exponent / opacity sums, depth |
-// rgb 3) in the 12-float record {s0, s1, s2, s3} {s4, s5, depth, -} {r, g, b, -}
-__device__ __forceinline__ int rec_off(int k) { return k < 7 ? k : k + 1; }
-
-// Sum the 10 values v[0..9] over the warp with exchanges that halve the number
-// of values each lane carries (xor 16: 10 -> 5, xor 8: 5 -> 3, xor 4: 3 -> 2,
-// xor 2: 2 -> 1) and a final xor-1 step (12 shuffles instead of 50), then add
-// the totals to the record: even lanes hold distinct values, so this is one
-// warp-wide scalar atomic add.
-__device__ __forceinline__ void warp_reduce_add10(float (&v)[10], float* __restrict__ rec) {
-  const int lane = threadIdx.x & 31;
-  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-  float u[5];
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {  // keep v[i] (b4 = 0) or v[i + 5] (b4 = 1)
-    const float send = b4 ? v[i] : v[i + 5];
-    const float keep = b4 ? v[i + 5] : v[i];
-    u[i] = keep + __shfl_xor_sync(kFull, send, 16);
-  }
-  float w3[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {  // keep u[0..2] (b3 = 0) or u[3..4], 0 (b3 = 1)
-    const float hi = i < 2 ? u[i + 3] : 0.f;
-    const float send = b3 ? u[i] : hi;
-    const float keep = b3 ? hi : u[i];
-    w3[i] = keep + __shfl_xor_sync(kFull, send, 8);
-  }
-  float w2[2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {  // keep w3[0..1] (b2 = 0) or w3[2], 0 (b2 = 1)
-    const float hi = i < 1 ? w3[i + 2] : 0.f;
-    const float send = b2 ? w3[i] : hi;
-    const float keep = b2 ? hi : w3[i];
-    w2[i] = keep + __shfl_xor_sync(kFull, send, 4);
-  }
-  float x;
-  {
-    const float send = b1 ? w2[0] : w2[1];
-    const float keep = b1 ? w2[1] : w2[0];
-    x = keep + __shfl_xor_sync(kFull, send, 2);
-  }
-  x += __shfl_xor_sync(kFull, x, 1);
-  // value held: 5 b4 + i3 with i3 = 3 b3 + 2 b2 + b1 among the five kept at
-  // xor 16; lanes with b2 and (b3 or b1) hold the zero pads
-  const int i3 = (b3 ? 3 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
-  const bool valid = !(b2 && (b3 || b1));
-  if (!(lane & 1) && valid) atomicAdd(&rec[rec_off((b4 ? 5 : 0) + i3)], x);
-}
-
-// Back-to-front step of one pixel for one Gaussian (pixel_q, then bwd_body):
-// updates the pixel's running transmittance T and "colour behind" U and adds
-// the Gaussian's gradient sums to v.  With ga = dL/dalpha * alpha (unclamped alpha) the
-// exponent and opacity gradients are linear in
+// Backward pass of region `quad` of the tile of visit k by one warp: back to
+// front, from the pixels' last contributors.  Per pixel, the running
+// transmittance T is recovered by division and U is the colour (and depth)
+// behind, minus the alpha image's term.  With ga = dL/dalpha * alpha
+// (unclamped alpha) the exponent and opacity gradients of a Gaussian are
+// linear in
 //   v[0] = sum ga t0, v[1] = sum ga t1, v[2] = sum ga t0 dx,
 //   v[3] = sum ga t1 dx, v[4] = sum ga t1 w, v[5] = sum ga
 // (t0 = i0 dx, t1 = i1 w, w = dy - k dx): the Gaussian's constants (i0, i1,
 // k, ln 2, 1 / opacity) are applied once per Gaussian in the projection
 // backward pass.  v[6] = sum w dD (depth), v[7..9] = sum w dC (colour).
-// Exponent of one pixel for one entry: q' = t0^2 + t1^2 and its parts.
-struct PixQ {
-  float dx, t0, wq, t1, q;
-  bool pass;  // inside the support and in front of the pixel's last contributor
-};
-__device__ __forceinline__ PixQ pixel_q(const float4& a, const float4& bb, float plx, float ply, bool behind_last) {
-  PixQ r;
-  r.dx = __fsub_rn(plx, a.x);
-  const float dy = __fsub_rn(ply, a.y);
-  r.t0 = __fmul_rn(a.z, r.dx);
-  r.wq = __fmaf_rn(-a.w, r.dx, dy);
-  r.t1 = __fmul_rn(bb.x, r.wq);
-  r.q = __fmaf_rn(r.t0, r.t0, __fmul_rn(r.t1, r.t1));
-  r.pass = behind_last && r.q <= bb.w;
-  return r;
-}
-
-// The rest of the back-to-front step, without branches: a lane whose pixel
-// does not take part runs it with weight 0 and leaves T, U and v unchanged.
-// FIRST: the entry's first pixel row of the lane writes the ten sums instead
-// of adding to them (no zeroing of v per entry; a zero term may then be
-// stored as -0, which adds like +0).
-template <bool FIRST>
-__device__ __forceinline__ void bwd_body(const PixQ& e, const float4& bb, const float4& c, const RasterParams& rp,
-                                         float& T, float& U, float dC0, float dC1, float dC2, float dD, float dA_T,
-                                         float (&v)[10]) {
-  const float araw = ex2_approx(__fsub_rn(bb.y, e.q));
-  const float al = fminf(rp.alpha_max, araw);
-  const float inv1m = rcp_approx(1.f - al);  // 1 - alpha in [0.01, 1)
-  const float Ti = T * inv1m;  // transmittance in front of this Gaussian
-  const float w = e.pass ? al * Ti : 0.f;
-  v[7] = FIRST ? w * dC0 : fmaf(w, dC0, v[7]);
-  v[8] = FIRST ? w * dC1 : fmaf(w, dC1, v[8]);
-  v[9] = FIRST ? w * dC2 : fmaf(w, dC2, v[9]);
-  v[6] = FIRST ? w * dD : fmaf(w, dD, v[6]);
-  const float cdot = c.x * dC0 + c.y * dC1 + c.z * dC2 + bb.z * dD;
-  // d/d alpha_i: colour/depth T_i c_i - (sum behind)/(1 - alpha_i); alpha image + T_final/(1 - alpha_i)
-  const float g_alpha = Ti * cdot - (U - dA_T) * inv1m;
-  U = fmaf(w, cdot, U);
-  T = e.pass ? Ti : T;
-  const float ga = (e.pass && araw <= rp.alpha_max) ? g_alpha * araw : 0.f;  // the 0.99 clamp has zero gradient
-  const float gt0 = ga * e.t0, gt1 = ga * e.t1;
-  v[0] = FIRST ? gt0 : v[0] + gt0;
-  v[1] = FIRST ? gt1 : v[1] + gt1;
-  v[2] = FIRST ? gt0 * e.dx : fmaf(gt0, e.dx, v[2]);
-  v[3] = FIRST ? gt1 * e.dx : fmaf(gt1, e.dx, v[3]);
-  v[4] = FIRST ? gt1 * e.wq : fmaf(gt1, e.wq, v[4]);
-  v[5] = FIRST ? ga : v[5] + ga;
-}
-
-// Backward pass of one 8 x 8 pixel block (quadrant `quad` of the tile of
-// visit k) by one warp, with the warp's shared staging buffers.
-template <int TW, int TH>
+// A lane's pixels share dx and t0, so v[0], v[2], v[3] follow from its sums
+// of ga and ga t1.
+template <int TW, int TH, int PPL>
 __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams& rp, uint32_t k, int quad,
-                                        Entry* __restrict__ buf, uint32_t* __restrict__ bid,
-                                        float4 (*__restrict__ s_raw)[32][3], uint32_t (*__restrict__ s_gid)[32],
-                                        const float* __restrict__ T_final_all,
+                                        WarpSmem& sm, const float* __restrict__ T_final_all,
                                         const int32_t* __restrict__ last_all, float* __restrict__ g2d) {
-  constexpr int WX = TW / 8;
+  using M = WarpMap<TW, TH, PPL, kBwdLanes<PPL>>;
+  constexpr int NP = (PPL + 1) / 2;  // pairs of pixels per lane
   const TileJob job = tile_job<TW, TH>(a, k);
   const RasterView& vw = a.v[job.v];
   const int width = vw.width, height = vw.height;
-  const uint32_t* __restrict__ ids = a.ids;
-  const float4* __restrict__ feat = a.feat;
   const float* __restrict__ T_final = T_final_all + vw.pix_base;
   const int32_t* __restrict__ last_in = last_all + vw.pix_base;
   const float* __restrict__ dLdc = vw.dLdc;
@@ -589,155 +708,176 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
   const float dscale = a.nvalid ? a.w_depth / (float)max(a.nvalid[job.v], 1u)
                                 : (a.depth_scale ? a.depth_scale[job.v] : 1.f);
   const int lane = threadIdx.x & 31;
-  const int bxi = (quad % WX) * 8, byi = (quad / WX) * 8;
-  const int lx = bxi + (lane & 7), ly0 = byi + (lane >> 3), ly1 = ly0 + 4;
-  const int px = job.ox + lx, py0 = job.oy + ly0, py1 = job.oy + ly1;
-  const bool in0 = px < width && py0 < height, in1 = px < width && py1 < height;
-  const float plx = (float)lx + 0.5f, ply0 = (float)ly0 + 0.5f, ply1 = (float)ly1 + 0.5f;
-  const float ox = (float)job.ox, oy = (float)job.oy, bx = (float)bxi, by = (float)byi;
-  const uint2 r = job.range;
+  const int bxi = (quad % (TW / M::RW)) * M::RW, byi = (quad / (TW / M::RW)) * M::RH;
+  const int lx = bxi + lane % M::RW, ly = byi + PPL * (lane / M::RW);
+  const int px = job.ox + lx, py = job.oy + ly;
+  const float plx = (float)lx + 0.5f;
   const size_t HW = (size_t)width * height;
-  __syncwarp();  // the warp's previous job is done with the buffers
+  __syncwarp();  // the warp's previous job is done with sm
 
-  // per-pixel state (two pixels per thread)
-  float T0 = 1.f, c00 = 0.f, c01 = 0.f, c02 = 0.f, d0 = 0.f, a0 = 0.f;
-  float T1 = 1.f, c10 = 0.f, c11 = 0.f, c12 = 0.f, d1 = 0.f, a1 = 0.f;
-  int last0 = 0, last1 = 0;
-  if (in0) {
-    const size_t p = (size_t)py0 * width + px;
-    T0 = T_final[p];
-    last0 = last_in[p];
-    c00 = dLdc[p];
-    c01 = dLdc[HW + p];
-    c02 = dLdc[2 * HW + p];
-    d0 = dLdd[p] * dscale;
-    a0 = dLda ? dLda[p] : 0.f;
-  }
-  if (in1) {
-    const size_t p = (size_t)py1 * width + px;
-    T1 = T_final[p];
-    last1 = last_in[p];
-    c10 = dLdc[p];
-    c11 = dLdc[HW + p];
-    c12 = dLdc[2 * HW + p];
-    d1 = dLdd[p] * dscale;
-    a1 = dLda ? dLda[p] : 0.f;
-  }
-  // U = sum over Gaussians behind of w_j (c_j . dC + z_j dD) + T_final (bg . dC)
-  float U0 = T0 * (rp.bg[0] * c00 + rp.bg[1] * c01 + rp.bg[2] * c02);
-  float U1 = T1 * (rp.bg[0] * c10 + rp.bg[1] * c11 + rp.bg[2] * c12);
-  const float dAT0 = a0 * T0, dAT1 = a1 * T1;
-
-  int wmax = max(last0, last1);
+  f2x PLY[NP], T[NP], U[NP], C0[NP], C1[NP], C2[NP], DD[NP];
+  int last[2 * NP];
+  int glast = 0;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, off));
+  for (int p = 0; p < NP; ++p) {
+    float t[2], c0[2], c1[2], c2[2], d[2], u[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int s = 2 * p + h;
+      t[h] = 1.f;
+      c0[h] = c1[h] = c2[h] = d[h] = u[h] = 0.f;
+      last[s] = 0;
+      if (s < PPL && px < width && py + s < height) {
+        const size_t q = (size_t)(py + s) * width + px;
+        t[h] = T_final[q];
+        last[s] = last_in[q];
+        c0[h] = dLdc[q];
+        c1[h] = dLdc[HW + q];
+        c2[h] = dLdc[2 * HW + q];
+        d[h] = dLdd[q] * dscale;
+        // sum over Gaussians behind of w_j (c_j . dC + z_j dD) + T_final (bg . dC - dA)
+        u[h] = t[h] * (rp.bg[0] * c0[h] + rp.bg[1] * c1[h] + rp.bg[2] * c2[h]) - (dLda ? dLda[q] * t[h] : 0.f);
+      }
+      glast = max(glast, last[s]);
+    }
+    PLY[p] = f2_pack((float)(ly + 2 * p) + 0.5f, (float)(ly + 2 * p + 1) + 0.5f);
+    T[p] = f2_pack(t[0], t[1]);
+    U[p] = f2_pack(u[0], u[1]);
+    C0[p] = f2_pack(c0[0], c0[1]);
+    C1[p] = f2_pack(c1[0], c1[1]);
+    C2[p] = f2_pack(c2[0], c2[1]);
+    DD[p] = f2_pack(d[0], d[1]);
+  }
+#pragma unroll
+  for (int off = M::LPG / 2; off > 0; off >>= 1) glast = max(glast, __shfl_xor_sync(kFull, glast, off));  // the group's
+  int wmax = glast;
+#pragma unroll
+  for (int off = 16; off >= M::LPG; off >>= 1) wmax = max(wmax, __shfl_xor_sync(kFull, wmax, off));
   if (wmax == 0) return;
 
-  // walk the list back to front in chunks of 32: chunk c in shared memory,
-  // chunk c - 32 in flight (cp.async), the ids of chunk c - 64 in a register
-  int c0 = ((wmax - 1) >> 5) << 5;
-  int cur = 0;
-  if (c0 + lane < wmax) {
-    const uint32_t g = checked_id(ids[r.x + c0 + lane], a.n_items);
-    s_gid[0][lane] = g;
-    cp_record(s_raw[0][lane], feat, g);
-  }
-  cp_commit();
-  uint32_t g2 = c0 >= 32 ? checked_id(ids[r.x + c0 - 32 + lane], a.n_items) : 0u;
-  for (; c0 >= 0; c0 -= 32, cur ^= 1) {
-    if (c0 >= 32) {
-      s_gid[cur ^ 1][lane] = g2;
-      cp_record(s_raw[cur ^ 1][lane], feat, g2);
+  Walk<M, -1> walk;
+  walk.ids = a.ids + job.range.x;
+  walk.feat = a.feat;
+  walk.sm = &sm;
+  walk.n = wmax;
+  walk.lane = lane;
+  walk.n_items = a.n_items;
+  walk.ox = (float)job.ox;
+  walk.oy = (float)job.oy;
+  walk.bx = (float)bxi;
+  walk.by = (float)byi;
+  walk.begin();
+  const f2x ONE2 = f2_pack(1.f, 1.f);
+  for (;;) {
+    while (__any_sync(kFull, walk.cur == 0u && walk.off < walk.top)) walk.step();
+    const bool can = walk.can_stage();
+    if (can && __any_sync(kFull, walk.cur == 0u)) {  // a group is dry
+      unsigned mine = walk.stage(rp);
+      const int over = walk.chunk(walk.top) + 32 - glast;  // entries behind every pixel of the group
+      if (over > 0) mine = over < 32 ? mine & (kFull >> over) : 0u;
+      walk.push(mine);
+      continue;
     }
-    cp_commit();
-    if (c0 >= 64) g2 = checked_id(ids[r.x + c0 - 64 + lane], a.n_items);
-    cp_wait_prev();
-    const bool have = c0 + lane < wmax;
-    Entry e;
-    const float4* raw = s_raw[cur][lane];
-    const bool hit = have && make_entry(raw[0], raw[1], raw[2], ox, oy, bx, by, rp, e) != 0u;
-    __syncwarp();
-    if (hit) {
-      buf[lane] = e;
-      bid[lane] = s_gid[cur][lane];
-    }
-    unsigned bal = __ballot_sync(kFull, hit);
-    __syncwarp();
-    while (bal) {
-      const int j = 31 - __clz(bal);
-      bal &= ~(1u << j);
-      const int idx = c0 + j;
-      const float4 a = buf[j].a;
-      const float4 bb = buf[j].b;
-      const float4 cc = buf[j].c;
-      float v[10];  // written by the first row's step
-      const unsigned halves = __float_as_uint(cc.w);
-      // both pixel rows' exponents first, then the rows' steps as straight-line
-      // code (independent chains); skipped when no lane of the warp takes part
-      // a half the support box misses (warp-uniform) is skipped
-      bool contrib;
-      if (halves == 3u) {
-        const PixQ e0 = pixel_q(a, bb, plx, ply0, idx < last0);
-        const PixQ e1 = pixel_q(a, bb, plx, ply1, idx < last1);
-        contrib = e0.pass || e1.pass;
-        if (!__any_sync(kFull, contrib)) continue;
-        bwd_body<true>(e0, bb, cc, rp, T0, U0, c00, c01, c02, d0, dAT0, v);
-        bwd_body<false>(e1, bb, cc, rp, T1, U1, c10, c11, c12, d1, dAT1, v);
-      } else if (halves == 1u) {
-        const PixQ e0 = pixel_q(a, bb, plx, ply0, idx < last0);
-        contrib = e0.pass;
-        if (!__any_sync(kFull, contrib)) continue;
-        bwd_body<true>(e0, bb, cc, rp, T0, U0, c00, c01, c02, d0, dAT0, v);
-      } else {
-        const PixQ e1 = pixel_q(a, bb, plx, ply1, idx < last1);
-        contrib = e1.pass;
-        if (!__any_sync(kFull, contrib)) continue;
-        bwd_body<true>(e1, bb, cc, rp, T1, U1, c10, c11, c12, d1, dAT1, v);
+    const int lim = walk.limit(can);
+    if (lim == walk.kEnd) break;
+    if (lim == walk.kAgain) continue;
+    do {
+      int idx;
+      const Entry& en = sm.e[walk.take(idx)];
+      const float4 ea = en.a, eb = en.b, ec = en.c;
+      const float dx = __fsub_rn(plx, ea.x);
+      const float t0 = __fmul_rn(ea.z, dx);
+      f2x TQ[NP], WQ[NP];
+      float ar[2 * NP], in[2 * NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const f2x DY = f2_sub(PLY[p], f2_bcast(ea.y));
+        WQ[p] = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
+        TQ[p] = f2_mul(WQ[p], f2_bcast(eb.x));
+        const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ[p], TQ[p]));
+        const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
+        ar[2 * p] = ex2_approx(f2_lo(ARG));
+        ar[2 * p + 1] = ex2_approx(f2_hi(ARG));
+        in[2 * p] = one_if_le_and(f2_lo(Q), eb.w, idx, last[2 * p]);
+        in[2 * p + 1] = one_if_le_and(f2_hi(Q), eb.w, idx, last[2 * p + 1]);
       }
-      const unsigned m = __ballot_sync(kFull, contrib);
-      if (m == 0) continue;
-      float* rec = g2d + 12 * (size_t)bid[j];
-      if (__popc(m) <= kAtomicLanes) {
-        if (contrib) {
-          // three 16-byte vector atomics per lane (red.global.add.v4.f32)
-          float4* r4 = reinterpret_cast<float4*>(rec);
-          atomicAdd(r4, make_float4(v[0], v[1], v[2], v[3]));
-          atomicAdd(r4 + 1, make_float4(v[4], v[5], v[6], 0.f));
-          atomicAdd(r4 + 2, make_float4(v[7], v[8], v[9], 0.f));
+      f2x AL[NP], AG[NP];  // alpha, and alpha where it is not clamped: 0 where the pixel takes no part
+#pragma unroll
+      for (int p = 0; p < NP; ++p) AL[p] = AG[p] = f2_mul(f2_pack(ar[2 * p], ar[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
+      if (eb.y > rp.log2_clamp) {  // the 0.99 clamp has zero gradient
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const bool c0 = f2_lo(AL[p]) > rp.alpha_max, c1 = f2_hi(AL[p]) > rp.alpha_max;
+          AG[p] = f2_pack(c0 ? 0.f : f2_lo(AL[p]), c1 ? 0.f : f2_hi(AL[p]));
+          AL[p] = f2_pack(c0 ? rp.alpha_max : f2_lo(AL[p]), c1 ? rp.alpha_max : f2_hi(AL[p]));
         }
-      } else {
-        warp_reduce_add10(v, rec);
       }
-    }
+      f2x GA = 0, GT = 0, GW = 0, V6 = 0, V7 = 0, V8 = 0, V9 = 0;  // sums over the lane's pairs
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const f2x OM = f2_sub(ONE2, AL[p]);  // in [0.01, 1]; 1 where the pixel takes no part: T, U unchanged
+        const f2x INV = f2_pack(rcp_approx(f2_lo(OM)), rcp_approx(f2_hi(OM)));
+        T[p] = f2_mul(T[p], INV);  // transmittance in front of this Gaussian
+        const f2x W = f2_mul(AL[p], T[p]);
+        const f2x CD = f2_fma_s(C0[p], ec.x, f2_fma_s(C1[p], ec.y, f2_fma_s(C2[p], ec.z, f2_mul(DD[p], f2_bcast(eb.z)))));
+        // d/d alpha_i: colour/depth T_i c_i - (sum behind)/(1 - alpha_i); alpha image + T_final/(1 - alpha_i)
+        const f2x GAL = f2_sub(f2_mul(T[p], CD), f2_mul(U[p], INV));
+        U[p] = f2_fma(W, CD, U[p]);
+        const f2x g = f2_mul(GAL, AG[p]);
+        const f2x gt = f2_mul(g, TQ[p]);
+        if (p == 0) {
+          GA = g;
+          GT = gt;
+          GW = f2_mul(gt, WQ[p]);
+          V6 = f2_mul(W, DD[p]);
+          V7 = f2_mul(W, C0[p]);
+          V8 = f2_mul(W, C1[p]);
+          V9 = f2_mul(W, C2[p]);
+        } else {
+          GA = f2_add(GA, g);
+          GT = f2_add(GT, gt);
+          GW = f2_fma(gt, WQ[p], GW);
+          V6 = f2_fma(W, DD[p], V6);
+          V7 = f2_fma(W, C0[p], V7);
+          V8 = f2_fma(W, C1[p], V8);
+          V9 = f2_fma(W, C2[p], V9);
+        }
+      }
+      float v[10];
+      v[5] = f2_lo(GA) + f2_hi(GA);
+      v[1] = f2_lo(GT) + f2_hi(GT);
+      v[4] = f2_lo(GW) + f2_hi(GW);
+      v[6] = f2_lo(V6) + f2_hi(V6);
+      v[7] = f2_lo(V7) + f2_hi(V7);
+      v[8] = f2_lo(V8) + f2_hi(V8);
+      v[9] = f2_lo(V9) + f2_hi(V9);
+      v[0] = v[5] * t0;
+      v[2] = v[0] * dx;
+      v[3] = v[1] * dx;
+      group_reduce_add10<M::LPG>(v, lane, g2d + 12 * (size_t)__float_as_uint(ec.w));
+    } while (can ? !__any_sync(kFull, walk.cur == 0u) : walk.any_up_to(lim));
   }
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  cp_wait_all();
 }
 
-// PERSIST = false: one CTA per tile visit, warp w on quadrant w.  Otherwise
-// a persistent grid whose warps pull jobs from `work` with next_job.
-template <int TW, int TH, bool PERSIST>
-__global__ void __launch_bounds__(kThreads, 6) raster_bwd_kernel(const __grid_constant__ RasterArgs a,
+// `work` as in raster_fwd_kernel.
+template <int TW, int TH, int PPL>
+__global__ void __launch_bounds__(kThreads, kBwdCtas) raster_bwd_kernel(const __grid_constant__ RasterArgs a,
                                                                  RasterParams rp,
                                                                  const float* __restrict__ T_final_all,
                                                                  const int32_t* __restrict__ last_all,
                                                                  float* __restrict__ g2d,
                                                                  uint32_t* __restrict__ work) {
   pdl_enter();
-  static_assert((TW / 8) * (TH / 8) == kThreads / 32, "four 8x8 warp blocks per tile");
-  __shared__ Entry s_e[kThreads / 32][32];
-  __shared__ uint32_t s_id[kThreads / 32][32];
-  __shared__ __align__(16) float4 s_raw[kThreads / 32][2][32][3];
-  __shared__ uint32_t s_gid[kThreads / 32][2][32];
+  constexpr uint32_t JOBS = 8 / PPL;
+  __shared__ __align__(16) WarpSmem s_w[kThreads / 32];
   const int warp = threadIdx.x >> 5;
-  if constexpr (!PERSIST) {
-    bwd_job<TW, TH>(a, rp, blockIdx.x, warp, s_e[warp], s_id[warp], s_raw[warp], s_gid[warp], T_final_all,
-                    last_all, g2d);
-  } else {
-    const uint32_t n_jobs = 4u * a.n_tiles;
-    uint32_t job;
-    while (next_job(work, n_jobs, job))
-      bwd_job<TW, TH>(a, rp, job >> 2, (int)(job & 3u), s_e[warp], s_id[warp], s_raw[warp], s_gid[warp],
-                      T_final_all, last_all, g2d);
+  init_warp_smem(s_w[warp]);
+  const uint32_t n_jobs = JOBS * a.n_tiles;
+  uint32_t job = blockIdx.x * (kThreads / 32) + warp;
+  while (work ? next_job(work, n_jobs, job) : job < n_jobs) {
+    bwd_job<TW, TH, PPL>(a, rp, job / JOBS, (int)(job % JOBS), s_w[warp], T_final_all, last_all, g2d);
+    if (!work) break;
   }
 }
 
@@ -752,6 +892,7 @@ RasterParams make_params(const RasterArgs& a) {
   rp.log2_alpha_min = log2f(a.alpha_min);
   rp.qmax_s = 9.f * kHalfLog2e;
   rp.t_eps = a.t_eps;
+  rp.log2_clamp = log2f(a.alpha_max) - 1e-5f;
   return rp;
 }
 
@@ -765,28 +906,38 @@ namespace {
 
 // Persistent grid: as many CTAs as fit on the GPU at once (occupancy of the
 // kernel x SMs; per_sm caches the occupancy query of one kernel), at most one
-// per tile visit.
+// per kThreads / 32 jobs.
 template <class K>
-int persistent_grid(K kernel, int& per_sm, int n_tiles, int num_sms) {
+int persistent_grid(K kernel, int& per_sm, int n_ctas, int num_sms) {
   if (per_sm == 0) {
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kThreads, 0) != cudaSuccess || b < 1) b = 1;
     per_sm = b;
   }
-  return std::max(1, std::min(n_tiles, per_sm * std::max(num_sms, 1)));
+  return std::max(1, std::min(n_ctas, per_sm * std::max(num_sms, 1)));
+}
+
+int job_ctas(uint32_t n_tiles, int ppl) {
+  return (int)(((int64_t)n_tiles * (8 / ppl) + kThreads / 32 - 1) / (kThreads / 32));
+}
+
+template <int TW, int TH, int PPL, bool COUNT, bool LOSS>
+void fwd_launch(const RasterArgs& a, const RasterParams& rp, float* T_final, int32_t* last,
+                unsigned long long* counters, cudaStream_t s) {
+  static int per_sm = 0;
+  const int nc = job_ctas(a.n_tiles, PPL);
+  auto* k = raster_fwd_kernel<TW, TH, PPL, COUNT, LOSS>;
+  launch_pdl(k, a.work ? persistent_grid(k, per_sm, nc, a.num_sms) : nc, kThreads, 0, s, a, rp, T_final, last, counters,
+             a.work);
 }
 
 template <int TW, int TH, bool COUNT, bool LOSS>
 void fwd_shape(const RasterArgs& a, const RasterParams& rp, float* T_final, int32_t* last,
                unsigned long long* counters, cudaStream_t s) {
-  const int nt = (int)a.n_tiles;
-  if (a.work) {
-    static int per_sm = 0;
-    auto* k = raster_fwd_kernel<TW, TH, COUNT, LOSS, true>;
-    launch_pdl(k, persistent_grid(k, per_sm, nt, a.num_sms), kThreads, 0, s, a, rp, T_final, last, counters, a.work);
-  } else {
-    launch_pdl(raster_fwd_kernel<TW, TH, COUNT, LOSS, false>, nt, kThreads, 0, s, a, rp, T_final, last, counters,
-               (uint32_t*)nullptr);
+  switch (raster_px_per_lane(a.n_tiles, a.num_sms)) {
+    case 4: fwd_launch<TW, TH, 4, COUNT, LOSS>(a, rp, T_final, last, counters, s); break;
+    case 2: fwd_launch<TW, TH, 2, COUNT, LOSS>(a, rp, T_final, last, counters, s); break;
+    default: fwd_launch<TW, TH, 1, COUNT, LOSS>(a, rp, T_final, last, counters, s); break;
   }
 }
 
@@ -798,20 +949,39 @@ void fwd_shapes(const RasterArgs& a, const RasterParams& rp, float* T_final, int
   else fwd_shape<32, 8, COUNT, LOSS>(a, rp, T_final, last, counters, s);
 }
 
+template <int TW, int TH, int PPL>
+void bwd_launch(const RasterArgs& a, const RasterParams& rp, const float* T_final, const int32_t* last, float* g2d,
+                cudaStream_t s) {
+  static int per_sm = 0;
+  const int nc = job_ctas(a.n_tiles, PPL);
+  auto* k = raster_bwd_kernel<TW, TH, PPL>;
+  launch_pdl(k, a.work ? persistent_grid(k, per_sm, nc, a.num_sms) : nc, kThreads, 0, s, a, rp, T_final, last, g2d,
+             a.work);
+}
+
 template <int TW, int TH>
 void bwd_shape(const RasterArgs& a, const RasterParams& rp, const float* T_final, const int32_t* last, float* g2d,
                cudaStream_t s) {
-  const int nt = (int)a.n_tiles;
-  if (a.work) {
-    static int per_sm = 0;
-    auto* k = raster_bwd_kernel<TW, TH, true>;
-    launch_pdl(k, persistent_grid(k, per_sm, nt, a.num_sms), kThreads, 0, s, a, rp, T_final, last, g2d, a.work);
-  } else {
-    launch_pdl(raster_bwd_kernel<TW, TH, false>, nt, kThreads, 0, s, a, rp, T_final, last, g2d, (uint32_t*)nullptr);
+  switch (raster_px_per_lane(a.n_tiles, a.num_sms)) {
+    case 4: bwd_launch<TW, TH, 4>(a, rp, T_final, last, g2d, s); break;
+    case 2: bwd_launch<TW, TH, 2>(a, rp, T_final, last, g2d, s); break;
+    default: bwd_launch<TW, TH, 1>(a, rp, T_final, last, g2d, s); break;
   }
 }
 
 }  // namespace
+
+// Four pixels per lane share an entry's loads and its list handling, but give
+// a tile only two warps.  Below about six tiles per SM the SMs hold too few
+// warps to hide a warp's latency, and two pixels per lane (twice the warps,
+// each with a shorter walk) are faster; below one tile per SM, one.  Measured,
+// forward + backward us at 4 / 2 / 1 pixels per lane: 80 tiles 55 / 48 / 44,
+// 300 tiles 55 / 49 / 54, 690 tiles 66 / 62 / 88, 1200 tiles 83 / 87 / 131,
+// 1908 tiles 97 / 108 / 176.
+int raster_px_per_lane(uint32_t n_tiles, int num_sms) {
+  const uint32_t sms = (uint32_t)std::max(num_sms, 1);
+  return n_tiles >= 6 * sms ? 4 : n_tiles >= sms ? 2 : 1;
+}
 
 void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsigned long long* counters,
                        cudaStream_t s) {
