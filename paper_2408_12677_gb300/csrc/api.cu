@@ -58,13 +58,15 @@ struct gs_ctx {
   uint32_t* scan_aux = nullptr;  // multi-block tile scan scratch
   uint32_t* bigq = nullptr;     // ids of Gaussians covering more than kBigTiles tiles
   uint32_t* d_bigmeta = nullptr;  // [0] length of the large-splat queue, [1] / [2] forward / backward raster
-                                  // job counters, [3] ticket of the fused-loss reduction (0 between launches)
+                                  // job counters, [3] ticket of the fused-loss reduction (0 between launches),
+                                  // [kHugeFlag] the difference grids are in use
   bool counts_zero = false;       // the tile counters and the large-splat queue length are 0 (the per-tile
                                   // sort, the last binning kernel, zeroes them)
   bool fwd_work_zero = false;     // the forward / backward raster job counters are 0 (the per-tile sort zeroes
   bool bwd_work_zero = false;     // both; a raster launch uses its counter up)
   bool g2d_zero = false;          // the gradient records are all 0 (their consumers clear what they read)
-  unsigned long long* d_binstats = nullptr;  // [0] total pairs, [1] longest tile list
+  unsigned long long* d_binstats = nullptr;  // [0] total pairs, [1] longest tile list; of cut lists also [2] the
+                                             // largest kept rank, [3] level-2 tiles, [4] a pixel did not stop
   long long* d_step = nullptr;               // device Adam step counter (step = 0 calls)
   int64_t cap_px = 0;
   float* T_final = nullptr;
@@ -92,7 +94,7 @@ struct gs_ctx {
   unsigned long long* h_pinned = nullptr;
   // eval counters (blended, visited) and per-stage event profiling
   bool counting = false;
-  unsigned long long* d_evals = nullptr;
+  unsigned long long* d_evals = nullptr;  // [2], [3]: the counters before a pass that may be repeated
   bool profiling = false;
   struct Ev {
     int stage;
@@ -138,6 +140,23 @@ struct gs_ctx {
   int64_t longest_seen = 0;
   bool bucket_ok = false;
   bool st_buckets = false;        // the last forward pass binned into the buckets
+  // long lists cut to their nearest entries (prefix.cu, sync mode)
+  int64_t cap_pfx = 0;            // tiles of the arrays below
+  uint32_t* pfx_lim = nullptr;
+  uint32_t* pfx_kept = nullptr;
+  uint32_t* pfx_off = nullptr;
+  uint32_t* pfx_cur = nullptr;
+  uint8_t* pfx_cut = nullptr;
+  uint8_t* pfx_level = nullptr;
+  uint32_t* pfx_gather = nullptr;
+  ushort4* pfx_rects = nullptr;          // rectangles by depth, for the level-2 tiles
+  int64_t cap_pfx_rects = 0;
+  int64_t cap_pfx_diff = 0;
+  int* pfx_diff = nullptr;
+  const uint32_t* pfx_sorted = nullptr;  // items by depth (of the current pass)
+  bool st_cut = false;            // the last forward pass's lists are cut (tcount, toffset: the full ones)
+  int* big_diff = nullptr;        // difference grids of the projection's large rectangles, 0 between passes
+  int64_t cap_big = 0;
   bool order_tiles = true;  // compute and use the visit order
   bool persistent = true;   // raster passes as persistent grids pulling (tile, quadrant) jobs
   int st_sh = 0;
@@ -303,6 +322,52 @@ gs_status ensure_tiles(gs_ctx* c, int64_t t) {
   return GS_OK;
 }
 
+// Cells of the views' difference grids ((tiles_x + 1) x (tiles_y + 1) each, end
+// to end), their first cells in base[].
+int64_t grid_layout(const TileMap& map, const int* tiles_y, uint32_t* base) {
+  int64_t cells = 0;
+  for (int v = 0; v < map.views; ++v) {
+    base[v] = (uint32_t)cells;
+    cells += ((int64_t)map.tiles_x[v] + 1) * (tiles_y[v] + 1);
+  }
+  return cells;
+}
+
+gs_status ensure_big(gs_ctx* c, int64_t cells) {
+  if (cells <= c->cap_big) return GS_OK;
+  if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
+  GS_CUDA(c, cudaDeviceSynchronize());
+  const int64_t cap = grow_target(cells, c->cap_big);
+  GS_GROW(c, cap_big, regrow(&c->big_diff, cap));
+  GS_GROW(c, cap_big, cudaMemset(c->big_diff, 0, sizeof(int) * (size_t)cap));
+  c->cap_big = cap;
+  return GS_OK;
+}
+
+gs_status ensure_prefix(gs_ctx* c, int64_t tiles, int64_t diff_cells) {
+  if (tiles > c->cap_pfx) {
+    if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
+    GS_CUDA(c, cudaDeviceSynchronize());
+    const int64_t cap = grow_target(tiles, c->cap_pfx);
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_lim, cap));
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_kept, cap));
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_off, cap));
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_cur, cap));
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_cut, cap));
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_level, cap));
+    GS_GROW(c, cap_pfx, regrow(&c->pfx_gather, cap));
+    c->cap_pfx = cap;
+  }
+  if (diff_cells > c->cap_pfx_diff) {
+    if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
+    GS_CUDA(c, cudaDeviceSynchronize());
+    const int64_t cap = grow_target(diff_cells, c->cap_pfx_diff);
+    GS_GROW(c, cap_pfx_diff, regrow(&c->pfx_diff, cap));
+    c->cap_pfx_diff = cap;
+  }
+  return GS_OK;
+}
+
 gs_status ensure_px(gs_ctx* c, int64_t npx) {
   if (npx <= c->cap_px) return GS_OK;
   if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
@@ -464,6 +529,8 @@ gs_status bin_and_sort_radix(gs_ctx* c, int n, const TileMap& map, cudaStream_t 
   c->st_pairs = c->sync ? P : -1;
   c->st_pair_buf = pcur;
   c->st_buckets = false;
+  c->st_ordered = false;
+  c->st_cut = false;
   return GS_OK;
 }
 
@@ -492,7 +559,7 @@ gs_status bin_buckets(gs_ctx* c, int n, const TileMap& map, cudaStream_t s) {
   tb.order = nullptr;
   tb.counted = true;
   tb.scan_aux = nullptr;
-  tb.raster_work = c->persistent ? c->d_bigmeta + 1 : nullptr;
+  tb.raster_work = c->d_bigmeta + 1;
   tb.bucket_ids = c->bids;
   tb.bucket_cap = c->bucket_cap;
   tb.cls_count = c->cls_count;
@@ -504,21 +571,134 @@ gs_status bin_buckets(gs_ctx* c, int n, const TileMap& map, cudaStream_t s) {
   }
   GS_CHECK_LAUNCH(c, "tile sort (buckets)");
   c->counts_zero = true;
-  if (tb.raster_work) c->fwd_work_zero = c->bwd_work_zero = true;
+  c->fwd_work_zero = c->bwd_work_zero = true;
   c->st_pairs = -1;
   c->st_pair_buf = 0;
   c->st_ordered = true;
   c->st_buckets = true;
+  c->st_cut = false;
+  return GS_OK;
+}
+
+// Long lists (sync mode): keep the nearest entries of every tile (prefix.cu),
+// in attempt 0 about kPrefixTarget of them out of the nearest kPrefixRanks
+// items, afterwards by the levels that the raster pass raised, out of all
+// items.  The tile counters and offsets keep the full lists'
+// (gs_get_tile_ranges).  *done = false when the grids would be too large (the
+// caller bins in full).
+constexpr uint32_t kPrefixTarget = 256, kPrefixRanks = 32768;
+gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, cudaStream_t s, int attempt,
+                     bool* done) {
+  const int64_t T = (int64_t)map.tile_base[map.views];
+  *done = false;
+  PrefixArgs a{};
+  a.map = map;
+  const int64_t cells = grid_layout(map, tiles_y, a.grid_base);
+  prefix_slabs(a, attempt ? (uint32_t)n : std::min((uint32_t)n, kPrefixRanks));
+  if (cells * a.slabs > ((int64_t)1 << 28)) return GS_OK;
+  gs_status st = ensure_prefix(c, T, cells * a.slabs);
+  if (st != GS_OK) return st;
+  for (int v = 0; v < map.views; ++v) a.tiles_y[v] = tiles_y[v];
+  a.grid_cells = (uint32_t)cells;
+  a.target = kPrefixTarget;
+  if (attempt == 0) {
+    SortBuffers sb;
+    for (int k = 0; k < 2; ++k) {
+      sb.keys[k] = c->dkey[k];
+      sb.vals[k] = c->dval[k];
+    }
+    sb.hist = c->hist;
+    sb.max_blocks = c->hist_blocks;
+    StageTimer t(c, GS_STAGE_DEPTH_SORT, s);
+    const int k = radix_sort_pairs(sb, c->zkey, nullptr, (uint32_t)n, nullptr, 32, c->num_sms, s, &c->launches);
+    c->pfx_sorted = c->dval[k >= 0 ? k : 0];
+  }
+  a.sorted = c->pfx_sorted;
+  a.rects = c->rects;
+  a.tiles = c->tiles;
+  a.diff = c->pfx_diff;
+  a.full = c->tcount;
+  a.level = c->pfx_level;
+  a.lim = c->pfx_lim;
+  a.kept = c->pfx_kept;
+  a.cut = c->pfx_cut;
+  a.max_lim = c->d_binstats + 2;
+  a.gather = c->pfx_gather;
+  a.n_gather = c->d_binstats + 3;
+  TileBinArgs tb;
+  tb.n = n;
+  tb.rects = c->rects;
+  tb.tiles = c->tiles;
+  tb.zkey = c->zkey;
+  tb.map = map;
+  tb.n_tiles = (int)T;
+  tb.num_sms = c->num_sms;
+  tb.counts = c->pfx_kept;
+  tb.offsets = c->pfx_off;
+  tb.cursors = c->pfx_cur;
+  tb.ids = nullptr;
+  tb.ranges = c->ranges;
+  tb.capacity = 0xFFFFFFF0u;
+  tb.n_pairs = c->d_npairs;
+  tb.stats = c->d_binstats;
+  tb.overflow = c->d_overflow;
+  tb.big_queue = c->bigq;
+  tb.big_len = c->d_bigmeta;
+  tb.order = c->order_tiles ? c->torder : nullptr;
+  tb.counted = true;
+  tb.scan_aux = c->scan_aux;
+  {
+    StageTimer t(c, GS_STAGE_DUPLICATE, s);
+    if (attempt == 0) GS_CUDA(c, cudaMemsetAsync(c->pfx_level, 0, (size_t)T, s));
+    GS_CUDA(c, cudaMemsetAsync(c->d_binstats + 4, 0, sizeof(unsigned long long), s));
+    launch_prefix_choose(a, s, &c->launches);
+    launch_tile_count_scan(tb, s, &c->launches);
+  }
+  GS_CHECK_LAUNCH(c, "prefix choose / scan");
+  GS_CUDA(c, cudaMemcpyAsync(c->h_pinned, c->d_binstats, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  GS_CUDA(c, cudaStreamSynchronize(s));
+  const uint32_t max_lim = (uint32_t)c->h_pinned[2], n_gather = (uint32_t)c->h_pinned[3];
+  if (n_gather > 0 && n > c->cap_pfx_rects) {
+    if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
+    GS_CUDA(c, cudaDeviceSynchronize());
+    const int64_t cap = grow_target(n, c->cap_pfx_rects);
+    GS_GROW(c, cap_pfx_rects, regrow(&c->pfx_rects, cap));
+    c->cap_pfx_rects = cap;
+  }
+  if ((st = ensure_pairs(c, std::max<int64_t>((int64_t)c->h_pinned[0], 1))) != GS_OK) return st;
+  tb.ids = c->pv[0];
+  tb.capacity = (uint32_t)std::min<int64_t>(c->cap_p, 0xFFFFFFF0ll);
+  tb.raster_work = c->d_bigmeta + 1;
+  tb.long_sorted = true;
+  {
+    StageTimer t(c, GS_STAGE_DUPLICATE, s);
+    launch_prefix_scatter(a, max_lim, c->pfx_cur, c->pv[0], tb.capacity, s, &c->launches);
+    launch_prefix_gather(a, n_gather, (uint32_t)n, c->pfx_rects, c->pfx_off, c->pv[0], tb.capacity, s, &c->launches);
+  }
+  {
+    StageTimer t(c, GS_STAGE_PAIR_SORT, s);
+    launch_tile_sort(tb, s, &c->launches);
+  }
+  GS_CHECK_LAUNCH(c, "prefix scatter / tile sort");
+  c->fwd_work_zero = c->bwd_work_zero = true;
+  c->st_pair_buf = 0;
+  c->st_ordered = tb.order != nullptr;
+  c->st_buckets = false;
+  c->st_cut = true;
+  *done = true;
   return GS_OK;
 }
 
 // Counting-scatter binning with per-tile sorts: count, scan (one host read of
 // the totals in sync mode), scatter, sort.  Falls back to the radix path when
-// some tile list is longer than the per-tile sort holds.  counted: the
+// some tile list is longer than the per-tile sort holds, by way of the lists'
+// nearest entries (bin_prefix) where tiles_y is given.  counted: the
 // projection already added every item's tiles to the (zeroed) tile
-// counters.
-gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, bool counted) {
+// counters, the large rectangles' (with tiles_y) to the difference grids.
+gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, bool counted,
+                       const int* tiles_y = nullptr) {
   const int64_t T = (int64_t)map.tile_base[map.views];
+  c->st_cut = false;
   if (c->sync) GS_CUDA(c, cudaMemsetAsync(c->d_overflow, 0, sizeof(uint32_t), s));
   TileBinArgs tb;
   tb.n = n;
@@ -542,6 +722,11 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
   tb.order = c->order_tiles ? c->torder : nullptr;
   tb.counted = counted;
   tb.scan_aux = c->scan_aux;
+  if (tiles_y) {
+    tb.big_diff = c->big_diff;
+    grid_layout(map, tiles_y, tb.big_base);
+    for (int v = 0; v < map.views; ++v) tb.tiles_y[v] = tiles_y[v];
+  }
   c->st_ordered = false;
   {
     StageTimer t(c, GS_STAGE_DUPLICATE, s);
@@ -563,7 +748,16 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
     c->bucket_ok = c->longest_seen <= entries / 2 && T * entries < ((int64_t)1 << 32) &&
                    ensure_buckets(c, T, (uint32_t)entries) == GS_OK &&
                    c->cap_bt * (int64_t)kLenClasses < ((int64_t)1 << 32);
-    if (longest > tile_sort_capacity()) return bin_and_sort_radix(c, n, map, s);
+    if (longest > tile_sort_capacity()) {
+      if (tiles_y && P <= 0xFFFFFFF0ll) {  // (more pairs than that are refused by the full binning)
+        bool done = false;
+        const gs_status ps = bin_prefix(c, n, map, tiles_y, s, 0, &done);
+        if (ps != GS_OK) return ps;
+        c->st_pairs = P;
+        if (done) return GS_OK;
+      }
+      return bin_and_sort_radix(c, n, map, s);
+    }
     gs_status st = ensure_pairs(c, std::max<int64_t>(P, 1));
     if (st != GS_OK) return st;
     tb.capacity = (uint32_t)std::min<int64_t>(c->cap_p, 0xFFFFFFF0ll);
@@ -575,14 +769,14 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
     StageTimer t(c, GS_STAGE_DUPLICATE, s);
     launch_tile_scatter(tb, s, &c->launches);
   }
-  tb.raster_work = c->persistent ? c->d_bigmeta + 1 : nullptr;
+  tb.raster_work = c->d_bigmeta + 1;
   {
     StageTimer t(c, GS_STAGE_PAIR_SORT, s);
     launch_tile_sort(tb, s, &c->launches);
   }
   GS_CHECK_LAUNCH(c, "tile scatter/sort");
   c->counts_zero = true;
-  if (tb.raster_work) c->fwd_work_zero = c->bwd_work_zero = true;
+  c->fwd_work_zero = c->bwd_work_zero = true;
   c->st_pairs = P;
   c->st_pair_buf = 0;
   c->st_ordered = tb.order != nullptr;
@@ -634,16 +828,16 @@ gs_status gs_ctx_create(gs_ctx** out, int device, int64_t pair_capacity) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_npairs, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_npairs_full, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_overflow, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_binstats, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_binstats, 5 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_step, sizeof(long long));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_dscale, kMaxViews * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_nvalid, kMaxViews * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(c->d_nvalid, 0, kMaxViews * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_bigmeta, 4 * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(c->d_bigmeta, 0, 4 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_bigmeta, 5 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMemset(c->d_bigmeta, 0, 5 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(c->d_step, 0, sizeof(long long));
   if (e == cudaSuccess) init_project_kernels();
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_evals, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_evals, 4 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemset(c->d_evals, 0, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemset(c->d_overflow, 0, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_bounds, sizeof(uint32_t));
@@ -703,6 +897,16 @@ gs_status gs_ctx_destroy(gs_ctx* c) {
   cudaFree(c->bids);
   cudaFree(c->cls_count);
   cudaFree(c->cls_tiles);
+  cudaFree(c->pfx_lim);
+  cudaFree(c->pfx_kept);
+  cudaFree(c->pfx_off);
+  cudaFree(c->pfx_cur);
+  cudaFree(c->pfx_cut);
+  cudaFree(c->pfx_level);
+  cudaFree(c->pfx_gather);
+  cudaFree(c->pfx_rects);
+  cudaFree(c->pfx_diff);
+  cudaFree(c->big_diff);
   cudaFree(c->qt_cells[0]);
   cudaFree(c->qt_cells[1]);
   cudaFree(c->qt_leaves);
@@ -957,8 +1161,9 @@ RasterArgs raster_args(gs_ctx* c, const gs_raster_cfg* cfg) {
   ra.n_ids = (uint32_t)std::min<int64_t>(c->st_buckets ? c->cap_bt * (int64_t)c->bucket_cap : c->cap_p, 0xFFFFFFFFll);
   ra.n_items = (uint32_t)(c->st_n * c->st_views);
   ra.order = c->st_ordered ? c->torder : nullptr;
-  ra.work = c->persistent ? c->d_bigmeta + 1 : nullptr;  // the forward counter; the backward pass uses [2]
+  ra.work = c->d_bigmeta + 1;  // the forward counter; the backward pass uses [2]
   ra.zero_work = true;
+  ra.persistent = c->persistent;
   ra.num_sms = c->num_sms;
   ra.loss_partials = nullptr;
   ra.w_color = 0.f;
@@ -1006,9 +1211,10 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   if ((st = layout_views(c, g->n, V, cams, cfg, L)) != GS_OK) return st;
   GS_CUDA(c, cudaSetDevice(c->device));
   const int n_items = (int)L.items;
+  uint32_t grid_base[kMaxViews] = {};
   if (c->sync) {
     if ((st = ensure_n(c, std::max(n_items, 1))) != GS_OK || (st = ensure_px(c, L.pixels)) != GS_OK ||
-        (st = ensure_tiles(c, L.tiles)) != GS_OK)
+        (st = ensure_tiles(c, L.tiles)) != GS_OK || (st = ensure_big(c, grid_layout(L.map, L.tiles_y, grid_base))) != GS_OK)
       return st;
   } else if (n_items > c->cap_n || L.pixels > c->cap_px || L.tiles > c->cap_t) {
     return fail(c, GS_ERR_CAPACITY, "no-sync mode: reserve items/pixels first (gs_ctx_reserve)");
@@ -1024,6 +1230,13 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   pa.nvalid = fl ? c->d_nvalid : nullptr;  // zeroed by the projection for the fused loss's count
   pa.step_inc = fl ? fl->step : nullptr;
   const bool buckets = !c->sync && c->bucket_ok && (int64_t)L.tiles <= c->cap_bt;
+  // large rectangles go to the difference grids (no-sync passes count tile by
+  // tile where no sync pass has sized the grids)
+  const bool grids = !buckets && grid_layout(L.map, L.tiles_y, grid_base) <= c->cap_big;
+  if (grids) {
+    pa.big_diff = c->big_diff;
+    for (int v = 0; v < V; ++v) pa.big_base[v] = grid_base[v];
+  }
   if (buckets) {  // and writes every pair into its tile's bucket
     pa.bucket_ids = c->bids;
     pa.bucket_cap = c->bucket_cap;
@@ -1034,7 +1247,9 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
     // every counter of the allocation, so that a later pass over more tiles
     // also starts from zeros
     GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta, 0, sizeof(uint32_t), s));
+    GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta + kHugeFlag, 0, sizeof(uint32_t), s));
     GS_CUDA(c, cudaMemsetAsync(c->tcount, 0, sizeof(uint32_t) * (size_t)c->cap_t, s));
+    if (c->big_diff) GS_CUDA(c, cudaMemsetAsync(c->big_diff, 0, sizeof(int) * (size_t)c->cap_big, s));
   }
   c->counts_zero = false;
   {
@@ -1044,7 +1259,10 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   if (g->n > 0) c->launches += 1;
   GS_CHECK_LAUNCH(c, "project_fwd");
 
-  if ((st = buckets ? bin_buckets(c, n_items, L.map, s) : bin_and_sort(c, n_items, L.map, s, true)) != GS_OK)
+  if (c->counting)  // (a pass over cut lists may be repeated)
+    GS_CUDA(c, cudaMemcpyAsync(c->d_evals + 2, c->d_evals, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+  if ((st = buckets ? bin_buckets(c, n_items, L.map, s)
+                    : bin_and_sort(c, n_items, L.map, s, true, grids ? L.tiles_y : nullptr)) != GS_OK)
     return st;
 
   c->st_n = g->n;
@@ -1060,6 +1278,7 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   c->st_map = L.map;
   c->st_sh = g->sh_degree;
 
+  for (int attempt = 0;; ++attempt) {
   RasterArgs ra = raster_args(c, cfg);
   for (int v = 0; v < V; ++v) {
     ra.v[v].color = color ? color[v] : nullptr;
@@ -1093,6 +1312,23 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   c->fwd_work_zero = false;
   c->launches += 1;
   GS_CHECK_LAUNCH(c, "raster_fwd");
+  if (!c->st_cut) break;
+  launch_raster_open(ra, c->last, c->pfx_cut, c->pfx_level, c->d_binstats + 4, s);
+  c->launches += 1;
+  GS_CHECK_LAUNCH(c, "raster_open");
+  GS_CUDA(c, cudaMemcpyAsync(c->h_pinned, c->d_binstats + 4, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+  GS_CUDA(c, cudaStreamSynchronize(s));
+  if (c->h_pinned[0] == 0) break;
+  // some list was cut too short: bin again with longer ones (the third time
+  // in full, which no pixel can exhaust)
+  if (attempt == 2) return fail(c, GS_ERR_CUDA, "a full list left a pixel open");
+  if (c->counting)
+    GS_CUDA(c, cudaMemcpyAsync(c->d_evals, c->d_evals + 2, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+  if (fl) GS_CUDA(c, cudaMemsetAsync(c->d_nvalid, 0, kMaxViews * sizeof(uint32_t), s));
+  bool done = false;
+  if ((st = bin_prefix(c, n_items, L.map, L.tiles_y, s, attempt + 1, &done)) != GS_OK) return st;
+  if (!done && (st = bin_and_sort_radix(c, n_items, L.map, s)) != GS_OK) return st;
+  }
   c->st_g = *g;
   for (int v = 0; v < V; ++v) {
     c->st_cam[v] = cams[v];
@@ -1138,7 +1374,7 @@ gs_status raster_backward(gs_ctx* c, const gs_raster_cfg* cfg, const float* cons
   // the buffer is new): then clear the whole buffer once
   if (!c->g2d_zero) GS_CUDA(c, cudaMemsetAsync(c->g2d, 0, sizeof(float4) * 3 * (size_t)c->cap_n, s));
   RasterArgs ra = raster_args(c, cfg);
-  if (ra.work) ra.work = c->d_bigmeta + 2;
+  ra.work = c->d_bigmeta + 2;
   ra.zero_work = !c->bwd_work_zero;
   ra.depth_scale = depth_scale;
   if (nvalid_w_depth) {  // the fused loss: dL/dD scale w_depth / (valid target depths) per view
@@ -1934,6 +2170,12 @@ gs_status gs_get_tile_ranges(gs_ctx* c, uint32_t* ranges, int64_t n_tiles, gs_st
   if (!ranges || n_tiles != c->st_tiles)
     return fail(c, GS_ERR_INVALID_ARG, "gs_get_tile_ranges: ranges is NULL or n_tiles is not the forward pass's");
   GS_CUDA(c, cudaSetDevice(c->device));
+  if (c->st_cut) {  // the full lists' ranges, of which the pass has the nearest entries
+    launch_full_ranges(c->toffset, c->tcount, (int)n_tiles, (uint2*)ranges, (cudaStream_t)stream);
+    c->launches += 1;
+    GS_CHECK_LAUNCH(c, "full ranges");
+    return GS_OK;
+  }
   GS_CUDA(c, cudaMemcpyAsync(ranges, c->ranges, sizeof(uint2) * (size_t)n_tiles, cudaMemcpyDeviceToDevice,
                              (cudaStream_t)stream));
   return GS_OK;
@@ -1942,7 +2184,8 @@ gs_status gs_get_tile_ranges(gs_ctx* c, uint32_t* ranges, int64_t n_tiles, gs_st
 gs_status gs_get_tile_order(gs_ctx* c, uint32_t* order, int64_t n_tiles, gs_stream_t stream) {
   if (!c) return GS_ERR_INVALID_ARG;
   if (!c->have_state) return fail(c, GS_ERR_STATE, "no forward pass on this context");
-  if (!c->st_ordered) return fail(c, GS_ERR_STATE, "the last forward pass visited the tiles in index order");
+  if (!c->st_ordered || c->st_cut)
+    return fail(c, GS_ERR_STATE, "the last forward pass did not visit the tiles in the order of their lists' lengths");
   if (!order || n_tiles != c->st_tiles)
     return fail(c, GS_ERR_INVALID_ARG, "gs_get_tile_order: order is NULL or n_tiles is not the forward pass's");
   GS_CUDA(c, cudaSetDevice(c->device));

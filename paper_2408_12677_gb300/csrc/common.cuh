@@ -237,6 +237,47 @@ __device__ __forceinline__ uint32_t warp_agg_inc(uint32_t* __restrict__ counter,
   return base + __popc(peers & ((1u << lane) - 1u));
 }
 
+// Adds x (the same on every active lane) to *p, equal addresses of the active
+// lanes in one atomic.
+__device__ __forceinline__ void warp_agg_add(int* p, int x, unsigned active) {
+  const unsigned peers = __match_any_sync(active, (unsigned long long)p);
+  if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(p, x * __popc(peers));
+}
+
+// 2D prefix sum of a difference grid of (TX + 1) x (TY + 1) cells by one block
+// of THREADS threads (rows by warps, then columns by threads), which turns
+// rectangles added as four corners into per-tile counts; f(tile, &cell, count)
+// is called for every tile of the TX x TY (row-major).
+template <int THREADS, class F>
+__device__ __forceinline__ void integrate_grid(int* __restrict__ g, int TX, int TY, F f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = TX + 1;
+  for (int y = warp; y < TY; y += THREADS / 32) {
+    int carry = 0;
+    for (int x0 = 0; x0 < TX; x0 += 32) {
+      const int x = x0 + lane;
+      int c = x < TX ? g[(size_t)y * w + x] : 0;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xFFFFFFFFu, c, off);
+        if (lane >= off) c += o;
+      }
+      c += carry;
+      if (x < TX) g[(size_t)y * w + x] = c;
+      carry = __shfl_sync(0xFFFFFFFFu, c, 31);
+    }
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < TX; x += THREADS) {
+    int run = 0;
+#pragma unroll 8
+    for (int y = 0; y < TY; ++y) {
+      run += g[(size_t)y * w + x];
+      g[(size_t)y * w + x] = run;
+      f(y * TX + x, &g[(size_t)y * w + x], run);
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Bounds-checked build (compiled with -DGS_CHECKED into libgsplat_checked.so):
 // every index read from memory (list ids, tile ranges, tile numbers computed

@@ -32,10 +32,16 @@ struct TileMap {
 // block that owns them (large splats cluster, which would leave a few blocks
 // running long).
 constexpr uint32_t kBigTiles = 32;
+constexpr int kHugeFlag = 4;
+
+// Gaussians covering more than this many tiles are counted by four corners of
+// a difference grid instead of tile by tile.  Integrating the grid takes the
+// tile scan 5-20 us (when there are any), 2000 to 10000 atomics' time.
+constexpr uint32_t kHugeTiles = 1024;
 
 struct ProjectArgs {
   uint32_t* big_queue;  // items with more than kBigTiles tiles
-  uint32_t* big_len;    // queue length (zeroed before the launch)
+  uint32_t* big_len;    // queue length (zeroed before the launch); big_len[kHugeFlag] != 0: the grids are in use
   int n;                // Gaussians
   int views;
   const float *means, *log_scales, *quats, *logits, *sh;
@@ -48,6 +54,11 @@ struct ProjectArgs {
   uint32_t* counts;               // per global tile (zeroed, nullable): the projection adds every
                                   // item's tiles
   uint32_t* nvalid = nullptr;     // per view (nullable): zeroed by the projection (block 0)
+  // nullable (no bucket mode): rectangles of more than kHugeTiles tiles are
+  // added to their view's difference grid (first cell big_base[v], tiles_x + 1
+  // cells per row) instead of to the counts; the tile scan integrates it
+  int* big_diff = nullptr;
+  uint32_t big_base[kMaxViews] = {};
   // per-tile buckets (nullable; graph-mode binning): every (item, tile) pair
   // is written straight to bucket_ids[tile * bucket_cap + slot], slot taken
   // from the tile's counter (a pair beyond the capacity sets bit 4 of
@@ -212,6 +223,11 @@ struct TileBinArgs {
   uint32_t* order;            // per tile (output, nullable): visit order, longest lists first
   bool counted;               // counts already hold every item's tiles (the projection counted them)
   uint32_t* scan_aux;         // scratch of tile_scan_aux_size(n_tiles) words for the multi-block scan
+  bool long_sorted = false;   // lists longer than the per-tile sort holds are in order already (left as they are)
+  int* big_diff = nullptr;    // nullable: difference grids of the large rectangles, added to the counts (and
+                              // zeroed) by the scan when there are any (see ProjectArgs)
+  uint32_t big_base[kMaxViews] = {};
+  int tiles_y[kMaxViews] = {};
   uint32_t* raster_work = nullptr;  // nullable: the forward and backward raster job counters, zeroed by the sort
   // bucket mode (nullable): the lists are the projection's per-tile buckets
   // (bucket_ids, tile t's list at t * bucket_cap, its length in counts[t]);
@@ -230,11 +246,44 @@ void launch_tile_count_scan(const TileBinArgs& a, cudaStream_t s, int64_t* launc
 void launch_tile_scatter(const TileBinArgs& a, cudaStream_t s, int64_t* launches);
 void launch_tile_sort(const TileBinArgs& a, cudaStream_t s, int64_t* launches);
 
+// long lists cut to their nearest entries (prefix.cu)
+constexpr int kPrefixSlabs = 50;  // enough for 2^31 ranks
+struct PrefixArgs {
+  TileMap map;
+  int tiles_y[kMaxViews];
+  uint32_t grid_base[kMaxViews];  // first cell of each view's (tiles_x + 1) x (tiles_y + 1) grid
+  uint32_t grid_cells;            // cells of a slab's grids
+  uint32_t ranks;                 // items looked at, nearest first
+  int slabs;
+  uint32_t bound[kPrefixSlabs];   // first rank behind each slab
+  uint32_t target;                // entries a tile of level 0 should get
+  const uint32_t* sorted;         // items by depth
+  const ushort4* rects;
+  const uint32_t* tiles;          // per item
+  int* diff;                      // scratch: slabs x grid_cells
+  const uint32_t* full;           // per tile: length of its full list
+  const uint8_t* level;           // per tile: 0 the target, 1 up to kTileSortCap entries, 2 all of them
+  uint32_t *lim, *kept;           // per tile (output): ranks below lim are kept; kept entries
+  uint8_t* cut;                   // per tile (output): 1 = not the full list
+  unsigned long long* max_lim;    // largest lim (output)
+  uint32_t* gather;               // the tiles of level 2 (output), *n_gather of them
+  unsigned long long* n_gather;
+};
+void prefix_slabs(PrefixArgs& a, uint32_t ranks);  // sets ranks, slabs, bound
+void launch_prefix_choose(const PrefixArgs& a, cudaStream_t s, int64_t* launches);
+void launch_prefix_scatter(const PrefixArgs& a, uint32_t max_lim, uint32_t* cursors, uint32_t* ids, uint32_t capacity,
+                           cudaStream_t s, int64_t* launches);
+// the level-2 tiles' lists out of all n items; srects: scratch of n rectangles
+void launch_prefix_gather(const PrefixArgs& a, uint32_t n_gather, uint32_t n, ushort4* srects, const uint32_t* offsets,
+                          uint32_t* ids, uint32_t capacity, cudaStream_t s, int64_t* launches);
+// out[t] = tile t's range in the full (virtual) pair list
+void launch_full_ranges(const uint32_t* offsets, const uint32_t* full, int n, uint2* out, cudaStream_t s);
+
 void launch_tile_ranges(const uint32_t* sorted_tiles, const uint32_t* n_dev, uint32_t n_max, uint2* ranges,
                         int n_tiles, int num_sms, cudaStream_t s, int64_t* launches);
 
-// raster passes: one CTA per global tile, visited in `order` when given
-// (the tile list sorted by descending list length) else in index order
+// raster passes: warps take regions of the tiles, in `order` when given (the
+// tiles by descending list length) else in index order
 struct RasterView {
   int width, height, tiles_x;
   uint32_t tile_base;  // first global tile of the view
@@ -256,8 +305,9 @@ struct RasterArgs {
   const float4* feat;
   uint32_t n_ids, n_items;  // entries of ids, records of feat (bounds of the checked build)
   const uint32_t* order;  // nullable
-  uint32_t* work;         // nullable: job counter of the persistent form
+  uint32_t* work;         // job counter
   bool zero_work;         // the launcher zeroes *work first (it is not known to be 0)
+  bool persistent;        // as many CTAs as the GPU holds at once, else one warp per job
   int num_sms;
   // fused loss (forward): per warp job partial sums {|colour residual|,
   // |depth residual| over valid targets, valid count} at
@@ -306,6 +356,10 @@ void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsig
 void launch_loss_tiles_finalize(const RasterArgs& a, float w_depth, float* loss, float* depth_scale,
                                 float* partials, uint32_t* ticket, long long* step, cudaStream_t s,
                                 int64_t* launches);
+// after a forward pass over cut lists: level[t] is raised and *open set for a
+// tile with cut[t] whose list ends before all of its pixels have stopped
+void launch_raster_open(const RasterArgs& a, const int32_t* last, const uint8_t* cut, uint8_t* level,
+                        unsigned long long* open, cudaStream_t s);
 void launch_raster_bwd(const RasterArgs& a, const float* T_final, const int32_t* last, float4* g2d, cudaStream_t s);
 
 // loss and optimiser: per view v, L_v = w_color mean |C - C^| + w_depth

@@ -342,7 +342,21 @@ __global__ void __launch_bounds__(kFwdThreads) project_fwd_kernel(const __grid_c
       const uint32_t nt = (uint32_t)(x1 - x0) * (uint32_t)(y1 - y0);
       block_count_tiles(a.counts, a.tile_base[v], a.tiles_x[v], x0, y0, x1, y1, nt <= kBigTiles ? nt : 0u, s_cnt,
                         s_box, a.bucket_ids, a.bucket_cap, a.overflow, (uint32_t)it);
-      unsigned big = __ballot_sync(0xFFFFFFFFu, nt > kBigTiles);
+      const bool huge = a.big_diff && nt > kHugeTiles;
+      const unsigned act = __ballot_sync(0xFFFFFFFFu, huge);
+      if (huge) {
+        // four corners instead of one atomic per tile (1.66 ms -> 0.08 ms with
+        // 200k rectangles of 4000 tiles); equal corners of a warp's
+        // rectangles, as those of clipped ones are, go in one atomic
+        const int w = a.tiles_x[v] + 1;
+        int* g = a.big_diff + a.big_base[v];
+        warp_agg_add(g + y0 * w + x0, 1, act);
+        warp_agg_add(g + y0 * w + x1, -1, act);
+        warp_agg_add(g + y1 * w + x0, -1, act);
+        warp_agg_add(g + y1 * w + x1, 1, act);
+        a.big_len[kHugeFlag] = 1u;
+      }
+      unsigned big = __ballot_sync(0xFFFFFFFFu, nt > kBigTiles && !huge);
       const int lane = threadIdx.x & 31;
       while (big) {
         const int src = __ffs(big) - 1;

@@ -21,6 +21,7 @@
 // 168 -> 100 us at 1200 x 680 with 300k Gaussians, 811 -> 654 us and 1759 ->
 // 1110 us for five such views.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -59,6 +60,9 @@ struct WarpMap {
   static_assert(TW * TH == 256 && TW % RW == 0 && TH % RH == 0 && JOBS == 8 / PPL, "regions tile the tile");
 };
 
+// Flag in a pixel's stored list position: it did not stop before the list's end.
+constexpr int kOpen = (int)0x80000000u;
+
 // One list entry in tile-local coordinates:
 //   a = {mu_x, mu_y, i0, -k}, b = {i1, log2 opacity, z, support radius r2},
 //   c = {r, g, b, item id}
@@ -91,6 +95,11 @@ __device__ __forceinline__ void cp_record(float4* dst, const float4* __restrict_
 }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// Support boxes of more than 512 tiles (half-extents' product): so many blocks
+// add to such a splat's gradient record that they queue up at its address, at
+// about 5 ns an addition (32 per tile).
+constexpr float kWide = 512.f * 256.f / 4.f;
+
 // Converts a gathered record to tile-local coordinates and tests the splat's
 // support bounding box against the blocks of the warp's region, whose first
 // pixel is (bx, by): bit l of the result is set when the box meets the pixel
@@ -98,10 +107,12 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 // accept: q' <= min(qmax, log2 o - log2 alpha_min) is the ellipse
 // (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents sqrt(R2) / i0 and
 // sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2); the widening covers float32 rounding
-// of the test and of the hardware square roots and reciprocals.
+// of the test and of the hardware square roots and reciprocals.  `wide`: the
+// box has more than 4 kWide pixels.
 template <class M>
 __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, float ox, float oy, float bx, float by,
-                                               const RasterParams& rp, uint32_t id, Entry& e) {
+                                               const RasterParams& rp, uint32_t id, Entry& e, bool& wide) {
+  wide = false;
   const float mlx = __fadd_rn(__fsub_rn(f0.x, ox), f0.z);
   const float mly = __fadd_rn(__fsub_rn(f0.y, oy), f0.w);
   const float R2 = fminf(rp.qmax_s, __fsub_rn(f1.w, rp.log2_alpha_min));
@@ -113,6 +124,7 @@ __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, 
   const float inv0 = rcp_approx(f1.x), inv1 = rcp_approx(f1.z);
   const float ex = Rr * inv0 + 1e-3f;
   const float ey = Rr * sqrt_approx(f1.y * f1.y * inv0 * inv0 + inv1 * inv1) + 1e-3f;
+  wide = ex * ey > kWide;
   // first and last block column and row whose centres lie within the box
   constexpr float BW = M::LPG, BH = M::ROWS, NC = M::RW / M::LPG, NR = M::RH / M::ROWS;
   const float rx = mlx - bx, ry = mly - by;
@@ -186,14 +198,16 @@ struct Walk {
     fetch(0);
   }
   // Converts the chunk at `top` and puts the following one into flight;
-  // returns its entries that meet the lane's group (bit i: entry i).
-  __device__ __forceinline__ unsigned stage(const RasterParams& rp) {
+  // returns its entries that meet the lane's group (bit i: entry i), in m the
+  // blocks that the lane's entry meets, in wide whether it is wide.
+  __device__ __forceinline__ unsigned stage(const RasterParams& rp, unsigned& m, bool& wide) {
     cp_wait_all();
     Entry e;
-    unsigned m = 0u;
+    m = 0u;
+    wide = false;
     if (chunk(top) + lane < n) {
       const float4* raw = sm->raw[lane];
-      m = make_entry<M>(raw[0], raw[1], raw[2], ox, oy, bx, by, rp, g_raw, e);
+      m = make_entry<M>(raw[0], raw[1], raw[2], ox, oy, bx, by, rp, g_raw, e, wide);
     }
     __syncwarp();  // every lane has read its last entry of the chunk that is overwritten
     if (m) sm->e[(top & (kRing - 1)) + lane] = e;
@@ -392,7 +406,8 @@ __device__ __forceinline__ f2x f2_fma_s(f2x x, float s, f2x y) {
 // row coordinate set to infinity, so that no entry accepts it; the clamp and
 // the stop of a pixel are branches that most entries do not take.  Stored per
 // pixel: the final T and the number of list entries in front of the one that
-// it stopped at (of the last entry that meets its block if it did not stop).
+// it stopped at (of the last entry that meets its block, and the flag kOpen,
+// if it did not stop).
 template <int TW, int TH, int PPL, bool COUNT, bool LOSS>
 __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams& rp, uint32_t tile, int quad,
                                         WarpSmem& sm, float* __restrict__ T_final_all,
@@ -451,7 +466,9 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
         if (__all_sync(kFull, out)) break;
         static_assert(M::LPG == 1, "a lane by itself");
         gone = out ? 1u : 0u;
-        walk.push(walk.stage(rp));
+        unsigned m;
+        bool wide;
+        walk.push(walk.stage(rp, m, wide));
         if (out) walk.drop();
         continue;
       }
@@ -557,7 +574,7 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
     if (depth) depth[p] = Df;
     if (alpha) alpha[p] = 1.f - Tf;
     T_final[p] = Tf;
-    last_out[p] = min(stop[s], walk.met);
+    last_out[p] = stop[s] == 0x7fffffff ? walk.met | kOpen : stop[s];
     if constexpr (LOSS) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -613,8 +630,8 @@ __device__ __forceinline__ uint32_t fwd_visit_tile(const RasterArgs& a, const ui
   return tile;
 }
 
-// `work` null: warp w of the grid on job w.  Otherwise a persistent grid whose
-// warps pull jobs from `work` with next_job.
+// The warps of the grid (a persistent one, or one warp per job) pull jobs from
+// `work` with next_job.
 template <int TW, int TH, int PPL, bool COUNT, bool LOSS>
 __global__ void __launch_bounds__(kThreads, kFwdCtas) raster_fwd_kernel(const __grid_constant__ RasterArgs a, RasterParams rp,
                                                               float* __restrict__ T_final_all,
@@ -629,12 +646,11 @@ __global__ void __launch_bounds__(kThreads, kFwdCtas) raster_fwd_kernel(const __
   if (a.cls_count) load_class_starts(a, s_start);  // CTA-uniform
   init_warp_smem(s_w[warp]);
   const uint32_t n_jobs = JOBS * a.n_tiles;
-  uint32_t job = blockIdx.x * (kThreads / 32) + warp;
-  while (work ? next_job(work, n_jobs, job) : job < n_jobs) {
+  uint32_t job;
+  while (next_job(work, n_jobs, job)) {
     const int quad = (int)(job % JOBS);
     fwd_job<TW, TH, PPL, COUNT, LOSS>(a, rp, fwd_visit_tile(a, s_start, job / JOBS, quad), quad, s_w[warp], T_final_all,
                                       last_all, counters);
-    if (!work) break;
   }
 }
 
@@ -676,6 +692,41 @@ __device__ __forceinline__ void group_reduce_add10(const float (&v)[10], int lan
     add_part(rec, l1 ? 1 : 0, x[0], x[1], x[2], l1 ? 0.f : x[3]);
     if (l1) add_part(rec, 2, x[3], x[4], x[5], 0.f);
   }
+}
+
+// float offset of gradient value k in the record
+__device__ __forceinline__ int rec_off(int k) { return k < 7 ? k : k + 1; }
+
+// Sums v[0..9] over the warp with exchanges that halve the number of values
+// each lane carries (xor 16: 10 -> 5, xor 8: 5 -> 3, xor 4: 3 -> 2, xor 2: 2
+// -> 1) and a final xor-1 step (12 shuffles instead of 50), then adds the
+// totals to the record: even lanes hold distinct values, so this is one
+// warp-wide scalar atomic add.
+__device__ __forceinline__ void warp_reduce_add10(const float (&v)[10], int lane, float* __restrict__ rec) {
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+  float u[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i)  // keep v[i] (b4 = 0) or v[i + 5] (b4 = 1)
+    u[i] = (b4 ? v[i + 5] : v[i]) + __shfl_xor_sync(kFull, b4 ? v[i] : v[i + 5], 16);
+  float w3[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {  // keep u[0..2] (b3 = 0) or u[3..4], 0 (b3 = 1)
+    const float hi = i < 2 ? u[i + 3] : 0.f;
+    w3[i] = (b3 ? hi : u[i]) + __shfl_xor_sync(kFull, b3 ? u[i] : hi, 8);
+  }
+  float w2[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {  // keep w3[0..1] (b2 = 0) or w3[2], 0 (b2 = 1)
+    const float hi = i < 1 ? w3[i + 2] : 0.f;
+    w2[i] = (b2 ? hi : w3[i]) + __shfl_xor_sync(kFull, b2 ? w3[i] : hi, 4);
+  }
+  float x = (b1 ? w2[1] : w2[0]) + __shfl_xor_sync(kFull, b1 ? w2[0] : w2[1], 2);
+  x += __shfl_xor_sync(kFull, x, 1);
+  // value held: 5 b4 + i3 with i3 = 3 b3 + 2 b2 + b1 among the five kept at
+  // xor 16; lanes with b2 and (b3 or b1) hold the zero pads
+  const int i3 = (b3 ? 3 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
+  const bool valid = !(b2 && (b3 || b1));
+  if (!(lane & 1) && valid && x != 0.f) atomicAdd(&rec[rec_off((b4 ? 5 : 0) + i3)], x);
 }
 
 // Backward pass of region `quad` of the tile of visit k by one warp: back to
@@ -730,7 +781,7 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
       if (s < PPL && px < width && py + s < height) {
         const size_t q = (size_t)(py + s) * width + px;
         t[h] = T_final[q];
-        last[s] = last_in[q];
+        last[s] = last_in[q] & ~kOpen;
         c0[h] = dLdc[q];
         c1[h] = dLdc[HW + q];
         c2[h] = dLdc[2 * HW + q];
@@ -768,94 +819,132 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
   walk.by = (float)byi;
   walk.begin();
   const f2x ONE2 = f2_pack(1.f, 1.f);
+  // every group's next entry
+  auto entry = [&](auto whole_warp) {
+          int idx;
+          const Entry& en = sm.e[walk.take(idx)];
+          const float4 ea = en.a, eb = en.b, ec = en.c;
+          const float dx = __fsub_rn(plx, ea.x);
+          const float t0 = __fmul_rn(ea.z, dx);
+          f2x TQ[NP], WQ[NP];
+          float ar[2 * NP], in[2 * NP];
+    #pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const f2x DY = f2_sub(PLY[p], f2_bcast(ea.y));
+            WQ[p] = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
+            TQ[p] = f2_mul(WQ[p], f2_bcast(eb.x));
+            const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ[p], TQ[p]));
+            const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
+            ar[2 * p] = ex2_approx(f2_lo(ARG));
+            ar[2 * p + 1] = ex2_approx(f2_hi(ARG));
+            in[2 * p] = one_if_le_and(f2_lo(Q), eb.w, idx, last[2 * p]);
+            in[2 * p + 1] = one_if_le_and(f2_hi(Q), eb.w, idx, last[2 * p + 1]);
+          }
+          f2x AL[NP], AG[NP];  // alpha, and alpha where it is not clamped: 0 where the pixel takes no part
+    #pragma unroll
+          for (int p = 0; p < NP; ++p) AL[p] = AG[p] = f2_mul(f2_pack(ar[2 * p], ar[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
+          if (eb.y > rp.log2_clamp) {  // the 0.99 clamp has zero gradient
+    #pragma unroll
+            for (int p = 0; p < NP; ++p) {
+              const bool c0 = f2_lo(AL[p]) > rp.alpha_max, c1 = f2_hi(AL[p]) > rp.alpha_max;
+              AG[p] = f2_pack(c0 ? 0.f : f2_lo(AL[p]), c1 ? 0.f : f2_hi(AL[p]));
+              AL[p] = f2_pack(c0 ? rp.alpha_max : f2_lo(AL[p]), c1 ? rp.alpha_max : f2_hi(AL[p]));
+            }
+          }
+          f2x GA = 0, GT = 0, GW = 0, V6 = 0, V7 = 0, V8 = 0, V9 = 0;  // sums over the lane's pairs
+    #pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const f2x OM = f2_sub(ONE2, AL[p]);  // in [0.01, 1]; 1 where the pixel takes no part: T, U unchanged
+            const f2x INV = f2_pack(rcp_approx(f2_lo(OM)), rcp_approx(f2_hi(OM)));
+            T[p] = f2_mul(T[p], INV);  // transmittance in front of this Gaussian
+            const f2x W = f2_mul(AL[p], T[p]);
+            const f2x CD = f2_fma_s(C0[p], ec.x, f2_fma_s(C1[p], ec.y, f2_fma_s(C2[p], ec.z, f2_mul(DD[p], f2_bcast(eb.z)))));
+            // d/d alpha_i: colour/depth T_i c_i - (sum behind)/(1 - alpha_i); alpha image + T_final/(1 - alpha_i)
+            const f2x GAL = f2_sub(f2_mul(T[p], CD), f2_mul(U[p], INV));
+            U[p] = f2_fma(W, CD, U[p]);
+            const f2x g = f2_mul(GAL, AG[p]);
+            const f2x gt = f2_mul(g, TQ[p]);
+            if (p == 0) {
+              GA = g;
+              GT = gt;
+              GW = f2_mul(gt, WQ[p]);
+              V6 = f2_mul(W, DD[p]);
+              V7 = f2_mul(W, C0[p]);
+              V8 = f2_mul(W, C1[p]);
+              V9 = f2_mul(W, C2[p]);
+            } else {
+              GA = f2_add(GA, g);
+              GT = f2_add(GT, gt);
+              GW = f2_fma(gt, WQ[p], GW);
+              V6 = f2_fma(W, DD[p], V6);
+              V7 = f2_fma(W, C0[p], V7);
+              V8 = f2_fma(W, C1[p], V8);
+              V9 = f2_fma(W, C2[p], V9);
+            }
+          }
+          float v[10];
+          v[5] = f2_lo(GA) + f2_hi(GA);
+          v[1] = f2_lo(GT) + f2_hi(GT);
+          v[4] = f2_lo(GW) + f2_hi(GW);
+          v[6] = f2_lo(V6) + f2_hi(V6);
+          v[7] = f2_lo(V7) + f2_hi(V7);
+          v[8] = f2_lo(V8) + f2_hi(V8);
+          v[9] = f2_lo(V9) + f2_hi(V9);
+          v[0] = v[5] * t0;
+          v[2] = v[0] * dx;
+          v[3] = v[1] * dx;
+          float* rec = g2d + 12 * (size_t)__float_as_uint(ec.w);
+          if constexpr (decltype(whole_warp)::value)
+            warp_reduce_add10(v, lane, rec);
+          else
+            group_reduce_add10<M::LPG>(v, lane, rec);
+  };
+  // The entries of a chunk from its first to its last wide one are held back
+  // until the groups are done with what comes before, and then walked by all
+  // groups together, every entry on every block: each Gaussian's sums go over
+  // the whole warp and to its record once, not once per block (the nearest
+  // splats of a map of large ones cover the image: 257k additions to one
+  // record took 1.30 ms where the pass now takes 0.13).
+  unsigned held = 0u, rest = 0u;  // the wide entries; the group's entries of the chunk after them
+  bool together = false;
   for (;;) {
     while (__any_sync(kFull, walk.cur == 0u && walk.off < walk.top)) walk.step();
-    const bool can = walk.can_stage();
+    const bool can = walk.can_stage() && !together && !held;
     if (can && __any_sync(kFull, walk.cur == 0u)) {  // a group is dry
-      unsigned mine = walk.stage(rp);
+      unsigned m;
+      bool wide;
+      unsigned mine = walk.stage(rp, m, wide);
       const int over = walk.chunk(walk.top) + 32 - glast;  // entries behind every pixel of the group
       if (over > 0) mine = over < 32 ? mine & (kFull >> over) : 0u;
+      const unsigned w = __ballot_sync(kFull, m != 0u && wide);
+      if (w) {  // (entry 31 comes first)
+        const unsigned behind = kFull << (31 - __clz(w)) << 1, front = (1u << (__ffs(w) - 1)) - 1u;
+        held = __ballot_sync(kFull, m != 0u) & ~behind & ~front;
+        rest = mine & front;
+        mine &= behind;
+      }
       walk.push(mine);
       continue;
     }
-    const int lim = walk.limit(can);
-    if (lim == walk.kEnd) break;
-    if (lim == walk.kAgain) continue;
-    do {
-      int idx;
-      const Entry& en = sm.e[walk.take(idx)];
-      const float4 ea = en.a, eb = en.b, ec = en.c;
-      const float dx = __fsub_rn(plx, ea.x);
-      const float t0 = __fmul_rn(ea.z, dx);
-      f2x TQ[NP], WQ[NP];
-      float ar[2 * NP], in[2 * NP];
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const f2x DY = f2_sub(PLY[p], f2_bcast(ea.y));
-        WQ[p] = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
-        TQ[p] = f2_mul(WQ[p], f2_bcast(eb.x));
-        const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ[p], TQ[p]));
-        const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
-        ar[2 * p] = ex2_approx(f2_lo(ARG));
-        ar[2 * p + 1] = ex2_approx(f2_hi(ARG));
-        in[2 * p] = one_if_le_and(f2_lo(Q), eb.w, idx, last[2 * p]);
-        in[2 * p + 1] = one_if_le_and(f2_hi(Q), eb.w, idx, last[2 * p + 1]);
-      }
-      f2x AL[NP], AG[NP];  // alpha, and alpha where it is not clamped: 0 where the pixel takes no part
-#pragma unroll
-      for (int p = 0; p < NP; ++p) AL[p] = AG[p] = f2_mul(f2_pack(ar[2 * p], ar[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
-      if (eb.y > rp.log2_clamp) {  // the 0.99 clamp has zero gradient
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          const bool c0 = f2_lo(AL[p]) > rp.alpha_max, c1 = f2_hi(AL[p]) > rp.alpha_max;
-          AG[p] = f2_pack(c0 ? 0.f : f2_lo(AL[p]), c1 ? 0.f : f2_hi(AL[p]));
-          AL[p] = f2_pack(c0 ? rp.alpha_max : f2_lo(AL[p]), c1 ? rp.alpha_max : f2_hi(AL[p]));
-        }
-      }
-      f2x GA = 0, GT = 0, GW = 0, V6 = 0, V7 = 0, V8 = 0, V9 = 0;  // sums over the lane's pairs
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const f2x OM = f2_sub(ONE2, AL[p]);  // in [0.01, 1]; 1 where the pixel takes no part: T, U unchanged
-        const f2x INV = f2_pack(rcp_approx(f2_lo(OM)), rcp_approx(f2_hi(OM)));
-        T[p] = f2_mul(T[p], INV);  // transmittance in front of this Gaussian
-        const f2x W = f2_mul(AL[p], T[p]);
-        const f2x CD = f2_fma_s(C0[p], ec.x, f2_fma_s(C1[p], ec.y, f2_fma_s(C2[p], ec.z, f2_mul(DD[p], f2_bcast(eb.z)))));
-        // d/d alpha_i: colour/depth T_i c_i - (sum behind)/(1 - alpha_i); alpha image + T_final/(1 - alpha_i)
-        const f2x GAL = f2_sub(f2_mul(T[p], CD), f2_mul(U[p], INV));
-        U[p] = f2_fma(W, CD, U[p]);
-        const f2x g = f2_mul(GAL, AG[p]);
-        const f2x gt = f2_mul(g, TQ[p]);
-        if (p == 0) {
-          GA = g;
-          GT = gt;
-          GW = f2_mul(gt, WQ[p]);
-          V6 = f2_mul(W, DD[p]);
-          V7 = f2_mul(W, C0[p]);
-          V8 = f2_mul(W, C1[p]);
-          V9 = f2_mul(W, C2[p]);
-        } else {
-          GA = f2_add(GA, g);
-          GT = f2_add(GT, gt);
-          GW = f2_fma(gt, WQ[p], GW);
-          V6 = f2_fma(W, DD[p], V6);
-          V7 = f2_fma(W, C0[p], V7);
-          V8 = f2_fma(W, C1[p], V8);
-          V9 = f2_fma(W, C2[p], V9);
-        }
-      }
-      float v[10];
-      v[5] = f2_lo(GA) + f2_hi(GA);
-      v[1] = f2_lo(GT) + f2_hi(GT);
-      v[4] = f2_lo(GW) + f2_hi(GW);
-      v[6] = f2_lo(V6) + f2_hi(V6);
-      v[7] = f2_lo(V7) + f2_hi(V7);
-      v[8] = f2_lo(V8) + f2_hi(V8);
-      v[9] = f2_lo(V9) + f2_hi(V9);
-      v[0] = v[5] * t0;
-      v[2] = v[0] * dx;
-      v[3] = v[1] * dx;
-      group_reduce_add10<M::LPG>(v, lane, g2d + 12 * (size_t)__float_as_uint(ec.w));
-    } while (can ? !__any_sync(kFull, walk.cur == 0u) : walk.any_up_to(lim));
+    int lim = walk.end;
+    if (!together && !held) {
+      lim = walk.limit(can);
+      if (lim == walk.kEnd) break;
+      if (lim == walk.kAgain) continue;
+    } else if (!__any_sync(kFull, walk.cur != 0u)) {  // the wide entries' turn, or they are done
+      walk.base = walk.off = walk.top - 32;
+      walk.cur = together ? rest : held;
+      together = !together;
+      held = 0u;
+      continue;
+    }
+    if (together) {
+      do entry(std::true_type());
+      while (__any_sync(kFull, walk.cur != 0u));
+    } else {
+      do entry(std::false_type());
+      while (can ? !__any_sync(kFull, walk.cur == 0u) : walk.any_up_to(lim));
+    }
   }
   cp_wait_all();
 }
@@ -874,10 +963,31 @@ __global__ void __launch_bounds__(kThreads, kBwdCtas) raster_bwd_kernel(const __
   const int warp = threadIdx.x >> 5;
   init_warp_smem(s_w[warp]);
   const uint32_t n_jobs = JOBS * a.n_tiles;
-  uint32_t job = blockIdx.x * (kThreads / 32) + warp;
-  while (work ? next_job(work, n_jobs, job) : job < n_jobs) {
+  uint32_t job;
+  while (next_job(work, n_jobs, job)) {
     bwd_job<TW, TH, PPL>(a, rp, job / JOBS, (int)(job % JOBS), s_w[warp], T_final_all, last_all, g2d);
-    if (!work) break;
+  }
+}
+
+// Marks the tiles whose list is cut and holds a pixel that did not stop (one
+// CTA of 256 threads per tile).
+__global__ void __launch_bounds__(256) raster_open_kernel(const __grid_constant__ RasterArgs a,
+                                                          const int32_t* __restrict__ last_all,
+                                                          const uint8_t* __restrict__ cut, uint8_t* __restrict__ level,
+                                                          unsigned long long* __restrict__ open) {
+  const uint32_t tile = blockIdx.x;
+  if (!cut[tile]) return;
+  int v = 0;
+  for (int k = 1; k < a.views; ++k)
+    if (tile >= a.v[k].tile_base) v = k;
+  const int lt = (int)(tile - a.v[v].tile_base);
+  const int px = lt % a.v[v].tiles_x * a.tile_w + (int)threadIdx.x % a.tile_w;
+  const int py = lt / a.v[v].tiles_x * a.tile_h + (int)threadIdx.x / a.tile_w;
+  const bool in = px < a.v[v].width && py < a.v[v].height;
+  const bool mine = in && (last_all[a.v[v].pix_base + (size_t)py * a.v[v].width + px] & kOpen);
+  if (__syncthreads_or(mine) && threadIdx.x == 0) {
+    level[tile] += 1;
+    atomicOr(open, 1ull);
   }
 }
 
@@ -927,7 +1037,7 @@ void fwd_launch(const RasterArgs& a, const RasterParams& rp, float* T_final, int
   static int per_sm = 0;
   const int nc = job_ctas(a.n_tiles, PPL);
   auto* k = raster_fwd_kernel<TW, TH, PPL, COUNT, LOSS>;
-  launch_pdl(k, a.work ? persistent_grid(k, per_sm, nc, a.num_sms) : nc, kThreads, 0, s, a, rp, T_final, last, counters,
+  launch_pdl(k, a.persistent ? persistent_grid(k, per_sm, nc, a.num_sms) : nc, kThreads, 0, s, a, rp, T_final, last, counters,
              a.work);
 }
 
@@ -955,7 +1065,7 @@ void bwd_launch(const RasterArgs& a, const RasterParams& rp, const float* T_fina
   static int per_sm = 0;
   const int nc = job_ctas(a.n_tiles, PPL);
   auto* k = raster_bwd_kernel<TW, TH, PPL>;
-  launch_pdl(k, a.work ? persistent_grid(k, per_sm, nc, a.num_sms) : nc, kThreads, 0, s, a, rp, T_final, last, g2d,
+  launch_pdl(k, a.persistent ? persistent_grid(k, per_sm, nc, a.num_sms) : nc, kThreads, 0, s, a, rp, T_final, last, g2d,
              a.work);
 }
 
@@ -987,7 +1097,7 @@ void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsig
                        cudaStream_t s) {
   if (a.n_tiles == 0) return;
   const RasterParams rp = make_params(a);
-  if (a.work && a.zero_work) cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
+  if (a.zero_work) cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
   const bool loss = a.loss_partials != nullptr;
   if (counters) {
     if (loss) fwd_shapes<true, true>(a, rp, T_final, last, counters, s);
@@ -998,10 +1108,15 @@ void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsig
   }
 }
 
+void launch_raster_open(const RasterArgs& a, const int32_t* last, const uint8_t* cut, uint8_t* level,
+                        unsigned long long* open, cudaStream_t s) {
+  if (a.n_tiles) raster_open_kernel<<<a.n_tiles, 256, 0, s>>>(a, last, cut, level, open);
+}
+
 void launch_raster_bwd(const RasterArgs& a, const float* T_final, const int32_t* last, float4* g2d, cudaStream_t s) {
   if (a.n_tiles == 0) return;
   const RasterParams rp = make_params(a);
-  if (a.work && a.zero_work) cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
+  if (a.zero_work) cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s);
   if (a.tile_w == 16) bwd_shape<16, 16>(a, rp, T_final, last, (float*)g2d, s);
   else if (a.tile_w == 8) bwd_shape<8, 32>(a, rp, T_final, last, (float*)g2d, s);
   else bwd_shape<32, 8>(a, rp, T_final, last, (float*)g2d, s);

@@ -130,6 +130,15 @@ __global__ void __launch_bounds__(kBinThreads) tile_count_kernel(const __grid_co
                        });
 }
 
+// Difference grids of the huge rectangles (TileBinArgs::big_diff).
+struct BigGrids {
+  int* diff;
+  const uint32_t* big_len;
+  int views;
+  int tiles_x[kMaxViews], tiles_y[kMaxViews];
+  uint32_t base[kMaxViews], tile_base[kMaxViews];
+};
+
 // Length class of a tile list for the visit order, four per octave: 0 for
 // an empty list, else 4 floor(log2 c) + (the two bits after c's leading one)
 // + 1, so classes grow with the length and tiles within 19% of each other's
@@ -142,18 +151,45 @@ __device__ __forceinline__ int length_class(uint32_t c) {
   return 4 * lead + frac + 1;
 }
 
+// Adds view v's huge rectangles to the tile counts and leaves its difference
+// grid zero (every thread of the block calls it).
+template <int THREADS>
+__device__ __forceinline__ void add_big_rects(const BigGrids& b, int v, uint32_t* __restrict__ counts) {
+  const int TX = b.tiles_x[v], TY = b.tiles_y[v];
+  int* g = b.diff + b.base[v];
+  integrate_grid<THREADS>(g, TX, TY, [&](int t, int* cell, int n) {
+    if (n) counts[b.tile_base[v] + t] += (uint32_t)n;
+    *cell = 0;
+  });
+  for (int x = threadIdx.x; x <= TX; x += THREADS) g[(size_t)TY * (TX + 1) + x] = 0;
+  for (int y = threadIdx.x; y < TY; y += THREADS) g[(size_t)y * (TX + 1) + TX] = 0;
+}
+
+// one block per view; nothing to do without huge rectangles
+__global__ void __launch_bounds__(kScanThreads) big_rects_kernel(const __grid_constant__ BigGrids b,
+                                                                 uint32_t* __restrict__ counts) {
+  pdl_enter();
+  if (b.big_len[kHugeFlag] == 0u) return;
+  add_big_rects<kScanThreads>(b, blockIdx.x, counts);
+}
+
 // offsets = exclusive scan of counts (clamped to 32 bits), cursors = offsets;
 // stats[0] = total pairs, stats[1] = longest list; n_pairs = min(total, capacity).
 // order (if non-null) = the tiles by descending length class, the order in
 // which the raster passes visit them (longest lists first, so that the
 // slowest tiles do not start last).
-__global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(int T, const uint32_t* __restrict__ counts,
+__global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(int T, uint32_t* counts,
                                                                  uint32_t* __restrict__ offsets,
                                                                  uint32_t* __restrict__ cursors, uint32_t capacity,
                                                                  uint32_t* __restrict__ n_pairs,
                                                                  unsigned long long* __restrict__ stats,
-                                                                 uint32_t* __restrict__ order) {
+                                                                 uint32_t* __restrict__ order,
+                                                                 const __grid_constant__ BigGrids big) {
   pdl_enter();
+  if (big.diff && big.big_len[kHugeFlag]) {
+    for (int v = 0; v < big.views; ++v) add_big_rects<kScanThreads>(big, v, counts);
+    __syncthreads();
+  }
   __shared__ unsigned long long s[kScanThreads];
   __shared__ uint32_t s_max[32];
   const int per = (T + kScanThreads - 1) / kScanThreads;
@@ -471,7 +507,7 @@ __global__ void __launch_bounds__(kSortThreads) tile_sort_kernel(const uint32_t*
                                                                  uint32_t n_items, uint32_t bucket_cap,
                                                                  uint32_t* __restrict__ cls_count,
                                                                  uint32_t* __restrict__ cls_tiles,
-                                                                 uint32_t cls_stride) {
+                                                                 uint32_t cls_stride, bool long_sorted) {
   pdl_enter();
   const bool buckets = cls_count != nullptr;  // the lists are per-tile buckets (see TileBinArgs)
   __shared__ unsigned long long s[CAP];
@@ -482,6 +518,7 @@ __global__ void __launch_bounds__(kSortThreads) tile_sort_kernel(const uint32_t*
     s_nlong = 0u;
     if (blockIdx.x == 0) {
       *big_len = 0u;
+      big_len[kHugeFlag] = 0u;
       if (raster_work) raster_work[0] = raster_work[1] = 0u;  // the raster passes' job counters
     }
   }
@@ -501,8 +538,8 @@ __global__ void __launch_bounds__(kSortThreads) tile_sort_kernel(const uint32_t*
       }
       uint2 rg = (n && fits) ? make_uint2(off, off + n) : make_uint2(0u, 0u);
       if (fits && n > (uint32_t)CAP) {
-        atomicOr(overflow, 2u);
-        rg = make_uint2(0u, 0u);
+        if (!long_sorted) atomicOr(overflow, 2u);
+        if (!long_sorted) rg = make_uint2(0u, 0u);
       } else if (fits && n > (uint32_t)kWarpSortMax) {
         s_long[atomicAdd(&s_nlong, 1u)] = make_uint2(off, n);
       }
@@ -568,11 +605,25 @@ void launch_tile_count_scan(const TileBinArgs& a, cudaStream_t s, int64_t* launc
       if (launches) *launches += 1;
     }
   }
+  BigGrids big{};
+  big.diff = a.big_diff;
+  big.big_len = a.big_len;
+  big.views = a.map.views;
+  for (int v = 0; v < a.map.views; ++v) {
+    big.tiles_x[v] = a.map.tiles_x[v];
+    big.tiles_y[v] = a.tiles_y[v];
+    big.base[v] = a.big_base[v];
+    big.tile_base[v] = a.map.tile_base[v];
+  }
   if (a.n_tiles <= 4 * kScanThreads || !a.scan_aux) {  // one block is enough
     launch_pdl(tile_scan_kernel, 1, kScanThreads, 0, s, a.n_tiles, a.counts, a.offsets, a.cursors, a.capacity,
-               a.n_pairs, a.stats, a.order);
+               a.n_pairs, a.stats, a.order, big);
     if (launches) *launches += 1;
   } else {
+    if (a.big_diff) {
+      launch_pdl(big_rects_kernel, a.map.views, kScanThreads, 0, s, big, a.counts);
+      if (launches) *launches += 1;
+    }
     const int nb = (a.n_tiles + kScanTiles - 1) / kScanTiles;
     uint32_t* tail = a.scan_aux + (size_t)kScanAux * nb;
     launch_pdl(tile_scan_up_kernel, nb, 256, 0, s, a.n_tiles, a.counts, a.scan_aux);
@@ -597,7 +648,7 @@ void launch_tile_sort(const TileBinArgs& a, cudaStream_t s, int64_t* launches) {
              buckets ? a.bucket_ids : a.ids, a.zkey, a.ranges, (uint32_t)a.n_tiles, a.capacity, a.overflow,
              const_cast<uint32_t*>(a.big_len), a.raster_work, (uint32_t)a.n, a.bucket_cap,
              buckets ? a.cls_count : nullptr,
-             a.cls_tiles, a.cls_stride);
+             a.cls_tiles, a.cls_stride, a.long_sorted);
   if (launches) *launches += 1;
 }
 
