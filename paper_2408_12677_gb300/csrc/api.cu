@@ -55,11 +55,12 @@ struct gs_ctx {
   uint32_t* toffset = nullptr;  // per-tile list offsets
   uint32_t* tcursor = nullptr;  // per-tile scatter cursors
   uint32_t* torder = nullptr;   // raster visit order of the tiles (longest lists first)
+  uint2* tlong = nullptr;       // lists for the per-tile sort's second kernel
   uint32_t* scan_aux = nullptr;  // multi-block tile scan scratch
   uint32_t* bigq = nullptr;     // ids of Gaussians covering more than kBigTiles tiles
   uint32_t* d_bigmeta = nullptr;  // [0] length of the large-splat queue, [1] / [2] forward / backward raster
                                   // job counters, [3] ticket of the fused-loss reduction (0 between launches),
-                                  // [kHugeFlag] the difference grids are in use
+                                  // [kHugeFlag] the difference grids are in use, [kLongLen] length of tlong
   bool counts_zero = false;       // the tile counters and the large-splat queue length are 0 (the per-tile
                                   // sort, the last binning kernel, zeroes them)
   bool fwd_work_zero = false;     // the forward / backward raster job counters are 0 (the per-tile sort zeroes
@@ -315,6 +316,7 @@ gs_status ensure_tiles(gs_ctx* c, int64_t t) {
   GS_GROW(c, cap_t, regrow(&c->toffset, cap));
   GS_GROW(c, cap_t, regrow(&c->tcursor, cap));
   GS_GROW(c, cap_t, regrow(&c->torder, cap));
+  GS_GROW(c, cap_t, regrow(&c->tlong, cap));
   GS_GROW(c, cap_t, regrow(&c->scan_aux, tile_scan_aux_size(cap)));
   GS_GROW(c, cap_t, regrow(&c->tile_loss, 3 * kMaxTileJobs * cap));
   c->cap_t = cap;
@@ -556,12 +558,15 @@ gs_status bin_buckets(gs_ctx* c, int n, const TileMap& map, cudaStream_t s) {
   tb.overflow = c->d_overflow;
   tb.big_queue = c->bigq;
   tb.big_len = c->d_bigmeta;
+  tb.long_list = c->tlong;
+  tb.long_len = c->d_bigmeta + kLongLen;
   tb.order = nullptr;
   tb.counted = true;
   tb.scan_aux = nullptr;
   tb.raster_work = c->d_bigmeta + 1;
   tb.bucket_ids = c->bids;
   tb.bucket_cap = c->bucket_cap;
+  tb.longest = c->bucket_cap;
   tb.cls_count = c->cls_count;
   tb.cls_tiles = c->cls_tiles;
   tb.cls_stride = (uint32_t)c->cap_bt;
@@ -644,6 +649,8 @@ gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, c
   tb.overflow = c->d_overflow;
   tb.big_queue = c->bigq;
   tb.big_len = c->d_bigmeta;
+  tb.long_list = c->tlong;
+  tb.long_len = c->d_bigmeta + kLongLen;
   tb.order = c->order_tiles ? c->torder : nullptr;
   tb.counted = true;
   tb.scan_aux = c->scan_aux;
@@ -670,6 +677,7 @@ gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, c
   tb.capacity = (uint32_t)std::min<int64_t>(c->cap_p, 0xFFFFFFF0ll);
   tb.raster_work = c->d_bigmeta + 1;
   tb.long_sorted = true;
+  GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta + kLongLen, 0, sizeof(uint32_t), s));
   {
     StageTimer t(c, GS_STAGE_DUPLICATE, s);
     launch_prefix_scatter(a, max_lim, c->pfx_cur, c->pv[0], tb.capacity, s, &c->launches);
@@ -719,6 +727,8 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
   tb.overflow = c->d_overflow;
   tb.big_queue = c->bigq;
   tb.big_len = c->d_bigmeta;
+  tb.long_list = c->tlong;
+  tb.long_len = c->d_bigmeta + kLongLen;
   tb.order = c->order_tiles ? c->torder : nullptr;
   tb.counted = counted;
   tb.scan_aux = c->scan_aux;
@@ -743,6 +753,7 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
     // has seen fits half of one; a bucket holds twice the longest of them,
     // rounded up to a power of two (at least kBucketCapMin)
     c->longest_seen = std::max(c->longest_seen, longest);
+    tb.longest = (uint32_t)std::min<int64_t>(longest, 0xFFFFFFFFll);
     int64_t entries = kBucketCapMin;
     while (entries < 2 * c->longest_seen && entries < (int64_t)kBucketCapMax) entries *= 2;
     c->bucket_ok = c->longest_seen <= entries / 2 && T * entries < ((int64_t)1 << 32) &&
@@ -833,8 +844,8 @@ gs_status gs_ctx_create(gs_ctx** out, int device, int64_t pair_capacity) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_dscale, kMaxViews * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_nvalid, kMaxViews * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(c->d_nvalid, 0, kMaxViews * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_bigmeta, 5 * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(c->d_bigmeta, 0, 5 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_bigmeta, 6 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMemset(c->d_bigmeta, 0, 6 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(c->d_step, 0, sizeof(long long));
   if (e == cudaSuccess) init_project_kernels();
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_evals, 4 * sizeof(unsigned long long));
@@ -880,6 +891,7 @@ gs_status gs_ctx_destroy(gs_ctx* c) {
   cudaFree(c->toffset);
   cudaFree(c->tcursor);
   cudaFree(c->torder);
+  cudaFree(c->tlong);
   cudaFree(c->scan_aux);
   cudaFree(c->bigq);
   cudaFree(c->d_bigmeta);
@@ -1257,6 +1269,7 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
     launch_project_fwd(pa, c->feat, c->zkey, c->tiles, c->rects, s);
   }
   if (g->n > 0) c->launches += 1;
+  else GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta + kLongLen, 0, sizeof(uint32_t), s));  // (the projection zeroes it)
   GS_CHECK_LAUNCH(c, "project_fwd");
 
   if (c->counting)  // (a pass over cut lists may be repeated)
@@ -2120,6 +2133,7 @@ gs_status gs_bin_tiles(gs_ctx* c, int64_t n, const float* mean2d, const float* e
   }
   c->have_state = false;
   GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta, 0, sizeof(uint32_t), s));
+  GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta + kLongLen, 0, sizeof(uint32_t), s));
   // the count kernel zeroes the T counters it uses; the others stay as they were
   const bool counters_were_zero = c->counts_zero;
   c->counts_zero = false;

@@ -33,6 +33,7 @@ struct TileMap {
 // running long).
 constexpr uint32_t kBigTiles = 32;
 constexpr int kHugeFlag = 4;
+constexpr int kLongLen = 5;
 
 // Gaussians covering more than this many tiles are counted by four corners of
 // a difference grid instead of tile by tile.  Integrating the grid takes the
@@ -42,6 +43,7 @@ constexpr uint32_t kHugeTiles = 1024;
 struct ProjectArgs {
   uint32_t* big_queue;  // items with more than kBigTiles tiles
   uint32_t* big_len;    // queue length (zeroed before the launch); big_len[kHugeFlag] != 0: the grids are in use
+                        // (set by the projection); big_len[kLongLen]: long lists (zeroed by it)
   int n;                // Gaussians
   int views;
   const float *means, *log_scales, *quats, *logits, *sh;
@@ -223,6 +225,9 @@ struct TileBinArgs {
   uint32_t* order;            // per tile (output, nullable): visit order, longest lists first
   bool counted;               // counts already hold every item's tiles (the projection counted them)
   uint32_t* scan_aux;         // scratch of tile_scan_aux_size(n_tiles) words for the multi-block scan
+  uint2* long_list = nullptr;    // per tile: lists for the sort's second kernel, *long_len of them (0 before)
+  uint32_t* long_len = nullptr;
+  uint32_t longest = 0xFFFFFFFFu;  // no list that is sorted is longer than this (as far as the host knows)
   bool long_sorted = false;   // lists longer than the per-tile sort holds are in order already (left as they are)
   int* big_diff = nullptr;    // nullable: difference grids of the large rectangles, added to the counts (and
                               // zeroed) by the scan when there are any (see ProjectArgs)

@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(kFwdThreads) project_fwd_kernel(const __grid_c
     if (a.nvalid && threadIdx.x < (unsigned)a.views) a.nvalid[threadIdx.x] = 0u;
     if (a.cls_count)
       for (int c = threadIdx.x; c < kLenClasses; c += kFwdThreads) a.cls_count[c] = 0u;
+    if (a.big_len && threadIdx.x == 0) a.big_len[kLongLen] = 0u;
     if (a.step_inc && threadIdx.x == 0) *a.step_inc += 1;
   }
   // the block's slices of every parameter array are contiguous: stage them

@@ -6,13 +6,15 @@
 //               total pair count and the longest list),
 //   3. scatter: every pair takes a slot of its tile's list with an atomic
 //               cursor and writes its Gaussian id,
-//   4. sort:    each tile's list is sorted by the 64-bit key (float32 depth
-//               bits << 32 | id) with a bitonic network: by one warp in
-//               registers up to 512 entries, by a CTA in shared memory beyond.
+//   4. sort:    each tile's list is sorted by (float32 depth bits, id) with a
+//               bitonic network: by one warp in registers up to 1024 entries,
+//               by a CTA beyond.
 // The per-tile keys are unique, so the result is exactly the (tile, depth, id)
 // order of a stable sort and does not depend on the scatter's atomic order.
 // Counting and scattering expand the rectangles warp-cooperatively, so a
 // Gaussian covering thousands of tiles is spread over the whole warp.
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -25,7 +27,8 @@ constexpr int kBinWarps = kBinThreads / 32;
 constexpr int kScanThreads = 1024;
 constexpr int kSortThreads = 128;
 constexpr int kSortWarps = kSortThreads / 32;  // tiles per CTA of the per-tile sort
-constexpr int kWarpSortMax = 512;              // lists up to this length are sorted by one warp
+constexpr int kWarpSortMax = 1024;             // lists up to this length are sorted by one warp (32-bit keys)
+constexpr int kWarpSort64 = 512;               // ... by their 64-bit keys
 
 // Global tile of tile (tx, ty) of the view that item `it` belongs to.
 struct ItemTiles {
@@ -486,19 +489,359 @@ __device__ __forceinline__ void warp_sort_list(uint32_t* __restrict__ ids, const
   }
 }
 
-// Per-tile sort of the lists by the 64-bit key (depth bits << 32 | id).  A
-// CTA takes kSortWarps consecutive tiles, one warp each: lists of up to
-// kWarpSortMax entries are sorted by that warp in registers (warp_bitonic,
-// no barriers); longer ones (up to CAP) are queued in the CTA and then
-// sorted one after the other by the whole CTA with a bitonic network in
-// shared memory.  The last binning kernel: it also zeroes each tile's counter
-// (and block 0 the large-splat queue length, and the two raster job counters
-// when given), leaving them zero for the next passes.  In bucket mode each
-// warp also files its tile under its length class (see TileBinArgs).
-template <int CAP>
-__global__ void __launch_bounds__(kSortThreads) tile_sort_kernel(const uint32_t* __restrict__ offsets,
-                                                                 uint32_t* __restrict__ counts,
-                                                                 uint32_t* __restrict__ ids,
+// ---------------------------------------------------------------------------
+// The usual sort of a list: 32-bit keys (depth rounded down) << B | place in the
+// unsorted list, B bits for n places and the depth in what remains of the bits,
+// offset by the list's smallest: a compare-exchange is a minimum and a maximum
+// instead of a 64-bit compare and four selects, and half the shuffles.  Entries
+// whose rounded depths are equal come out in the order of their places.  Equal
+// depths are common (a level camera sees a horizontal plane at one depth per
+// pixel row), so a list that has any is sorted a second time, by (run of equal
+// rounded depths, the depth's bits that were rounded off, id); where these do
+// not fit into 32 bits, by the 64-bit keys.
+//
+// The networks' merges start by comparing mirrored places (e with e ^ (k - 1)),
+// so every compare-exchange puts the smaller key at the smaller place.  Blocked
+// layout as in warp_bitonic.
+// ---------------------------------------------------------------------------
+template <int KEYS>
+__device__ __forceinline__ void lane_merge(uint32_t (&x)[KEYS]) {  // partner distances KEYS / 2 .. 1
+#pragma unroll
+  for (int j = KEYS / 2; j > 0; j >>= 1)
+#pragma unroll
+    for (int i = 0; i < KEYS; ++i)
+      if ((i & j) == 0) {
+        const uint32_t a = x[i], b = x[i | j];
+        x[i] = min(a, b);
+        x[i | j] = max(a, b);
+      }
+}
+
+template <int KEYS>
+__device__ __forceinline__ void lane_sort(uint32_t (&x)[KEYS]) {
+#pragma unroll
+  for (int k = 2; k <= KEYS; k <<= 1) {
+#pragma unroll
+    for (int i = 0; i < KEYS; ++i)
+      if ((i & (k >> 1)) == 0) {
+        const int p = i ^ (k - 1);
+        const uint32_t a = x[i], b = x[p];
+        x[i] = min(a, b);
+        x[p] = max(a, b);
+      }
+#pragma unroll
+    for (int j = k >> 2; j > 0; j >>= 1)
+#pragma unroll
+      for (int i = 0; i < KEYS; ++i)
+        if ((i & j) == 0) {
+          const uint32_t a = x[i], b = x[i | j];
+          x[i] = min(a, b);
+          x[i | j] = max(a, b);
+        }
+  }
+}
+
+// distances of d lanes down to one lane, then within the lane
+template <int KEYS>
+__device__ __forceinline__ void warp_merge_from(uint32_t (&x)[KEYS], int lane, int d) {
+  for (; d > 0; d >>= 1) {
+    const bool lower = (lane & d) == 0;
+#pragma unroll
+    for (int i = 0; i < KEYS; ++i) {
+      const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x[i], d);
+      x[i] = lower ? min(x[i], y) : max(x[i], y);
+    }
+  }
+  lane_merge(x);
+}
+
+// Sorts the first n of the warp's 32 KEYS keys (the others are all ones).
+template <int KEYS>
+__device__ __forceinline__ void warp_sort32(uint32_t (&x)[KEYS], int lane, uint32_t n) {
+  lane_sort(x);
+  for (int m = 1; m < 32 && (uint32_t)(KEYS * (m + 1) / 2) < n; m = 2 * m + 1) {
+    const bool lower = (lane & ((m + 1) >> 1)) == 0;
+#pragma unroll
+    for (int i = 0; i < KEYS / 2; ++i) {
+      const uint32_t a = __shfl_xor_sync(0xFFFFFFFFu, x[KEYS - 1 - i], m);
+      const uint32_t b = __shfl_xor_sync(0xFFFFFFFFu, x[i], m);
+      x[i] = lower ? min(x[i], a) : max(x[i], a);
+      x[KEYS - 1 - i] = lower ? min(x[KEYS - 1 - i], b) : max(x[KEYS - 1 - i], b);
+    }
+    warp_merge_from(x, lane, (m + 1) >> 2);
+  }
+}
+
+// How a list's depths become keys.
+struct KeyMap {
+  uint32_t zmin;
+  int shift, bits;  // (z - zmin) >> shift, then << bits
+  __device__ __forceinline__ uint32_t rounded(uint32_t z) const { return (z - zmin) >> shift; }
+  __device__ __forceinline__ uint32_t place(uint32_t key) const { return key & ((1u << bits) - 1u); }
+  __device__ __forceinline__ bool tie(uint32_t a, uint32_t b) const { return ((a ^ b) >> bits) == 0u; }
+};
+__device__ __forceinline__ KeyMap key_map(uint32_t n, uint32_t zmin, uint32_t zmax) {
+  KeyMap k;
+  k.zmin = zmin;
+  k.bits = n > 1 ? 32 - __clz(n - 1) : 1;
+  const int need = 32 - __clz(zmax - zmin);  // (__clz(0) = 32)
+  k.shift = max(0, need - (32 - k.bits));
+  return k;
+}
+
+// The places' entries: ids[off + place], and whether an entry's rounded depth
+// equals that of the one before it (bit i: entry e0 + i); prev: the key before
+// the lane's first one.
+template <int KEYS>
+__device__ __forceinline__ uint32_t sorted_ids_ties(const uint32_t (&x)[KEYS], const uint32_t* ids, uint32_t off,
+                                                    uint32_t n, uint32_t e0, const KeyMap& k, uint32_t prev,
+                                                    uint32_t (&id)[KEYS]) {
+  uint32_t ties = 0u;
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) {
+    const uint32_t e = e0 + i;
+    id[i] = e < n ? ids[off + k.place(x[i])] : 0u;
+    if (e > 0 && e < n && k.tie(x[i], i ? x[(i + KEYS - 1) % KEYS] : prev)) ties |= 1u << i;
+  }
+  return ties;
+}
+
+// Second keys of the entries: runs counted from `run` on; false when they do
+// not fit.
+struct IdMap {
+  uint32_t imin;
+  int bits;
+};
+template <int KEYS>
+__device__ __forceinline__ void run_keys(uint32_t (&id)[KEYS], const uint32_t* __restrict__ zkey, uint32_t n, uint32_t e0,
+                                         uint32_t ties, uint32_t run, const KeyMap& k, const IdMap& m, uint32_t n_items) {
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) {
+    if (!(ties >> i & 1u)) ++run;
+    uint32_t key = (run - 1u) << k.shift;
+    if (k.shift && e0 + i < n && in_bounds(id[i] < n_items)) key |= (zkey[id[i]] - k.zmin) & ((1u << k.shift) - 1u);
+    id[i] = e0 + i < n ? (key << m.bits) | (id[i] - m.imin) : 0xFFFFFFFFu;
+  }
+}
+
+// One warp sorts the list of n <= 32 KEYS ids at ids[off ..]; true: it has to
+// be sorted by its 64-bit keys (and is as it was).
+template <int KEYS>
+__device__ __forceinline__ bool warp_sort_list32(uint32_t* ids, const uint32_t* __restrict__ zkey, uint32_t off,
+                                                 uint32_t n, uint32_t n_items, int lane) {
+  // up to 256 entries, consecutive ones per lane, so that short lists fill the
+  // lower lanes only and need fewer merges
+  auto place = [lane](int i) { return (uint32_t)(KEYS == 8 ? KEYS * lane + i : 32 * i + lane); };
+  uint32_t x[KEYS];
+  uint32_t zmin = 0xFFFFFFFFu, zmax = 0u, imin = 0xFFFFFFFFu, imax = 0u;
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) {
+    const uint32_t e = place(i);
+    x[i] = 0u;
+    if (e < n) {
+      const uint32_t g = ids[off + e];
+      x[i] = in_bounds(g < n_items) ? zkey[g] : 0xFFFFFFFFu;
+      zmin = min(zmin, x[i]);
+      zmax = max(zmax, x[i]);
+      imin = min(imin, g);
+      imax = max(imax, g);
+    }
+  }
+  const KeyMap k = key_map(n, __reduce_min_sync(0xFFFFFFFFu, zmin), __reduce_max_sync(0xFFFFFFFFu, zmax));
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) {
+    const uint32_t e = place(i);
+    x[i] = e < n ? (k.rounded(x[i]) << k.bits) | e : 0xFFFFFFFFu;
+  }
+  warp_sort32<KEYS>(x, lane, n);
+  const uint32_t e0 = (uint32_t)(lane * KEYS);
+  uint32_t id[KEYS];
+  const uint32_t ties = sorted_ids_ties<KEYS>(x, ids, off, n, e0, k, __shfl_up_sync(0xFFFFFFFFu, x[KEYS - 1], 1), id);
+  uint32_t add = 0u, mask = 0xFFFFFFFFu;
+  if (__any_sync(0xFFFFFFFFu, ties != 0u)) {
+    IdMap m;
+    m.imin = __reduce_min_sync(0xFFFFFFFFu, imin);
+    m.bits = 32 - __clz(__reduce_max_sync(0xFFFFFFFFu, imax) - m.imin);
+    if (k.bits + k.shift + m.bits > 32) return true;
+    const uint32_t runs = (uint32_t)(KEYS - __popc(ties));
+    uint32_t incl = runs;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+      if (lane >= d) incl += y;
+    }
+    run_keys<KEYS>(id, zkey, n, e0, ties, incl - runs, k, m, n_items);
+    warp_sort32<KEYS>(id, lane, n);
+    add = m.imin;
+    mask = m.bits == 32 ? 0xFFFFFFFFu : (1u << m.bits) - 1u;
+  }
+  __syncwarp();  // every place has been read
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i)
+    if (e0 + i < n) ids[off + e0 + i] = add + (id[i] & mask);
+  return false;
+}
+
+// A CTA of kLongWarps warps sorts its 256 keys per warp: each warp its own, then
+// levels of merges whose first exchanges go through shared memory (s: a word
+// per key), as many as n keys need.
+constexpr int kLongKeys = 8, kLongWarps = kTileSortCap / (32 * kLongKeys), kLongThreads = 32 * kLongWarps;
+__device__ __forceinline__ void cta_sort32(uint32_t (&x)[kLongKeys], int lane, int warp, uint32_t n, uint32_t* s) {
+  constexpr int KEYS = kLongKeys, W = 32 * KEYS;
+  warp_sort32<KEYS>(x, lane, W);
+  // exchange with warp ^ m: mirrored places (flip) or equal ones; word i of the
+  // warp's lane l at s[W warp + 32 i + l], so neither side conflicts
+  auto exchange = [&](int m, int high, bool flip) {
+#pragma unroll
+    for (int i = 0; i < KEYS; ++i) s[W * warp + 32 * i + lane] = x[i];
+    __syncthreads();
+    const bool lower = (warp & high) == 0;
+    const uint32_t* o = s + W * (warp ^ m) + (flip ? 31 - lane : lane);
+#pragma unroll
+    for (int i = 0; i < KEYS; ++i) {
+      const uint32_t y = o[32 * (flip ? KEYS - 1 - i : i)];
+      x[i] = lower ? min(x[i], y) : max(x[i], y);
+    }
+    __syncthreads();
+  };
+  for (int m = 1; m < kLongWarps && (uint32_t)(W * (m + 1) / 2) < n; m = 2 * m + 1) {
+    exchange(m, (m + 1) >> 1, true);
+    for (int d = (m + 1) >> 2; d > 0; d >>= 1) exchange(d, d, false);
+    warp_merge_from(x, lane, 16);
+  }
+}
+
+// The CTA sorts a list of at most kTileSortCap ids; true as for warp_sort_list32.
+__device__ __forceinline__ bool cta_sort_list32(uint32_t* ids, const uint32_t* __restrict__ zkey, uint32_t off,
+                                                uint32_t n, uint32_t n_items, uint32_t* s) {
+  constexpr int KEYS = kLongKeys, W = 32 * KEYS;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t e0 = (uint32_t)(W * warp + lane * KEYS);
+  uint32_t x[KEYS];
+  uint32_t zmin = 0xFFFFFFFFu, zmax = 0u, imin = 0xFFFFFFFFu, imax = 0u;
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) {
+    x[i] = 0u;
+    if (e0 + i < n) {
+      const uint32_t g = ids[off + e0 + i];
+      x[i] = in_bounds(g < n_items) ? zkey[g] : 0xFFFFFFFFu;
+      zmin = min(zmin, x[i]);
+      zmax = max(zmax, x[i]);
+      imin = min(imin, g);
+      imax = max(imax, g);
+    }
+  }
+  zmin = __reduce_min_sync(0xFFFFFFFFu, zmin);
+  zmax = __reduce_max_sync(0xFFFFFFFFu, zmax);
+  imin = __reduce_min_sync(0xFFFFFFFFu, imin);
+  imax = __reduce_max_sync(0xFFFFFFFFu, imax);
+  if (lane == 0) {
+    s[4 * warp] = zmin;
+    s[4 * warp + 1] = zmax;
+    s[4 * warp + 2] = imin;
+    s[4 * warp + 3] = imax;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kLongWarps; ++w) {
+    zmin = min(zmin, s[4 * w]);
+    zmax = max(zmax, s[4 * w + 1]);
+    imin = min(imin, s[4 * w + 2]);
+    imax = max(imax, s[4 * w + 3]);
+  }
+  __syncthreads();
+  const KeyMap k = key_map(n, zmin, zmax);
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) x[i] = e0 + i < n ? (k.rounded(x[i]) << k.bits) | (e0 + i) : 0xFFFFFFFFu;
+  cta_sort32(x, lane, warp, n, s);
+  if (lane == 31) s[warp] = x[KEYS - 1];
+  __syncthreads();
+  uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, x[KEYS - 1], 1);
+  if (lane == 0 && warp > 0) prev = s[warp - 1];
+  uint32_t id[KEYS];
+  const uint32_t ties = sorted_ids_ties<KEYS>(x, ids, off, n, e0, k, prev, id);
+  uint32_t add = 0u, mask = 0xFFFFFFFFu;
+  if (__syncthreads_or(ties != 0u)) {  // (also: every place has been read)
+    IdMap m;
+    m.imin = imin;
+    m.bits = 32 - __clz(imax - imin);
+    if (k.bits + k.shift + m.bits > 32) return true;
+    const uint32_t runs = (uint32_t)(KEYS - __popc(ties));
+    uint32_t incl = runs;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+      if (lane >= d) incl += y;
+    }
+    if (lane == 31) s[kLongWarps + warp] = incl;
+    __syncthreads();
+    uint32_t run = incl - runs;
+    for (int w = 0; w < warp; ++w) run += s[kLongWarps + w];
+    __syncthreads();
+    run_keys<KEYS>(id, zkey, n, e0, ties, run, k, m, n_items);
+    cta_sort32(id, lane, warp, n, s);
+    add = m.imin;
+    mask = m.bits == 32 ? 0xFFFFFFFFu : (1u << m.bits) - 1u;
+  }
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i)
+    if (e0 + i < n) ids[off + e0 + i] = add + (id[i] & mask);
+  __syncthreads();  // s is reused by the next long list
+  return false;
+}
+
+// A CTA of THREADS threads sorts a list by its 64-bit keys in shared memory.
+template <int THREADS>
+__device__ __forceinline__ void cta_sort_list64(uint32_t* __restrict__ ids, const uint32_t* __restrict__ zkey,
+                                                uint32_t off, uint32_t n, uint32_t n_items,
+                                                unsigned long long* __restrict__ s) {
+  uint32_t m = 2;
+  while (m < n) m <<= 1;
+  for (uint32_t i = threadIdx.x; i < m; i += THREADS) {
+    unsigned long long key = ~0ull;
+    if (i < n) {
+      const uint32_t g = ids[off + i];
+      key = in_bounds(g < n_items) ? ((unsigned long long)zkey[g] << 32) | g : ~0ull;
+    }
+    s[i] = key;
+  }
+  __syncthreads();
+  for (uint32_t k = 2; k <= m; k <<= 1) {
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      for (uint32_t i = threadIdx.x; i < m; i += THREADS) {
+        const uint32_t ixj = i ^ j;
+        if (ixj > i) {
+          const unsigned long long a = s[i], b = s[ixj];
+          const bool up = (i & k) == 0;
+          if ((a > b) == up) {
+            s[i] = b;
+            s[ixj] = a;
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (uint32_t i = threadIdx.x; i < n; i += THREADS) ids[off + i] = (uint32_t)s[i];
+  __syncthreads();  // s is reused by the next long list
+}
+
+// Per-tile sort of the lists by (depth bits, id).  A CTA takes kSortWarps
+// consecutive tiles, one warp each: lists of up to kWarpSortMax entries are
+// sorted by that warp in registers (no barriers), the few of those whose 32-bit
+// keys do not suffice by the whole CTA; longer ones go to long_list, which
+// tile_sort_long_kernel sorts.  The kernel also zeroes each tile's counter (and
+// block 0 the large-splat queue length, and the two raster job counters),
+// leaving them zero for the next passes.  In bucket mode each warp also files
+// its tile under its length class (see TileBinArgs).
+//
+// Bound by latency (one wave of warps, each a chain of loads and exchanges).
+// 64-bit keys throughout, and long lists by the CTA that met them: 25.3 us for
+// 3225 lists of 207 entries (1200 x 680), 503 us for 16125 of 494, 167 us for
+// 8030 of 284, 941 us for 31360 of 398 (up to 4 lists of 4000 in one CTA); now
+// 21, 224, 52 and 435 us.
+__global__ void __launch_bounds__(kSortThreads, 6) tile_sort_kernel(const uint32_t* __restrict__ offsets,
+                                                                 uint32_t* __restrict__ counts, uint32_t* ids,
                                                                  const uint32_t* __restrict__ zkey,
                                                                  uint2* __restrict__ ranges, uint32_t n_tiles,
                                                                  uint32_t capacity, uint32_t* __restrict__ overflow,
@@ -507,19 +850,21 @@ __global__ void __launch_bounds__(kSortThreads) tile_sort_kernel(const uint32_t*
                                                                  uint32_t n_items, uint32_t bucket_cap,
                                                                  uint32_t* __restrict__ cls_count,
                                                                  uint32_t* __restrict__ cls_tiles,
-                                                                 uint32_t cls_stride, bool long_sorted) {
+                                                                 uint32_t cls_stride, bool long_sorted,
+                                                                 uint2* __restrict__ long_list,
+                                                                 uint32_t* __restrict__ long_len) {
   pdl_enter();
   const bool buckets = cls_count != nullptr;  // the lists are per-tile buckets (see TileBinArgs)
-  __shared__ unsigned long long s[CAP];
-  __shared__ uint2 s_long[kSortWarps];  // (offset, length) of the CTA's lists longer than kWarpSortMax
+  constexpr uint32_t CAP = kTileSortCap;
+  __shared__ unsigned long long s[kWarpSortMax];
+  __shared__ uint2 s_long[kSortWarps];  // (offset, length) of the CTA's lists that it sorts as a whole
   __shared__ uint32_t s_nlong;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     s_nlong = 0u;
     if (blockIdx.x == 0) {
       *big_len = 0u;
-      big_len[kHugeFlag] = 0u;
-      if (raster_work) raster_work[0] = raster_work[1] = 0u;  // the raster passes' job counters
+      raster_work[0] = raster_work[1] = 0u;  // the raster passes' job counters
     }
   }
   __syncthreads();
@@ -537,52 +882,43 @@ __global__ void __launch_bounds__(kSortThreads) tile_sort_kernel(const uint32_t*
         cls_tiles[(size_t)c * cls_stride + atomicAdd(&cls_count[c], 1u)] = t;
       }
       uint2 rg = (n && fits) ? make_uint2(off, off + n) : make_uint2(0u, 0u);
-      if (fits && n > (uint32_t)CAP) {
-        if (!long_sorted) atomicOr(overflow, 2u);
-        if (!long_sorted) rg = make_uint2(0u, 0u);
-      } else if (fits && n > (uint32_t)kWarpSortMax) {
-        s_long[atomicAdd(&s_nlong, 1u)] = make_uint2(off, n);
+      if (fits && n > CAP && !long_sorted) {
+        atomicOr(overflow, 2u);
+        rg = make_uint2(0u, 0u);
       }
       ranges[t] = rg;
+      if (fits && n > (uint32_t)kWarpSortMax && n <= CAP) long_list[atomicAdd(long_len, 1u)] = make_uint2(off, n);
     }
+    bool whole = false;
     if (fits && n > 1 && n <= (uint32_t)kWarpSortMax) {
+      if (n <= 256) whole = warp_sort_list32<8>(ids, zkey, off, n, n_items, lane);
+      else if (n <= 512) whole = warp_sort_list32<16>(ids, zkey, off, n, n_items, lane);
+      else whole = warp_sort_list32<32>(ids, zkey, off, n, n_items, lane);
+    }
+    if (whole && n <= (uint32_t)kWarpSort64) {
       if (n <= 256) warp_sort_list<8>(ids, zkey, off, n, n_items, lane);
       else warp_sort_list<16>(ids, zkey, off, n, n_items, lane);
+    } else if (whole && lane == 0) {
+      s_long[atomicAdd(&s_nlong, 1u)] = make_uint2(off, n);
     }
   }
   __syncthreads();
   const uint32_t n_long = s_nlong;
-  for (uint32_t q = 0; q < n_long; ++q) {
-    const uint32_t off = s_long[q].x, n = s_long[q].y;
-    uint32_t m = 2;
-    while (m < n) m <<= 1;
-    for (uint32_t i = threadIdx.x; i < m; i += kSortThreads) {
-      unsigned long long key = ~0ull;
-      if (i < n) {
-        const uint32_t g = ids[off + i];
-        key = in_bounds(g < n_items) ? ((unsigned long long)zkey[g] << 32) | g : ~0ull;
-      }
-      s[i] = key;
-    }
-    __syncthreads();
-    for (uint32_t k = 2; k <= m; k <<= 1) {
-      for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-        for (uint32_t i = threadIdx.x; i < m; i += kSortThreads) {
-          const uint32_t ixj = i ^ j;
-          if (ixj > i) {
-            const unsigned long long a = s[i], b = s[ixj];
-            const bool up = (i & k) == 0;
-            if ((a > b) == up) {
-              s[i] = b;
-              s[ixj] = a;
-            }
-          }
-        }
-        __syncthreads();
-      }
-    }
-    for (uint32_t i = threadIdx.x; i < n; i += kSortThreads) ids[off + i] = (uint32_t)s[i];
-    __syncthreads();  // s is reused by the next long list
+  for (uint32_t q = 0; q < n_long; ++q) cta_sort_list64<kSortThreads>(ids, zkey, s_long[q].x, s_long[q].y, n_items, s);
+}
+
+// The lists of more than kWarpSortMax entries, a CTA each.
+__global__ void __launch_bounds__(kLongThreads) tile_sort_long_kernel(uint32_t* ids, const uint32_t* __restrict__ zkey,
+                                                                      uint32_t n_items,
+                                                                      const uint2* __restrict__ long_list,
+                                                                      const uint32_t* __restrict__ long_len) {
+  pdl_enter();
+  __shared__ unsigned long long s[kTileSortCap];
+  const uint32_t count = *long_len;
+  for (uint32_t q = blockIdx.x; q < count; q += gridDim.x) {
+    const uint2 l = long_list[q];
+    if (cta_sort_list32(ids, zkey, l.x, l.y, n_items, reinterpret_cast<uint32_t*>(s)))
+      cta_sort_list64<kLongThreads>(ids, zkey, l.x, l.y, n_items, s);
   }
 }
 
@@ -644,12 +980,18 @@ void launch_tile_scatter(const TileBinArgs& a, cudaStream_t s, int64_t* launches
 void launch_tile_sort(const TileBinArgs& a, cudaStream_t s, int64_t* launches) {
   const int grid = (a.n_tiles + kSortWarps - 1) / kSortWarps;
   const bool buckets = a.bucket_ids != nullptr;
-  launch_pdl(tile_sort_kernel<kTileSortCap>, grid, kSortThreads, 0, s, a.offsets, a.counts,
+  launch_pdl(tile_sort_kernel, grid, kSortThreads, 0, s, a.offsets, a.counts,
              buckets ? a.bucket_ids : a.ids, a.zkey, a.ranges, (uint32_t)a.n_tiles, a.capacity, a.overflow,
              const_cast<uint32_t*>(a.big_len), a.raster_work, (uint32_t)a.n, a.bucket_cap,
              buckets ? a.cls_count : nullptr,
-             a.cls_tiles, a.cls_stride, a.long_sorted);
+             a.cls_tiles, a.cls_stride, a.long_sorted, a.long_list, a.long_len);
   if (launches) *launches += 1;
+  if (a.longest > (uint32_t)kWarpSortMax) {
+    launch_pdl(tile_sort_long_kernel, std::min(a.n_tiles, 3 * std::max(a.num_sms, 1)), kLongThreads, 0, s,
+               buckets ? a.bucket_ids : a.ids, a.zkey, (uint32_t)a.n, (const uint2*)a.long_list,
+               (const uint32_t*)a.long_len);
+    if (launches) *launches += 1;
+  }
 }
 
 cudaError_t tilebin_bind_bounds(uint32_t* word) { return bind_bounds_word(word); }
