@@ -1,7 +1,5 @@
 // Projection of 3D Gaussians to 2D splats (Eq. 2-5) and its backward pass,
 // including the gradient w.r.t. the camera pose.
-#include <type_traits>
-
 #include "common.cuh"
 #include "internal.h"
 
@@ -409,10 +407,10 @@ struct GaussGrad {
   float pose[6];
 };
 
-template <int D>
+template <int D, class SH>
 __device__ __forceinline__ void gaussian_grad(const CamView& cv, float dilation, const float (&p)[3],
                                               const float (&q4)[4], const float (&ls)[3], float logit,
-                                              const float* __restrict__ shp, float4 G0, float4 G1, float4 G2,
+                                              const SH& shp, float4 G0, float4 G1, float4 G2,
                                               GaussGrad<D>& out) {
   constexpr int K = (D + 1) * (D + 1);
   float pc[3];
@@ -636,7 +634,8 @@ __global__ void __launch_bounds__(kBwdThreads) project_bwd_kernel(const __grid_c
         zero_record(g2d + 3 * it);
         any = true;
         GaussGrad<D> gg;
-        gaussian_grad<D>(a.cv[v], a.dilation, p, q4, ls, logit, a.sh + (size_t)i * K * 3, G0, G1, G2, gg);
+        const float* row = a.sh + (size_t)i * K * 3;
+        gaussian_grad<D>(a.cv[v], a.dilation, p, q4, ls, logit, row, G0, G1, G2, gg);
         alog += gg.glogit;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -687,50 +686,32 @@ __device__ __forceinline__ void adam_update(float& p, float g, float& m, float& 
 }
 
 // Backward of the projection fused with the Adam step, for one optimisation
-// iteration on a batch of views.  A block (one warp) owns 32 consecutive
-// Gaussians:
+// iteration on one view.  A block (one warp) owns 32 consecutive Gaussians:
 //   1. its slices of the parameter array and of the two Adam moments (each
 //      slice contiguous in the flat layout) are copied to shared memory with
 //      cp.async, the parameters as a first group and the moments as a second,
 //      so the moment loads stay in flight during step 2;
-//   2. one thread per Gaussian turns its gradient records (one per view)
-//      into parameter gradients summed over the views, kept in shared memory;
+//   2. one thread per Gaussian turns its gradient record into parameter
+//      gradients, kept in shared memory, the SH gradient in factored form (Y_k *
+//      graw_c);
 //   3. coalesced sweeps apply Adam to every float and store p, m, v.
-// No gradient buffer is written or read.  With one view the SH gradient is
-// kept in factored form (Y_k * graw_c) and the SH moments are staged too;
-// with several views the SH gradients are summed in shared memory rows and
-// the SH moments are staged as well, beside the summed rows.  Blocks of one
-// warp (27 KB for one view, 8 blocks per SM) let the staging, gradient and
-// sweep phases of different blocks overlap.
-template <bool MULTI>
-constexpr int fused_threads() { return 32; }
-static_assert(fused_threads<false>() == 32 && fused_threads<true>() == 32,
-              "the fused loss reduction takes one warp per block");
+// No gradient buffer is written or read.  Blocks of one warp (27 KB, 8 blocks
+// per SM) let the staging, gradient and sweep phases of different blocks
+// overlap.
+constexpr int kFusedThreads = 32;
+static_assert(kFusedThreads == 32, "the fused loss reduction takes one warp per block");
 
 template <int D>
 struct FusedSmem {
   static constexpr int K = (D + 1) * (D + 1);
   static constexpr int NS = 3 * K;
   static constexpr int RS = (NS % 2 == 0) ? NS + 1 : NS;  // odd row stride: conflict-free per-thread rows
-  static constexpr int B = fused_threads<false>();
+  static constexpr int B = kFusedThreads;
   float p[B * 11], m[B * 11], v[B * 11];  // means (3B) | log-scales (3B) | quats (4B) | logits (B)
   float g[B * 11];                        // gradients, same layout
   float sp[B * RS], sm[B * NS + 4], sv[B * NS + 4];  // SH moments at their slice's offset within 16 B
   float Y[B][K + 1];
   float graw[B][4];
-};
-
-template <int D>
-struct FusedSmemMulti {
-  static constexpr int K = (D + 1) * (D + 1);
-  static constexpr int NS = 3 * K;
-  static constexpr int RS = (NS % 2 == 0) ? NS + 1 : NS;
-  static constexpr int B = fused_threads<true>();
-  float p[B * 11], m[B * 11], v[B * 11];
-  float g[B * 11];
-  float sp[B * RS];  // SH parameters, one row per Gaussian
-  float gs[B * RS];  // SH gradients summed over the views, same rows
-  float sm[B * NS + 4], sv[B * NS + 4];  // SH moments
 };
 
 // The training step's loss reduction (see LossFoldArgs), by one warp per
@@ -793,17 +774,17 @@ __device__ __forceinline__ void fused_loss_reduce(const LossFoldArgs& L) {
   }
 }
 
-template <int D, bool MULTI>
-__global__ void __launch_bounds__(fused_threads<MULTI>()) project_bwd_adam_kernel(const __grid_constant__ ProjectArgs a,
+template <int D>
+__global__ void __launch_bounds__(kFusedThreads) project_bwd_adam_kernel(const __grid_constant__ ProjectArgs a,
                                                                          float4* __restrict__ g2d,
                                                                          float* __restrict__ P, float* __restrict__ M,
                                                                          float* __restrict__ V, AdamArgs ad,
                                                                          float* __restrict__ pose_partials,
                                                                          const __grid_constant__ LossFoldArgs L) {
   pdl_enter();
-  if (L.out && threadIdx.x < 32) fused_loss_reduce(L);  // blocks of one warp: the whole block
+  if (L.out && threadIdx.x < 32) fused_loss_reduce(L);  // one warp's work  // blocks of one warp: the whole block
   device_bias_corrections(ad);
-  using S = typename std::conditional<MULTI, FusedSmemMulti<D>, FusedSmem<D>>::type;
+  using S = FusedSmem<D>;
   constexpr int K = S::K, NS = S::NS, RS = S::RS, B = S::B;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   S& sm = *reinterpret_cast<S*>(smem_raw);
@@ -858,51 +839,30 @@ __global__ void __launch_bounds__(fused_threads<MULTI>()) project_bwd_adam_kerne
     for (int j = 0; j < 4; ++j) q4[j] = sm.p[6 * B + 4 * t + j];
   }
   float am[3] = {0.f, 0.f, 0.f}, als[3] = {0.f, 0.f, 0.f}, aq[4] = {0.f, 0.f, 0.f, 0.f}, alog = 0.f;
-  if constexpr (MULTI) {
-    if (t < cnt)
-      for (int e = 0; e < NS; ++e) sm.gs[t * RS + e] = 0.f;
-  }
-  for (int v = 0; v < (MULTI ? a.views : 1); ++v) {  // the one-view variant runs for one view only
-    float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (t < cnt) {
-      if (v > 0) {
-        const int64_t it = (int64_t)v * N + base + t;
-        G0 = g2d[3 * it];
-        G1 = g2d[3 * it + 1];
-        G2 = g2d[3 * it + 2];
-        if (nonzero_record(G0, G1, G2)) zero_record(g2d + 3 * it);
+  float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (t < cnt) {
+    GaussGrad<D> gg;
+    const bool nz = nonzero_record(G0, G1, G2);
+    if (nz) {
+      const float* row = sm.sp + t * RS;
+      gaussian_grad<D>(a.cv[0], a.dilation, pq, q4, ls, sm.p[10 * B + t], row, G0, G1, G2, gg);
+      alog = gg.glogit;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        am[c] = gg.gm[c];
+        als[c] = gg.gls[c];
       }
-      GaussGrad<D> gg;
-      const bool nz = nonzero_record(G0, G1, G2);
-      if (nz) {
-        gaussian_grad<D>(a.cv[v], a.dilation, pq, q4, ls, sm.p[10 * B + t], sm.sp + t * RS, G0, G1, G2, gg);
-        alog += gg.glogit;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          am[c] += gg.gm[c];
-          als[c] += gg.gls[c];
-        }
+      for (int j = 0; j < 4; ++j) aq[j] = gg.gq[j];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) aq[j] += gg.gq[j];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) pose[k] = gg.pose[k];
-      }
-      if constexpr (MULTI) {
-        if (nz) {
-#pragma unroll
-          for (int k = 0; k < K; ++k)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) sm.gs[t * RS + 3 * k + c] += gg.Y[k] * gg.graw[c];
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sm.graw[t][c] = nz ? gg.graw[c] : 0.f;
-#pragma unroll
-        for (int k = 0; k < K; ++k) sm.Y[t][k] = nz ? gg.Y[k] : 0.f;
-      }
+      for (int k = 0; k < 6; ++k) pose[k] = gg.pose[k];
     }
-    if (pose_partials) block_pose_partial(pose, pose_partials + ((size_t)blockIdx.x * a.views + v) * 6);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sm.graw[t][c] = nz ? gg.graw[c] : 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) sm.Y[t][k] = nz ? gg.Y[k] : 0.f;
   }
+  if (pose_partials) block_pose_partial(pose, pose_partials + (size_t)blockIdx.x * 6);
   if (t < cnt) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -930,45 +890,275 @@ __global__ void __launch_bounds__(fused_threads<MULTI>()) project_bwd_adam_kerne
       V[f] = v;
     }
   }
-  if constexpr (B == 32) {
-    // a warp per block: walk the SH rows, lane t on columns t, t + 32, ...
-    // (coalesced rows, and each lane's coefficient (k, c) fixed per column)
+  // walk the SH rows, lane t on columns t, t + 32, ... (coalesced rows, and each
+  // lane's coefficient (k, c) fixed per column)
 #pragma unroll
-    for (int c0 = 0; c0 < NS; c0 += B) {
-      const int rr = c0 + t;
-      if (rr < NS) {
-        const int k = rr / 3, c = rr - 3 * k;
-        const float lr = k == 0 ? ad.lr[4] : ad.lr[5];
-        for (int gi = 0; gi < cnt; ++gi) {
-          const int e = gi * NS + rr;
-          float p = sm.sp[gi * RS + rr], m = sm.sm[shM + e], v = sm.sv[shV + e];
-          float g;
-          if constexpr (MULTI)
-            g = sm.gs[gi * RS + rr];
-          else
-            g = sm.Y[gi][k] * sm.graw[gi][c];
-          adam_update(p, g, m, v, lr, ad);
-          const int64_t f = gsh + e;
-          P[f] = p;
-          M[f] = m;
-          V[f] = v;
-        }
+  for (int c0 = 0; c0 < NS; c0 += B) {
+    const int rr = c0 + t;
+    if (rr < NS) {
+      const int k = rr / 3, c = rr - 3 * k;
+      const float lr = k == 0 ? ad.lr[4] : ad.lr[5];
+      for (int gi = 0; gi < cnt; ++gi) {
+        const int e = gi * NS + rr;
+        float p = sm.sp[gi * RS + rr], m = sm.sm[shM + e], v = sm.sv[shV + e];
+        adam_update(p, sm.Y[gi][k] * sm.graw[gi][c], m, v, lr, ad);
+        const int64_t f = gsh + e;
+        P[f] = p;
+        M[f] = m;
+        V[f] = v;
       }
     }
-  } else {
-    for (int e = t; e < cnt * NS; e += B) {
-      const int gi = e / NS, rr = e - gi * NS;
-      const int k = rr / 3, c = rr - 3 * k;
-      const int64_t f = gsh + e;
-      float p = sm.sp[gi * RS + rr], m = sm.sm[shM + e], v = sm.sv[shV + e], g;
-      if constexpr (MULTI)
-        g = sm.gs[gi * RS + rr];
+  }
+}
+
+// The same for several views: a block owns kMultiB consecutive Gaussians, one
+// per thread, whose gradient records (one per view) are turned into parameter
+// gradients summed over the views in shared memory.  The parameters are staged,
+// the SH slice in 16-byte pieces of the global array whatever the slice's own
+// alignment; the moments are on their way to L2 meanwhile and go from there to
+// registers and back in float4 (all but the pieces that the slice shares with
+// its neighbours).  Bound by the views' gradients (900 instructions per visible
+// item) beside HBM: staging the moments too, 32 Gaussians per block, left 5
+// blocks of one warp per SM (489 us for 5 views of 2^20 slots, 381 us for 8
+// views of 500k); now 6 blocks of two warps with 165 registers (427, 316 us).
+// For one view, where the staged form has 8 blocks, it is the faster one (91
+// against 96 us for 300k).
+constexpr int kMultiB = 64;  // Gaussians and threads of a block
+
+// The SH slice of a block in pieces of four floats aligned in the global
+// array: piece c holds the slice's floats 4 c - shift .. 4 c - shift + 3, shift
+// = the slice's place within 16 bytes.  Rows whose length is a multiple of 4
+// floats are kept 4 floats apart in shared memory (a thread reads its own row:
+// 4-way bank conflicts instead of 16-way); pieces keep their 16-byte alignment.
+template <int D>
+struct ShRows {
+  static constexpr int K = (D + 1) * (D + 1);
+  static constexpr int NS = 3 * K;
+  static constexpr bool kPad = NS % 4 == 0;
+  static constexpr int RS = kPad ? NS + 4 : NS;
+  static constexpr int WORDS = (kMultiB + 1) * RS + 8;
+  // shared-memory word of piece c's first float
+  static __device__ __forceinline__ int piece(int c) {
+    return kPad ? (c / (NS / 4)) * RS + 4 * (c % (NS / 4)) : 4 * c;
+  }
+  // shared-memory word of float rr of row t
+  static __device__ __forceinline__ int word(int t, int rr, int shift) {
+    if constexpr (!kPad) return t * NS + rr + shift;
+    const int q = rr + shift;
+    return q < NS ? t * RS + q : (t + 1) * RS + q - NS;
+  }
+};
+
+template <int D>
+struct MultiSmem {
+  static constexpr int K = ShRows<D>::K, NS = ShRows<D>::NS;
+  static constexpr int GS = NS % 2 == 0 ? NS + 1 : NS;  // summed SH gradients' row stride
+  static constexpr int B = kMultiB;
+  float sp[ShRows<D>::WORDS];  // SH parameters
+  float p[B * 11];             // means (3B) | log-scales (3B) | quats (4B) | logits (B)
+  float g[B * 11];             // gradients, same layout
+  float gs[B * GS];            // SH gradients summed over the views
+  __device__ __forceinline__ float grad(int t, int rr) const { return gs[t * GS + rr]; }
+};
+
+__device__ __forceinline__ void prefetch_l2(const float* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// A row of SH parameters as gaussian_grad reads it.
+template <int D>
+struct ShRow {
+  const float* sp;
+  int t, shift;
+  __device__ __forceinline__ float operator[](int rr) const { return sp[ShRows<D>::word(t, rr, shift)]; }
+};
+
+template <int D>
+__global__ void __launch_bounds__(kMultiB, 6)
+    project_bwd_adam_multi_kernel(const __grid_constant__ ProjectArgs a, float4* __restrict__ g2d,
+                                  float* __restrict__ P, float* __restrict__ M, float* __restrict__ V, AdamArgs ad,
+                                  float* __restrict__ pose_partials, const __grid_constant__ LossFoldArgs L) {
+  pdl_enter();
+  if (L.out && threadIdx.x < 32) fused_loss_reduce(L);  // one warp's work
+  device_bias_corrections(ad);
+  using S = MultiSmem<D>;
+  using Rows = ShRows<D>;
+  constexpr int K = S::K, NS = S::NS, B = kMultiB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  S& sm = *reinterpret_cast<S*>(smem_raw);
+  const int64_t N = a.n;
+  const int base = blockIdx.x * B;
+  const int cnt = min(B, a.n - base);
+  const int t = threadIdx.x;
+  const int64_t g0[4] = {3 * (int64_t)base, 3 * N + 3 * (int64_t)base, 6 * N + 4 * (int64_t)base, 10 * N + base};
+  const int so[4] = {0, 3 * B, 6 * B, 10 * B};
+  const int len[4] = {3 * cnt, 3 * cnt, 4 * cnt, cnt};
+  const int64_t gsh = 11 * N + (int64_t)base * NS;
+  const int total = cnt * NS;
+  // (a slice whose arrays lie differently within 16 bytes is swept float by float)
+  const int shift = (int)(((uintptr_t)(P + gsh) >> 2) & 3u);
+  const bool vec = ((((uintptr_t)(M + gsh) >> 2) & 3u) == (unsigned)shift) &&
+                   ((((uintptr_t)(V + gsh) >> 2) & 3u) == (unsigned)shift);
+  const int pieces = (total + shift + 3) >> 2;
+
+  // the moments' slices on their way to L2 while the gradients are computed
+  for (int l = t; 32 * l < total; l += B) {
+    prefetch_l2(M + gsh + 32 * l);
+    prefetch_l2(V + gsh + 32 * l);
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    for (int l = t; 32 * l < len[r]; l += B) {
+      prefetch_l2(M + g0[r] + 32 * l);
+      prefetch_l2(V + g0[r] + 32 * l);
+    }
+  // 1. asynchronous staging of the parameters; whole pieces as one copy
+  {
+    const float* src = P + gsh - shift;
+    for (int c = t; c < pieces; c += B) {
+      const int e = 4 * c - shift;  // first float of the piece in the slice
+      float* dst = sm.sp + Rows::piece(c);
+      if (e >= 0 && e + 4 <= total)
+        cp_async16(dst, src + 4 * c);
       else
-        g = sm.Y[gi][k] * sm.graw[gi][c];
-      adam_update(p, g, m, v, k == 0 ? ad.lr[4] : ad.lr[5], ad);
-      P[f] = p;
-      M[f] = m;
-      V[f] = v;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (e + j >= 0 && e + j < total) cp_async4(dst + j, src + 4 * c + j);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    for (int e = t; e < len[r]; e += B) cp_async4(&sm.p[so[r] + e], P + g0[r] + e);
+  cp_async_commit();
+  float4 G0 = make_float4(0.f, 0.f, 0.f, 0.f), G1 = G0, G2 = G0;
+  if (t < cnt) {
+    const int64_t i = base + t;
+    G0 = g2d[3 * i];
+    G1 = g2d[3 * i + 1];
+    G2 = g2d[3 * i + 2];
+    if (nonzero_record(G0, G1, G2)) zero_record(g2d + 3 * i);
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+
+  // 2. per-Gaussian gradients
+  float pq[3], ls[3], q4[4];
+  if (t < cnt) {
+    for (int c = 0; c < 3; ++c) {
+      pq[c] = sm.p[3 * t + c];
+      ls[c] = sm.p[3 * B + 3 * t + c];
+    }
+    for (int j = 0; j < 4; ++j) q4[j] = sm.p[6 * B + 4 * t + j];
+  }
+  float am[3] = {0.f, 0.f, 0.f}, als[3] = {0.f, 0.f, 0.f}, aq[4] = {0.f, 0.f, 0.f, 0.f}, alog = 0.f;
+  for (int e = 0; e < NS; ++e) sm.gs[t * S::GS + e] = 0.f;
+  for (int v = 0; v < a.views; ++v) {
+    float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (t < cnt) {
+      if (v > 0) {
+        const int64_t it = (int64_t)v * N + base + t;
+        G0 = g2d[3 * it];
+        G1 = g2d[3 * it + 1];
+        G2 = g2d[3 * it + 2];
+        if (nonzero_record(G0, G1, G2)) zero_record(g2d + 3 * it);
+      }
+      GaussGrad<D> gg;
+      const bool nz = nonzero_record(G0, G1, G2);
+      if (nz) {
+        const ShRow<D> row{sm.sp, t, shift};
+        gaussian_grad<D>(a.cv[v], a.dilation, pq, q4, ls, sm.p[10 * B + t], row, G0, G1, G2, gg);
+        alog += gg.glogit;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          am[c] += gg.gm[c];
+          als[c] += gg.gls[c];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) aq[j] += gg.gq[j];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) pose[k] = gg.pose[k];
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) sm.gs[t * S::GS + 3 * k + c] += gg.Y[k] * gg.graw[c];
+      }
+    }
+    if (pose_partials) block_pose_partial(pose, pose_partials + ((size_t)blockIdx.x * a.views + v) * 6);
+  }
+  if (t < cnt) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      sm.g[3 * t + c] = am[c];
+      sm.g[3 * B + 3 * t + c] = als[c];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sm.g[6 * B + 4 * t + j] = aq[j];
+    sm.g[10 * B + t] = alog;
+  }
+  __syncthreads();
+
+  // 3. Adam sweeps (dense: zero gradients still update the moments)
+  auto one = [&](int e) {  // float e of the SH slice
+    const int gi = e / NS, rr = e - gi * NS;
+    float p = sm.sp[Rows::word(gi, rr, shift)], m = M[gsh + e], v = V[gsh + e];
+    adam_update(p, sm.grad(gi, rr), m, v, rr < 3 ? ad.lr[4] : ad.lr[5], ad);
+    P[gsh + e] = p;
+    M[gsh + e] = m;
+    V[gsh + e] = v;
+  };
+  if (vec) {
+    const int whole0 = shift ? 1 : 0, whole1 = (total + shift) >> 2;  // pieces within the slice
+    float4* P4 = reinterpret_cast<float4*>(P + gsh - shift);
+    float4* M4 = reinterpret_cast<float4*>(M + gsh - shift);
+    float4* V4 = reinterpret_cast<float4*>(V + gsh - shift);
+    constexpr int U = 4;  // pieces whose moments are loaded together
+    for (int c0 = whole0 + t; c0 < whole1; c0 += U * B) {
+      float4 m4[U], v4[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (c0 + u * B < whole1) {
+          m4[u] = M4[c0 + u * B];
+          v4[u] = V4[c0 + u * B];
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int c = c0 + u * B;
+        if (c >= whole1) break;
+        float4 p4 = *reinterpret_cast<const float4*>(sm.sp + Rows::piece(c));
+        float* pp = &p4.x;
+        float* mm = &m4[u].x;
+        float* vv = &v4[u].x;
+        const int e0 = 4 * c - shift, gi0 = e0 / NS, rr0 = e0 - gi0 * NS;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool next = rr0 + j >= NS;
+          const int gi = next ? gi0 + 1 : gi0, rr = next ? rr0 + j - NS : rr0 + j;
+          adam_update(pp[j], sm.grad(gi, rr), mm[j], vv[j], rr < 3 ? ad.lr[4] : ad.lr[5], ad);
+        }
+        P4[c] = p4;
+        M4[c] = m4[u];
+        V4[c] = v4[u];
+      }
+    }
+    const int head = whole0 ? min(4 - shift, total) : 0, tail = max(head, 4 * whole1 - shift);
+    if (t < head) one(t);
+    if (t < total - tail) one(tail + t);
+  } else {
+    for (int e = t; e < total; e += B) one(e);
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const float lr = ad.lr[r];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int e = t + k * B;
+      if (e < len[r]) {
+        const int l = so[r] + e;
+        const int64_t f = g0[r] + e;
+        float p = sm.p[l], m = M[f], v = V[f];
+        adam_update(p, sm.g[l], m, v, lr, ad);
+        P[f] = p;
+        M[f] = m;
+        V[f] = v;
+      }
     }
   }
 }
@@ -1036,26 +1226,25 @@ int launch_project_bwd(const ProjectArgs& a, float4* g2d, float* g_means, float*
 int launch_project_bwd_adam(const ProjectArgs& a, float4* g2d, float* params, float* m, float* v,
                             const AdamArgs& ad, float* pose_partials, cudaStream_t s, const LossFoldArgs* loss) {
   if (a.n <= 0) return 0;
-  const int bt = a.views == 1 ? fused_threads<false>() : fused_threads<true>();
+  const int bt = a.views == 1 ? kFusedThreads : kMultiB;
   const int nb = (a.n + bt - 1) / bt;
   LossFoldArgs L{};
   if (loss) L = *loss;
-#define GS_FUSED(D_, M_, S_)                                                                                  \
-  launch_pdl(project_bwd_adam_kernel<D_, M_>, nb, fused_threads<M_>(), sizeof(S_<D_>), s, a, g2d, params, m, v, ad, \
-             pose_partials, L)
+#define GS_FUSED(K_, D_, S_) \
+  launch_pdl(K_<D_>, nb, bt, sizeof(S_<D_>), s, a, g2d, params, m, v, ad, pose_partials, L)
   if (a.views == 1) {
     switch (a.sh_degree) {
-      case 0: GS_FUSED(0, false, FusedSmem); break;
-      case 1: GS_FUSED(1, false, FusedSmem); break;
-      case 2: GS_FUSED(2, false, FusedSmem); break;
-      default: GS_FUSED(3, false, FusedSmem); break;
+      case 0: GS_FUSED(project_bwd_adam_kernel, 0, FusedSmem); break;
+      case 1: GS_FUSED(project_bwd_adam_kernel, 1, FusedSmem); break;
+      case 2: GS_FUSED(project_bwd_adam_kernel, 2, FusedSmem); break;
+      default: GS_FUSED(project_bwd_adam_kernel, 3, FusedSmem); break;
     }
   } else {
     switch (a.sh_degree) {
-      case 0: GS_FUSED(0, true, FusedSmemMulti); break;
-      case 1: GS_FUSED(1, true, FusedSmemMulti); break;
-      case 2: GS_FUSED(2, true, FusedSmemMulti); break;
-      default: GS_FUSED(3, true, FusedSmemMulti); break;
+      case 0: GS_FUSED(project_bwd_adam_multi_kernel, 0, MultiSmem); break;
+      case 1: GS_FUSED(project_bwd_adam_multi_kernel, 1, MultiSmem); break;
+      case 2: GS_FUSED(project_bwd_adam_multi_kernel, 2, MultiSmem); break;
+      default: GS_FUSED(project_bwd_adam_multi_kernel, 3, MultiSmem); break;
     }
   }
 #undef GS_FUSED
@@ -1063,17 +1252,16 @@ int launch_project_bwd_adam(const ProjectArgs& a, float4* g2d, float* params, fl
 }
 
 void init_project_kernels() {
-#define GS_ATTR(D_, M_, S_)                                                                           \
-  cudaFuncSetAttribute(project_bwd_adam_kernel<D_, M_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                       (int)sizeof(S_<D_>))
-  GS_ATTR(0, false, FusedSmem);
-  GS_ATTR(1, false, FusedSmem);
-  GS_ATTR(2, false, FusedSmem);
-  GS_ATTR(3, false, FusedSmem);
-  GS_ATTR(0, true, FusedSmemMulti);
-  GS_ATTR(1, true, FusedSmemMulti);
-  GS_ATTR(2, true, FusedSmemMulti);
-  GS_ATTR(3, true, FusedSmemMulti);
+#define GS_ATTR(K_, D_, S_) \
+  cudaFuncSetAttribute(K_<D_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(S_<D_>))
+  GS_ATTR(project_bwd_adam_kernel, 0, FusedSmem);
+  GS_ATTR(project_bwd_adam_kernel, 1, FusedSmem);
+  GS_ATTR(project_bwd_adam_kernel, 2, FusedSmem);
+  GS_ATTR(project_bwd_adam_kernel, 3, FusedSmem);
+  GS_ATTR(project_bwd_adam_multi_kernel, 0, MultiSmem);
+  GS_ATTR(project_bwd_adam_multi_kernel, 1, MultiSmem);
+  GS_ATTR(project_bwd_adam_multi_kernel, 2, MultiSmem);
+  GS_ATTR(project_bwd_adam_multi_kernel, 3, MultiSmem);
 #undef GS_ATTR
 }
 
