@@ -496,9 +496,10 @@ __device__ __forceinline__ void warp_sort_list(uint32_t* __restrict__ ids, const
 // instead of a 64-bit compare and four selects, and half the shuffles.  Entries
 // whose rounded depths are equal come out in the order of their places.  Equal
 // depths are common (a level camera sees a horizontal plane at one depth per
-// pixel row), so a list that has any is sorted a second time, by (run of equal
-// rounded depths, the depth's bits that were rounded off, id); where these do
-// not fit into 32 bits, by the 64-bit keys.
+// pixel row), so in a list that has any the runs of equal rounded depths are
+// put in order by (the depth's bits that were rounded off, id): by neighbour
+// exchanges within the runs, if these take long by a second sort with the run
+// in front, and where the keys do not fit into 32 bits by the 64-bit keys.
 //
 // The networks' merges start by comparing mirrored places (e with e ^ (k - 1)),
 // so every compare-exchange puts the smaller key at the smaller place.  Blocked
@@ -606,22 +607,64 @@ __device__ __forceinline__ uint32_t sorted_ids_ties(const uint32_t (&x)[KEYS], c
   return ties;
 }
 
-// Second keys of the entries: runs counted from `run` on; false when they do
-// not fit.
+// Second keys of the entries: the depth's bits that were rounded off, id.
 struct IdMap {
   uint32_t imin;
   int bits;
+  __device__ __forceinline__ uint32_t id(uint32_t key) const {
+    return imin + (key & (bits == 32 ? 0xFFFFFFFFu : (1u << bits) - 1u));
+  }
 };
+__device__ __forceinline__ IdMap id_map(uint32_t imin, uint32_t imax) { return IdMap{imin, 32 - __clz(imax - imin)}; }
 template <int KEYS>
-__device__ __forceinline__ void run_keys(uint32_t (&id)[KEYS], const uint32_t* __restrict__ zkey, uint32_t n, uint32_t e0,
-                                         uint32_t ties, uint32_t run, const KeyMap& k, const IdMap& m, uint32_t n_items) {
+__device__ __forceinline__ void second_keys(uint32_t (&id)[KEYS], const uint32_t* __restrict__ zkey, uint32_t n,
+                                            uint32_t e0, const KeyMap& k, const IdMap& m, uint32_t n_items) {
+#pragma unroll
+  for (int i = 0; i < KEYS; ++i) {
+    uint32_t low = 0u;
+    if (k.shift && e0 + i < n && in_bounds(id[i] < n_items)) low = (zkey[id[i]] - k.zmin) & ((1u << k.shift) - 1u);
+    id[i] = e0 + i < n ? (k.shift ? low << m.bits : 0u) | (id[i] - m.imin) : 0xFFFFFFFFu;
+  }
+}
+// ... led by the run, counted from `run` on
+template <int KEYS>
+__device__ __forceinline__ void run_keys(uint32_t (&x)[KEYS], uint32_t n, uint32_t e0, uint32_t ties, uint32_t run,
+                                         int low_bits) {
 #pragma unroll
   for (int i = 0; i < KEYS; ++i) {
     if (!(ties >> i & 1u)) ++run;
-    uint32_t key = (run - 1u) << k.shift;
-    if (k.shift && e0 + i < n && in_bounds(id[i] < n_items)) key |= (zkey[id[i]] - k.zmin) & ((1u << k.shift) - 1u);
-    id[i] = e0 + i < n ? (key << m.bits) | (id[i] - m.imin) : 0xFFFFFFFFu;
+    if (e0 + i < n) x[i] |= (run - 1u) << low_bits;
   }
+}
+
+// A pass of neighbour exchanges within the runs (odd-even transposition; every
+// other pair of neighbours, then the rest), and whether each run is in order.
+// Runs are short (1.5 entries on average) and nearly in order, so a few
+// passes do what another sort would.
+constexpr int kSettleRounds = 8, kSettlePasses = 2;
+template <int KEYS>
+__device__ __forceinline__ void settle_pass(uint32_t (&x)[KEYS], uint32_t ties, int lane) {
+#pragma unroll
+  for (int first = 0; first < 2; ++first)
+#pragma unroll
+    for (int i = first; i + 1 < KEYS; i += 2) {
+      const uint32_t a = x[i], b = x[i + 1];
+      const bool sw = (ties >> (i + 1) & 1u) && b < a;
+      x[i] = sw ? b : a;
+      x[i + 1] = sw ? a : b;
+    }
+  const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, x[0], 1), prev = __shfl_up_sync(0xFFFFFFFFu, x[KEYS - 1], 1);
+  const bool tie = __shfl_down_sync(0xFFFFFFFFu, ties, 1) & 1u;
+  if (lane < 31 && tie) x[KEYS - 1] = min(x[KEYS - 1], next);
+  if (lane > 0 && (ties & 1u)) x[0] = max(x[0], prev);
+}
+template <int KEYS>
+__device__ __forceinline__ bool settled(const uint32_t (&x)[KEYS], uint32_t ties, int lane) {
+  const uint32_t prev = __shfl_up_sync(0xFFFFFFFFu, x[KEYS - 1], 1);
+  bool ok = lane == 0 || !(ties & 1u) || prev <= x[0];
+#pragma unroll
+  for (int i = 0; i + 1 < KEYS; ++i) ok = ok && (!(ties >> (i + 1) & 1u) || x[i] <= x[i + 1]);
+  return __all_sync(0xFFFFFFFFu, ok);
 }
 
 // One warp sorts the list of n <= 32 KEYS ids at ids[off ..]; true: it has to
@@ -657,28 +700,32 @@ __device__ __forceinline__ bool warp_sort_list32(uint32_t* ids, const uint32_t* 
   const uint32_t e0 = (uint32_t)(lane * KEYS);
   uint32_t id[KEYS];
   const uint32_t ties = sorted_ids_ties<KEYS>(x, ids, off, n, e0, k, __shfl_up_sync(0xFFFFFFFFu, x[KEYS - 1], 1), id);
-  uint32_t add = 0u, mask = 0xFFFFFFFFu;
+  IdMap m{0u, 32};
   if (__any_sync(0xFFFFFFFFu, ties != 0u)) {
-    IdMap m;
-    m.imin = __reduce_min_sync(0xFFFFFFFFu, imin);
-    m.bits = 32 - __clz(__reduce_max_sync(0xFFFFFFFFu, imax) - m.imin);
-    if (k.bits + k.shift + m.bits > 32) return true;
-    const uint32_t runs = (uint32_t)(KEYS - __popc(ties));
-    uint32_t incl = runs;
+    m = id_map(__reduce_min_sync(0xFFFFFFFFu, imin), __reduce_max_sync(0xFFFFFFFFu, imax));
+    if (k.shift + m.bits > 32) return true;
+    second_keys<KEYS>(id, zkey, n, e0, k, m, n_items);
+    int round = 0;
+    for (; round < kSettleRounds && !settled<KEYS>(id, ties, lane); ++round)
+#pragma unroll 1
+      for (int p = 0; p < kSettlePasses; ++p) settle_pass<KEYS>(id, ties, lane);
+    if (round == kSettleRounds) {
+      if (k.bits + k.shift + m.bits > 32) return true;
+      const uint32_t runs = (uint32_t)(KEYS - __popc(ties));
+      uint32_t incl = runs;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (lane >= d) incl += y;
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= d) incl += y;
+      }
+      run_keys<KEYS>(id, n, e0, ties, incl - runs, k.shift + m.bits);
+      warp_sort32<KEYS>(id, lane, n);
     }
-    run_keys<KEYS>(id, zkey, n, e0, ties, incl - runs, k, m, n_items);
-    warp_sort32<KEYS>(id, lane, n);
-    add = m.imin;
-    mask = m.bits == 32 ? 0xFFFFFFFFu : (1u << m.bits) - 1u;
   }
   __syncwarp();  // every place has been read
 #pragma unroll
   for (int i = 0; i < KEYS; ++i)
-    if (e0 + i < n) ids[off + e0 + i] = add + (id[i] & mask);
+    if (e0 + i < n) ids[off + e0 + i] = m.id(id[i]);
   return false;
 }
 
@@ -760,32 +807,46 @@ __device__ __forceinline__ bool cta_sort_list32(uint32_t* ids, const uint32_t* _
   if (lane == 0 && warp > 0) prev = s[warp - 1];
   uint32_t id[KEYS];
   const uint32_t ties = sorted_ids_ties<KEYS>(x, ids, off, n, e0, k, prev, id);
-  uint32_t add = 0u, mask = 0xFFFFFFFFu;
+  if (lane == 0) s[kLongWarps + warp] = ties & 1u;
+  IdMap m{0u, 32};
   if (__syncthreads_or(ties != 0u)) {  // (also: every place has been read)
-    IdMap m;
-    m.imin = imin;
-    m.bits = 32 - __clz(imax - imin);
-    if (k.bits + k.shift + m.bits > 32) return true;
-    const uint32_t runs = (uint32_t)(KEYS - __popc(ties));
-    uint32_t incl = runs;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (lane >= d) incl += y;
+    m = id_map(imin, imax);
+    if (k.shift + m.bits > 32) return true;
+    second_keys<KEYS>(id, zkey, n, e0, k, m, n_items);
+    const bool tie_next = warp + 1 < kLongWarps && s[kLongWarps + warp + 1] != 0u;  // of the next warp's first entry
+    __syncthreads();
+    bool open = true;
+    for (int round = 0; round < kSettleRounds && open; ++round) {
+#pragma unroll 1
+      for (int p = 0; p < kSettlePasses; ++p) settle_pass<KEYS>(id, ties, lane);
+      if (lane == 0) s[warp] = id[0];
+      if (lane == 31) s[kLongWarps + warp] = id[KEYS - 1];
+      __syncthreads();
+      if (lane == 0 && warp > 0 && (ties & 1u)) id[0] = max(id[0], s[kLongWarps + warp - 1]);
+      if (lane == 31 && tie_next) id[KEYS - 1] = min(id[KEYS - 1], s[warp + 1]);
+      open = __syncthreads_or(!settled<KEYS>(id, ties, lane));
     }
-    if (lane == 31) s[kLongWarps + warp] = incl;
-    __syncthreads();
-    uint32_t run = incl - runs;
-    for (int w = 0; w < warp; ++w) run += s[kLongWarps + w];
-    __syncthreads();
-    run_keys<KEYS>(id, zkey, n, e0, ties, run, k, m, n_items);
-    cta_sort32(id, lane, warp, n, s);
-    add = m.imin;
-    mask = m.bits == 32 ? 0xFFFFFFFFu : (1u << m.bits) - 1u;
+    if (open) {
+      if (k.bits + k.shift + m.bits > 32) return true;
+      const uint32_t runs = (uint32_t)(KEYS - __popc(ties));
+      uint32_t incl = runs;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= d) incl += y;
+      }
+      if (lane == 31) s[kLongWarps + warp] = incl;
+      __syncthreads();
+      uint32_t run = incl - runs;
+      for (int w = 0; w < warp; ++w) run += s[kLongWarps + w];
+      __syncthreads();
+      run_keys<KEYS>(id, n, e0, ties, run, k.shift + m.bits);
+      cta_sort32(id, lane, warp, n, s);
+    }
   }
 #pragma unroll
   for (int i = 0; i < KEYS; ++i)
-    if (e0 + i < n) ids[off + e0 + i] = add + (id[i] & mask);
+    if (e0 + i < n) ids[off + e0 + i] = m.id(id[i]);
   __syncthreads();  // s is reused by the next long list
   return false;
 }
@@ -838,8 +899,10 @@ __device__ __forceinline__ void cta_sort_list64(uint32_t* __restrict__ ids, cons
 // Bound by latency (one wave of warps, each a chain of loads and exchanges).
 // 64-bit keys throughout, and long lists by the CTA that met them: 25.3 us for
 // 3225 lists of 207 entries (1200 x 680), 503 us for 16125 of 494, 167 us for
-// 8030 of 284, 941 us for 31360 of 398 (up to 4 lists of 4000 in one CTA); now
-// 21, 224, 52 and 435 us.
+// 8030 of 284, 941 us for 31360 of 398 (up to 4 lists of 4000 in one CTA).  With
+// a second sort (by 64 bits for the longer lists of a million Gaussians, where
+// the second keys with the run do not fit) in place of the neighbour exchanges
+// 21, 224, 52 and 435 us; now 18.3, 155, 41 and 222 us.
 __global__ void __launch_bounds__(kSortThreads, 6) tile_sort_kernel(const uint32_t* __restrict__ offsets,
                                                                  uint32_t* __restrict__ counts, uint32_t* ids,
                                                                  const uint32_t* __restrict__ zkey,
