@@ -23,7 +23,7 @@ namespace gs {
 namespace {
 
 constexpr int kBinThreads = 256;
-constexpr int kBinWarps = kBinThreads / 32;
+constexpr int kScatterItems = 64;  // items per block of the scatter into lists of few items
 constexpr int kScanThreads = 1024;
 constexpr int kSortThreads = 128;
 constexpr int kSortWarps = kSortThreads / 32;  // tiles per CTA of the per-tile sort
@@ -43,27 +43,29 @@ __device__ __forceinline__ ItemTiles item_tiles(const TileMap& map, uint32_t it)
 // Calls f(item, global tile, active) for every tile of every item's
 // rectangle.  Items with more than kBigTiles tiles come from the queue
 // the projection built (see the end); the others are expanded by their
-// block, 256 consecutive items at a time: a block scan of their tile counts
+// block, ITEMS consecutive items at a time: a block scan of their tile counts
 // gives each item's first pair, and the block's threads take consecutive
 // pairs (owner found by binary search over the prefix in shared memory), so
 // one large splat is spread over the whole block and large splats clustered
-// in one region are averaged over 256 items.
-// `active` is the mask of lanes of the calling warp that call f together.
-template <bool SMALL = true, class F>
+// in one region are averaged over ITEMS items.
+// `active` is the mask of lanes of the calling warp that call f together, 0
+// when their tiles are known to differ.
+template <int ITEMS = kBinThreads, class F>
 __device__ __forceinline__ void for_each_pair(int n, const ushort4* __restrict__ rects,
                                               const uint32_t* __restrict__ tiles, const TileMap& map,
                                               const uint32_t* __restrict__ big_queue,
                                               const uint32_t* __restrict__ big_len, F f) {
-  __shared__ uint32_t s_excl[kBinThreads];
-  __shared__ ushort4 s_rect[kBinThreads];
-  __shared__ ItemTiles s_map[kBinThreads];
-  __shared__ uint32_t s_wsum[kBinWarps];
+  __shared__ uint32_t s_excl[ITEMS];
+  __shared__ ushort4 s_rect[ITEMS];
+  __shared__ ItemTiles s_map[ITEMS];
+  __shared__ uint32_t s_wsum[ITEMS / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int base = blockIdx.x * kBinThreads; SMALL && base < n; base += gridDim.x * kBinThreads) {
+  for (int base = blockIdx.x * ITEMS; base < n; base += gridDim.x * ITEMS) {
+    const bool item = (int)threadIdx.x < ITEMS;
     const int g = base + threadIdx.x;
-    uint32_t cnt = g < n ? tiles[g] : 0u;
+    uint32_t cnt = item && g < n ? tiles[g] : 0u;
     if (cnt > kBigTiles) cnt = 0;  // expanded from the queue below
-    const ushort4 r = g < n ? rects[g] : make_ushort4(0, 0, 0, 0);
+    const ushort4 r = item && g < n ? rects[g] : make_ushort4(0, 0, 0, 0);
     uint32_t incl = cnt;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -71,18 +73,20 @@ __device__ __forceinline__ void for_each_pair(int n, const ushort4* __restrict__
       if (lane >= off) incl += y;
     }
     __syncthreads();  // previous round done with the shared arrays
-    if (lane == 31) s_wsum[w] = incl;
+    if (item && lane == 31) s_wsum[w] = incl;
     __syncthreads();
     uint32_t wpre = 0, total = 0;
 #pragma unroll
-    for (int k = 0; k < kBinWarps; ++k) {
+    for (int k = 0; k < ITEMS / 32; ++k) {
       const uint32_t sk = s_wsum[k];
       wpre += k < w ? sk : 0u;
       total += sk;
     }
-    s_excl[threadIdx.x] = wpre + incl - cnt;
-    s_rect[threadIdx.x] = r;
-    s_map[threadIdx.x] = item_tiles(map, (uint32_t)min(g, n - 1));
+    if (item) {
+      s_excl[threadIdx.x] = wpre + incl - cnt;
+      s_rect[threadIdx.x] = r;
+      s_map[threadIdx.x] = item_tiles(map, (uint32_t)min(g, n - 1));
+    }
     __syncthreads();
     for (uint32_t k0 = 0; k0 < total; k0 += kBinThreads) {
       const uint32_t k = k0 + threadIdx.x;
@@ -90,7 +94,7 @@ __device__ __forceinline__ void for_each_pair(int n, const ushort4* __restrict__
       if (k >= total) break;
       int o = 0;
 #pragma unroll
-      for (int step = kBinThreads / 2; step > 0; step >>= 1)
+      for (int step = ITEMS / 2; step > 0; step >>= 1)
         if (s_excl[o + step] <= k) o += step;
       const ushort4 ro = s_rect[o];
       const ItemTiles mt = s_map[o];
@@ -112,25 +116,30 @@ __device__ __forceinline__ void for_each_pair(int n, const ushort4* __restrict__
     const uint32_t cnt = tiles[g];
     const ItemTiles mt = item_tiles(map, g);
     const uint32_t width = (uint32_t)(ro.z - ro.x);
-    for (uint32_t k0 = 0; k0 < cnt; k0 += 32) {
-      const uint32_t k = k0 + lane;
-      const unsigned active = __ballot_sync(0xFFFFFFFFu, k < cnt);
-      if (k >= cnt) break;
+    for (uint32_t k = lane; k < cnt; k += 32) {
       const uint32_t ty = ro.y + k / width, tx = ro.x + k % width;
-      f((int)g, mt.base + ty * mt.stride + tx, active);
+      f((int)g, mt.base + ty * mt.stride + tx, 0u);
     }
   }
+}
+
+// One more at tile t's counter: its value before.  Neighbouring items meet the
+// same tiles, so a warp's equal tiles go in one atomic (2.3M pairs: 19 us, 65
+// us with an atomic each); the lanes of a large rectangle never share one
+// (8.6M pairs, mostly of large ones: 246 -> 131 us without the matching).
+__device__ __forceinline__ uint32_t count_tile(uint32_t* __restrict__ counter, uint32_t t, unsigned active) {
+  return active ? warp_agg_inc(counter, t, active) : atomicAdd(&counter[t], 1u);
 }
 
 // Every (item, tile) pair adds one to its tile's counter (when the
 // projection has not counted them itself, as for gs_bin_tiles).
 __global__ void __launch_bounds__(kBinThreads) tile_count_kernel(const __grid_constant__ TileBinArgs a) {
   pdl_enter();
-  for_each_pair<true>(a.n, a.rects, a.tiles, a.map, a.big_queue, a.big_len,
-                       [&](int, uint32_t t, unsigned active) {
-                         // (the checked build counts a tile beyond the grid into tile 0, reported)
-                         warp_agg_inc(a.counts, in_bounds(t < (uint32_t)a.n_tiles) ? t : 0u, active);
-                       });
+  for_each_pair(a.n, a.rects, a.tiles, a.map, a.big_queue, a.big_len,
+                [&](int, uint32_t t, unsigned active) {
+                  // (the checked build counts a tile beyond the grid into tile 0, reported)
+                  count_tile(a.counts, in_bounds(t < (uint32_t)a.n_tiles) ? t : 0u, active);
+                });
 }
 
 // Difference grids of the huge rectangles (TileBinArgs::big_diff).
@@ -413,17 +422,18 @@ __global__ void __launch_bounds__(256) tile_scan_down_kernel(int T, const uint32
   }
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kBinThreads) tile_scatter_kernel(const __grid_constant__ TileBinArgs a) {
   pdl_enter();
   bool over = false;
-  for_each_pair(a.n, a.rects, a.tiles, a.map, a.big_queue, a.big_len,
-                [&](int g, uint32_t t, unsigned active) {
-                  const uint32_t pos = warp_agg_inc(a.cursors, in_bounds(t < (uint32_t)a.n_tiles) ? t : 0u, active);
-                  if (pos < a.capacity)
-                    a.ids[pos] = (uint32_t)g;
-                  else
-                    over = true;
-                });
+  for_each_pair<ITEMS>(a.n, a.rects, a.tiles, a.map, a.big_queue, a.big_len,
+                       [&](int g, uint32_t t, unsigned active) {
+                         const uint32_t pos = count_tile(a.cursors, in_bounds(t < (uint32_t)a.n_tiles) ? t : 0u, active);
+                         if (pos < a.capacity)
+                           a.ids[pos] = (uint32_t)g;
+                         else
+                           over = true;
+                       });
   if (over) atomicOr(a.overflow, 1u);
 }
 
@@ -1035,7 +1045,14 @@ void launch_tile_count_scan(const TileBinArgs& a, cudaStream_t s, int64_t* launc
 
 void launch_tile_scatter(const TileBinArgs& a, cudaStream_t s, int64_t* launches) {
   if (a.n > 0) {
-    launch_pdl(tile_scatter_kernel, bin_grid(a.n, a.num_sms), kBinThreads, 0, s, a);
+    // 64 items a block while that gives every block one round: more pairs in
+    // flight, fewer rounds (25.7 -> 20.6 us with the scan for 100k items, 25.0
+    // -> 20.1 us for 50k); with more items the blocks of 256 have enough of
+    // them, and fewer scans (1M items: 37 against 46 us)
+    if (a.n <= kScatterItems * 16 * max(a.num_sms, 1))
+      launch_pdl(tile_scatter_kernel<kScatterItems>, (a.n + kScatterItems - 1) / kScatterItems, kBinThreads, 0, s, a);
+    else
+      launch_pdl(tile_scatter_kernel<kBinThreads>, bin_grid(a.n, a.num_sms), kBinThreads, 0, s, a);
     if (launches) *launches += 1;
   }
 }
