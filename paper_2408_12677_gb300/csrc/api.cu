@@ -379,7 +379,7 @@ gs_status ensure_px(gs_ctx* c, int64_t npx) {
   GS_GROW(c, cap_px, regrow(&c->last, cap));
   GS_GROW(c, cap_px, regrow(&c->dl_img, 4 * cap));
   // per-block partials (blocks of every view: <= blocks(total) + views) and per-view scales
-  const int64_t lb = loss_blocks((int)std::min<int64_t>(cap, INT32_MAX - 4096));
+  const int64_t lb = loss_blocks_max(cap);
   GS_GROW(c, cap_px, regrow(&c->loss_partials, 3 * (lb + kMaxViews) + kMaxViews + 4));
   c->cap_px = cap;
   c->have_state = false;
@@ -1571,12 +1571,16 @@ gs_status loss_views(gs_ctx* c, int32_t V, const gs_camera* cams, const float* c
     if (!color[v] || !depth[v] || !target_rgb[v] || !target_depth[v] || !dL_dcolor[v] || !dL_ddepth[v])
       return fail(c, GS_ERR_INVALID_ARG, "loss: NULL image pointer");
     const int64_t npx = (int64_t)cams[v].width * cams[v].height;
-    la.v[v] = LossView{(int)npx, (int)blocks, color[v], depth[v], target_rgb[v], target_depth[v], dL_dcolor[v],
+    la.v[v] = LossView{(int)npx, 0, color[v], depth[v], target_rgb[v], target_depth[v], dL_dcolor[v],
                        dL_ddepth[v]};
     pixels += npx;
-    blocks += loss_blocks((int)npx);
   }
   if (pixels >= ((int64_t)1 << 31)) return fail(c, GS_ERR_INVALID_ARG, "a batch must have < 2^31 pixels");
+  la.items = loss_items(pixels);
+  for (int v = 0; v < V; ++v) {
+    la.v[v].block_base = (int)blocks;
+    blocks += loss_blocks(la.v[v].npix, la.items);
+  }
   la.n_blocks = (int)blocks;
   GS_CUDA(c, cudaSetDevice(c->device));
   gs_status st;

@@ -377,11 +377,14 @@ struct LossView {
 };
 struct LossArgs {
   int views, n_blocks;
+  int items;  // pixels per thread: loss_items of the call's pixels
   float w_color, w_depth;
   float* loss;
   LossView v[kMaxViews];
 };
-int loss_blocks(int npix);
+int loss_items(int64_t pixels);
+int64_t loss_blocks(int64_t npix, int items);
+int64_t loss_blocks_max(int64_t pixels);  // most blocks of a single-view call of up to that many pixels
 // partials: >= 3 * n_blocks + kMaxViews floats
 void launch_loss(const LossArgs& a, float* partials, cudaStream_t s, int64_t* launches);
 // step_dev non-null: bias corrections from the device step counter instead

@@ -56,7 +56,8 @@ extern "C" gs_status gs_loss_l1_noalloc(const gs_camera* cam, const float* color
   if (!color || !depth || !target_rgb || !target_depth || !loss || !dL_dcolor || !dL_ddepth) return GS_ERR_INVALID_ARG;
   const int64_t npix = (int64_t)cam->width * cam->height;
   if (npix > kMaxPixels) return GS_ERR_CAPACITY;
-  if (3 * (int64_t)gs::loss_blocks((int)npix) + 1 > kScratchFloats) return GS_ERR_CAPACITY;
+  const int items = gs::loss_items(npix);
+  if (3 * gs::loss_blocks(npix, items) + 1 > kScratchFloats) return GS_ERR_CAPACITY;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return GS_ERR_CUDA;
   if (dev < 0 || dev >= kMaxDevices) return GS_ERR_INVALID_ARG;
@@ -64,7 +65,8 @@ extern "C" gs_status gs_loss_l1_noalloc(const gs_camera* cam, const float* color
   if (scratch_for(dev, &scratch) != cudaSuccess) return GS_ERR_CUDA;
   gs::LossArgs la;
   la.views = 1;
-  la.n_blocks = gs::loss_blocks((int)npix);
+  la.n_blocks = (int)gs::loss_blocks(npix, items);
+  la.items = items;
   la.w_color = w_color;
   la.w_depth = w_depth;
   la.loss = loss;
