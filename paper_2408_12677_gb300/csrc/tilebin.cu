@@ -48,8 +48,10 @@ __device__ __forceinline__ ItemTiles item_tiles(const TileMap& map, uint32_t it)
 // pairs (owner found by binary search over the prefix in shared memory), so
 // one large splat is spread over the whole block and large splats clustered
 // in one region are averaged over ITEMS items.
-// `active` is the mask of lanes of the calling warp that call f together, 0
-// when their tiles are known to differ.
+// f's third argument is the mask of lanes of the calling warp that call f
+// together, or Distinct{} when their tiles are known to differ.
+struct Distinct {};
+constexpr uint32_t kHugeSpread = 256;
 template <int ITEMS = kBinThreads, class F>
 __device__ __forceinline__ void for_each_pair(int n, const ushort4* __restrict__ rects,
                                               const uint32_t* __restrict__ tiles, const TileMap& map,
@@ -116,19 +118,32 @@ __device__ __forceinline__ void for_each_pair(int n, const ushort4* __restrict__
     const uint32_t cnt = tiles[g];
     const ItemTiles mt = item_tiles(map, g);
     const uint32_t width = (uint32_t)(ro.z - ro.x);
-    for (uint32_t k = lane; k < cnt; k += 32) {
-      const uint32_t ty = ro.y + k / width, tx = ro.x + k % width;
-      f((int)g, mt.base + ty * mt.stride + tx, 0u);
+    auto tile = [&](uint32_t k) { return mt.base + (ro.y + k / width) * mt.stride + ro.x + k % width; };
+    if (cnt > kHugeSpread) {
+      for (uint32_t k = lane; k < cnt; k += 32) f((int)g, tile(k), Distinct{});
+    } else {
+      for (uint32_t k0 = 0; k0 < cnt; k0 += 32) {
+        const uint32_t k = k0 + lane;
+        const unsigned active = __ballot_sync(0xFFFFFFFFu, k < cnt);
+        if (k >= cnt) break;
+        f((int)g, tile(k), active);
+      }
     }
   }
 }
 
 // One more at tile t's counter: its value before.  Neighbouring items meet the
 // same tiles, so a warp's equal tiles go in one atomic (2.3M pairs: 19 us, 65
-// us with an atomic each); the lanes of a large rectangle never share one
-// (8.6M pairs, mostly of large ones: 246 -> 131 us without the matching).
+// us with an atomic each).  The lanes of a large rectangle never share one, and
+// from kHugeSpread tiles on go without the matching (8.6M pairs, most of
+// rectangles of 1400 tiles: 206 -> 131 us; below, where queued rectangles of a
+// few rounds crowd the same tiles, it was slower: 175 -> 203 us for 12.6M pairs
+// of 8 views).
 __device__ __forceinline__ uint32_t count_tile(uint32_t* __restrict__ counter, uint32_t t, unsigned active) {
-  return active ? warp_agg_inc(counter, t, active) : atomicAdd(&counter[t], 1u);
+  return warp_agg_inc(counter, t, active);
+}
+__device__ __forceinline__ uint32_t count_tile(uint32_t* __restrict__ counter, uint32_t t, Distinct) {
+  return atomicAdd(&counter[t], 1u);
 }
 
 // Every (item, tile) pair adds one to its tile's counter (when the
@@ -136,7 +151,7 @@ __device__ __forceinline__ uint32_t count_tile(uint32_t* __restrict__ counter, u
 __global__ void __launch_bounds__(kBinThreads) tile_count_kernel(const __grid_constant__ TileBinArgs a) {
   pdl_enter();
   for_each_pair(a.n, a.rects, a.tiles, a.map, a.big_queue, a.big_len,
-                [&](int, uint32_t t, unsigned active) {
+                [&](int, uint32_t t, auto active) {
                   // (the checked build counts a tile beyond the grid into tile 0, reported)
                   count_tile(a.counts, in_bounds(t < (uint32_t)a.n_tiles) ? t : 0u, active);
                 });
@@ -427,7 +442,7 @@ __global__ void __launch_bounds__(kBinThreads) tile_scatter_kernel(const __grid_
   pdl_enter();
   bool over = false;
   for_each_pair<ITEMS>(a.n, a.rects, a.tiles, a.map, a.big_queue, a.big_len,
-                       [&](int g, uint32_t t, unsigned active) {
+                       [&](int g, uint32_t t, auto active) {
                          const uint32_t pos = count_tile(a.cursors, in_bounds(t < (uint32_t)a.n_tiles) ? t : 0u, active);
                          if (pos < a.capacity)
                            a.ids[pos] = (uint32_t)g;
