@@ -139,6 +139,9 @@ struct gs_ctx {
   uint32_t* cls_tiles = nullptr;  // kLenClasses * cap_bt
   int64_t cap_bt = 0;
   int64_t longest_seen = 0;
+  // of the last sync-mode binning (0: not known), for the raster passes' regions
+  int64_t seen_pairs = 0, seen_longest = 0;
+  int st_ppl = 4;  // pixels per lane of the last forward pass
   bool bucket_ok = false;
   bool st_buckets = false;        // the last forward pass binned into the buckets
   // long lists cut to their nearest entries (prefix.cu, sync mode)
@@ -761,6 +764,8 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
     // has seen fits half of one; a bucket holds twice the longest of them,
     // rounded up to a power of two (at least kBucketCapMin)
     c->longest_seen = std::max(c->longest_seen, longest);
+    c->seen_pairs = P;
+    c->seen_longest = longest;
     tb.longest = (uint32_t)std::min<int64_t>(longest, 0xFFFFFFFFll);
     int64_t entries = kBucketCapMin;
     while (entries < 2 * c->longest_seen && entries < (int64_t)kBucketCapMax) entries *= 2;
@@ -1186,6 +1191,7 @@ RasterArgs raster_args(gs_ctx* c, const gs_raster_cfg* cfg) {
   ra.persistent = c->persistent;
   ra.num_sms = c->num_sms;
   ra.loss_partials = nullptr;
+  ra.px_per_lane = c->st_ppl;
   ra.w_color = 0.f;
   ra.depth_scale = nullptr;
   ra.nvalid = nullptr;
@@ -1298,6 +1304,8 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   c->st_tiles = L.tiles;
   c->st_map = L.map;
   c->st_sh = g->sh_degree;
+  c->st_ppl = raster_px_per_lane((uint32_t)c->st_tiles, c->num_sms, c->st_cut ? 0 : c->seen_pairs,
+                                 c->st_cut ? 0 : c->seen_longest);
 
   for (int attempt = 0;; ++attempt) {
   RasterArgs ra = raster_args(c, cfg);
@@ -1488,7 +1496,7 @@ gs_status render_bwd_adam_views(gs_ctx* c, const gs_gaussians* g, int32_t V, con
     }
     LossFoldArgs L{};
     if (lf) {  // the forward pass's loss partials (per tile and warp job)
-      const int64_t jobs = raster_jobs_per_tile((uint32_t)c->st_tiles, c->num_sms);
+      const int64_t jobs = 8 / c->st_ppl;
       L.partials = c->tile_loss;
       L.blk = c->loss_partials;
       L.out = lf->loss;

@@ -316,8 +316,9 @@ struct RasterArgs {
   int num_sms;
   // fused loss (forward): per warp job partial sums {|colour residual|,
   // |depth residual| over valid targets, valid count} at
-  // loss_partials[3 (raster_jobs_per_tile tile + job) + i]; null = no loss
+  // loss_partials[3 (8 / px_per_lane * tile + job) + i]; null = no loss
   float* loss_partials;
+  int px_per_lane;  // 4, 2 or 1: a tile has 8 / px_per_lane jobs
   float w_color;
   // backward: dL/dD = dLdd * depth_scale[v] when non-null (the scale the
   // fused loss finalises on the device)
@@ -342,8 +343,7 @@ struct RasterArgs {
 bool raster_shape_supported(int tw, int th);
 // pixels per lane of the raster passes (4, 2 or 1) and the warp jobs (regions
 // of 32 px per lane pixels, one loss partial each) that a tile then has
-int raster_px_per_lane(uint32_t n_tiles, int num_sms);
-inline int raster_jobs_per_tile(uint32_t n_tiles, int num_sms) { return 8 / raster_px_per_lane(n_tiles, num_sms); }
+int raster_px_per_lane(uint32_t n_tiles, int num_sms, int64_t pairs, int64_t longest);
 constexpr int kMaxTileJobs = 8;
 // bounds-checked build: point the translation unit's kernels at the
 // context's bounds word (no-op in the normal build)

@@ -372,7 +372,7 @@ void launch_loss_tiles_finalize(const RasterArgs& a, float w_depth, float* loss,
   la.w_depth = w_depth;
   la.loss = loss;
   int blocks = 0;
-  const uint32_t jobs = (uint32_t)raster_jobs_per_tile(a.n_tiles, a.num_sms);
+  const uint32_t jobs = (uint32_t)(8 / a.px_per_lane);
   for (int v = 0; v < a.views; ++v) {
     const uint32_t j0 = jobs * a.v[v].tile_base;
     const uint32_t j1 = jobs * (v + 1 < a.views ? a.v[v + 1].tile_base : a.n_tiles);

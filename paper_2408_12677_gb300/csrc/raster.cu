@@ -1044,7 +1044,7 @@ void fwd_launch(const RasterArgs& a, const RasterParams& rp, float* T_final, int
 template <int TW, int TH, bool COUNT, bool LOSS>
 void fwd_shape(const RasterArgs& a, const RasterParams& rp, float* T_final, int32_t* last,
                unsigned long long* counters, cudaStream_t s) {
-  switch (raster_px_per_lane(a.n_tiles, a.num_sms)) {
+  switch (a.px_per_lane) {
     case 4: fwd_launch<TW, TH, 4, COUNT, LOSS>(a, rp, T_final, last, counters, s); break;
     case 2: fwd_launch<TW, TH, 2, COUNT, LOSS>(a, rp, T_final, last, counters, s); break;
     default: fwd_launch<TW, TH, 1, COUNT, LOSS>(a, rp, T_final, last, counters, s); break;
@@ -1072,7 +1072,7 @@ void bwd_launch(const RasterArgs& a, const RasterParams& rp, const float* T_fina
 template <int TW, int TH>
 void bwd_shape(const RasterArgs& a, const RasterParams& rp, const float* T_final, const int32_t* last, float* g2d,
                cudaStream_t s) {
-  switch (raster_px_per_lane(a.n_tiles, a.num_sms)) {
+  switch (a.px_per_lane) {
     case 4: bwd_launch<TW, TH, 4>(a, rp, T_final, last, g2d, s); break;
     case 2: bwd_launch<TW, TH, 2>(a, rp, T_final, last, g2d, s); break;
     default: bwd_launch<TW, TH, 1>(a, rp, T_final, last, g2d, s); break;
@@ -1088,9 +1088,16 @@ void bwd_shape(const RasterArgs& a, const RasterParams& rp, const float* T_final
 // forward + backward us at 4 / 2 / 1 pixels per lane: 80 tiles 55 / 48 / 44,
 // 300 tiles 55 / 49 / 54, 690 tiles 66 / 62 / 88, 1200 tiles 83 / 87 / 131,
 // 1908 tiles 97 / 108 / 176.
-int raster_px_per_lane(uint32_t n_tiles, int num_sms) {
-  const uint32_t sms = (uint32_t)std::max(num_sms, 1);
-  return n_tiles >= 6 * sms ? 4 : n_tiles >= sms ? 2 : 1;
+int raster_px_per_lane(uint32_t n_tiles, int num_sms, int64_t pairs, int64_t longest) {
+  const int64_t sms = std::max(num_sms, 1), warps = sms * kFwdCtas * kThreads / 32;
+  int ppl = n_tiles >= 6 * sms ? 4 : n_tiles >= sms ? 2 : 1;
+  // A warp walks its list alone: where the longest is several times a warp's
+  // share of all (a few tiles whose pixels do not stop), the pass takes as long
+  // as that walk, and smaller regions make it shorter: 8 views of 234k Gaussians
+  // with lists of 334 and one of 15804, forward + backward 2782 -> 1919 us.
+  // Lists below 1024 end soon enough.
+  while (ppl > 1 && longest >= 1024 && longest * warps > 4 * pairs * (8 / ppl)) ppl /= 2;
+  return ppl;
 }
 
 void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsigned long long* counters,
