@@ -1,5 +1,7 @@
 // Projection of 3D Gaussians to 2D splats (Eq. 2-5) and its backward pass,
 // including the gradient w.r.t. the camera pose.
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -735,32 +737,50 @@ __device__ __forceinline__ void adam_update(float& p, float g, float& m, float& 
 }
 
 // Backward of the projection fused with the Adam step, for one optimisation
-// iteration on one view.  A block (one warp) owns 32 consecutive Gaussians:
+// iteration on a batch of views.  A block (one warp) owns 32 consecutive
+// Gaussians:
 //   1. its slices of the parameter array and of the two Adam moments (each
 //      slice contiguous in the flat layout) are copied to shared memory with
 //      cp.async, the parameters as a first group and the moments as a second,
 //      so the moment loads stay in flight during step 2;
-//   2. one thread per Gaussian turns its gradient record into parameter
-//      gradients, kept in shared memory, the SH gradient in factored form (Y_k *
-//      graw_c);
+//   2. one thread per Gaussian turns its gradient records (one per view)
+//      into parameter gradients summed over the views, kept in shared memory;
 //   3. coalesced sweeps apply Adam to every float and store p, m, v.
-// No gradient buffer is written or read.  Blocks of one warp (27 KB, 8 blocks
-// per SM) let the staging, gradient and sweep phases of different blocks
-// overlap.
-constexpr int kFusedThreads = 32;
-static_assert(kFusedThreads == 32, "the fused loss reduction takes one warp per block");
+// No gradient buffer is written or read.  With one view the SH gradient is
+// kept in factored form (Y_k * graw_c) and the SH moments are staged too;
+// with several views the SH gradients are summed in shared memory rows and
+// the SH moments are staged as well, beside the summed rows.  Blocks of one
+// warp (27 KB for one view, 8 blocks per SM) let the staging, gradient and
+// sweep phases of different blocks overlap.
+template <bool MULTI>
+constexpr int fused_threads() { return 32; }
+static_assert(fused_threads<false>() == 32 && fused_threads<true>() == 32,
+              "the fused loss reduction takes one warp per block");
 
 template <int D>
 struct FusedSmem {
   static constexpr int K = (D + 1) * (D + 1);
   static constexpr int NS = 3 * K;
   static constexpr int RS = (NS % 2 == 0) ? NS + 1 : NS;  // odd row stride: conflict-free per-thread rows
-  static constexpr int B = kFusedThreads;
+  static constexpr int B = fused_threads<false>();
   float p[B * 11], m[B * 11], v[B * 11];  // means (3B) | log-scales (3B) | quats (4B) | logits (B)
   float g[B * 11];                        // gradients, same layout
   float sp[B * RS], sm[B * NS + 4], sv[B * NS + 4];  // SH moments at their slice's offset within 16 B
   float Y[B][K + 1];
   float graw[B][4];
+};
+
+template <int D>
+struct FusedSmemMulti {
+  static constexpr int K = (D + 1) * (D + 1);
+  static constexpr int NS = 3 * K;
+  static constexpr int RS = (NS % 2 == 0) ? NS + 1 : NS;
+  static constexpr int B = fused_threads<true>();
+  float p[B * 11], m[B * 11], v[B * 11];
+  float g[B * 11];
+  float sp[B * RS];  // SH parameters, one row per Gaussian
+  float gs[B * RS];  // SH gradients summed over the views, same rows
+  float sm[B * NS + 4], sv[B * NS + 4];  // SH moments
 };
 
 // The training step's loss reduction (see LossFoldArgs), by one warp per
@@ -823,17 +843,17 @@ __device__ __forceinline__ void fused_loss_reduce(const LossFoldArgs& L) {
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(kFusedThreads) project_bwd_adam_kernel(const __grid_constant__ ProjectArgs a,
+template <int D, bool MULTI>
+__global__ void __launch_bounds__(fused_threads<MULTI>()) project_bwd_adam_kernel(const __grid_constant__ ProjectArgs a,
                                                                          float4* __restrict__ g2d,
                                                                          float* __restrict__ P, float* __restrict__ M,
                                                                          float* __restrict__ V, AdamArgs ad,
                                                                          float* __restrict__ pose_partials,
                                                                          const __grid_constant__ LossFoldArgs L) {
   pdl_enter();
-  if (L.out && threadIdx.x < 32) fused_loss_reduce(L);  // one warp's work  // blocks of one warp: the whole block
+  if (L.out && threadIdx.x < 32) fused_loss_reduce(L);  // blocks of one warp: the whole block
   device_bias_corrections(ad);
-  using S = FusedSmem<D>;
+  using S = typename std::conditional<MULTI, FusedSmemMulti<D>, FusedSmem<D>>::type;
   constexpr int K = S::K, NS = S::NS, RS = S::RS, B = S::B;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   S& sm = *reinterpret_cast<S*>(smem_raw);
@@ -888,30 +908,51 @@ __global__ void __launch_bounds__(kFusedThreads) project_bwd_adam_kernel(const _
     for (int j = 0; j < 4; ++j) q4[j] = sm.p[6 * B + 4 * t + j];
   }
   float am[3] = {0.f, 0.f, 0.f}, als[3] = {0.f, 0.f, 0.f}, aq[4] = {0.f, 0.f, 0.f, 0.f}, alog = 0.f;
-  float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (t < cnt) {
-    GaussGrad<D> gg;
-    const bool nz = nonzero_record(G0, G1, G2);
-    if (nz) {
-      const float* row = sm.sp + t * RS;
-      gaussian_grad<D>(a.cv[0], a.dilation, pq, q4, ls, sm.p[10 * B + t], row, G0, G1, G2, gg);
-      alog = gg.glogit;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        am[c] = gg.gm[c];
-        als[c] = gg.gls[c];
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) aq[j] = gg.gq[j];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) pose[k] = gg.pose[k];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) sm.graw[t][c] = nz ? gg.graw[c] : 0.f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) sm.Y[t][k] = nz ? gg.Y[k] : 0.f;
+  if constexpr (MULTI) {
+    if (t < cnt)
+      for (int e = 0; e < NS; ++e) sm.gs[t * RS + e] = 0.f;
   }
-  if (pose_partials) block_pose_partial(pose, pose_partials + (size_t)blockIdx.x * 6);
+  for (int v = 0; v < (MULTI ? a.views : 1); ++v) {  // the one-view variant runs for one view only
+    float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (t < cnt) {
+      if (v > 0) {
+        const int64_t it = (int64_t)v * N + base + t;
+        G0 = g2d[3 * it];
+        G1 = g2d[3 * it + 1];
+        G2 = g2d[3 * it + 2];
+        if (nonzero_record(G0, G1, G2)) zero_record(g2d + 3 * it);
+      }
+      GaussGrad<D> gg;
+      const bool nz = nonzero_record(G0, G1, G2);
+      if (nz) {
+        gaussian_grad<D>(a.cv[v], a.dilation, pq, q4, ls, sm.p[10 * B + t], sm.sp + t * RS, G0, G1, G2, gg);
+        alog += gg.glogit;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          am[c] += gg.gm[c];
+          als[c] += gg.gls[c];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) aq[j] += gg.gq[j];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) pose[k] = gg.pose[k];
+      }
+      if constexpr (MULTI) {
+        if (nz) {
+#pragma unroll
+          for (int k = 0; k < K; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sm.gs[t * RS + 3 * k + c] += gg.Y[k] * gg.graw[c];
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sm.graw[t][c] = nz ? gg.graw[c] : 0.f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) sm.Y[t][k] = nz ? gg.Y[k] : 0.f;
+      }
+    }
+    if (pose_partials) block_pose_partial(pose, pose_partials + ((size_t)blockIdx.x * a.views + v) * 6);
+  }
   if (t < cnt) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -939,60 +980,83 @@ __global__ void __launch_bounds__(kFusedThreads) project_bwd_adam_kernel(const _
       V[f] = v;
     }
   }
-  // walk the SH rows, lane t on columns t, t + 32, ... (coalesced rows, and each
-  // lane's coefficient (k, c) fixed per column)
+  if constexpr (B == 32) {
+    // a warp per block: walk the SH rows, lane t on columns t, t + 32, ...
+    // (coalesced rows, and each lane's coefficient (k, c) fixed per column)
 #pragma unroll
-  for (int c0 = 0; c0 < NS; c0 += B) {
-    const int rr = c0 + t;
-    if (rr < NS) {
-      const int k = rr / 3, c = rr - 3 * k;
-      const float lr = k == 0 ? ad.lr[4] : ad.lr[5];
-      for (int gi = 0; gi < cnt; ++gi) {
-        const int e = gi * NS + rr;
-        float p = sm.sp[gi * RS + rr], m = sm.sm[shM + e], v = sm.sv[shV + e];
-        adam_update(p, sm.Y[gi][k] * sm.graw[gi][c], m, v, lr, ad);
-        const int64_t f = gsh + e;
-        P[f] = p;
-        M[f] = m;
-        V[f] = v;
+    for (int c0 = 0; c0 < NS; c0 += B) {
+      const int rr = c0 + t;
+      if (rr < NS) {
+        const int k = rr / 3, c = rr - 3 * k;
+        const float lr = k == 0 ? ad.lr[4] : ad.lr[5];
+        for (int gi = 0; gi < cnt; ++gi) {
+          const int e = gi * NS + rr;
+          float p = sm.sp[gi * RS + rr], m = sm.sm[shM + e], v = sm.sv[shV + e];
+          float g;
+          if constexpr (MULTI)
+            g = sm.gs[gi * RS + rr];
+          else
+            g = sm.Y[gi][k] * sm.graw[gi][c];
+          adam_update(p, g, m, v, lr, ad);
+          const int64_t f = gsh + e;
+          P[f] = p;
+          M[f] = m;
+          V[f] = v;
+        }
       }
+    }
+  } else {
+    for (int e = t; e < cnt * NS; e += B) {
+      const int gi = e / NS, rr = e - gi * NS;
+      const int k = rr / 3, c = rr - 3 * k;
+      const int64_t f = gsh + e;
+      float p = sm.sp[gi * RS + rr], m = sm.sm[shM + e], v = sm.sv[shV + e], g;
+      if constexpr (MULTI)
+        g = sm.gs[gi * RS + rr];
+      else
+        g = sm.Y[gi][k] * sm.graw[gi][c];
+      adam_update(p, g, m, v, k == 0 ? ad.lr[4] : ad.lr[5], ad);
+      P[f] = p;
+      M[f] = m;
+      V[f] = v;
     }
   }
 }
 
-// The same for several views: a block owns kMultiB consecutive Gaussians, one
-// per thread, whose gradient records (one per view) are turned into parameter
-// gradients summed over the views in shared memory.  The parameters are staged,
-// the SH slice in 16-byte pieces of the global array whatever the slice's own
-// alignment; the moments are on their way to L2 meanwhile and go from there to
-// registers and back in float4 (all but the pieces that the slice shares with
-// its neighbours).  Bound by the views' gradients (900 instructions per visible
-// item) beside HBM: staging the moments too, 32 Gaussians per block, left 5
-// blocks of one warp per SM (489 us for 5 views of 2^20 slots, 381 us for 8
-// views of 500k); now 6 blocks of two warps with 165 registers (427, 316 us).
-// For one view, where the staged form has 8 blocks, it is the faster one (91
-// against 96 us for 300k).
+// The same for several views of a large map with degree-3 SH: a block owns
+// kMultiB consecutive Gaussians, one per thread, whose gradient records (one per
+// view) are turned into parameter gradients summed over the views in shared
+// memory.  The parameters are staged, the SH slice in 16-byte pieces of the global array
+// whatever the slice's own alignment; the moments are on their way to L2
+// meanwhile and go from there to registers and back in float4 (all but the
+// pieces that the slice shares with its neighbours).  Bound by the views'
+// gradients (900 instructions per visible item) beside HBM: staging the moments
+// too, 32 Gaussians per block, leaves 5 blocks of one warp per SM (489 us for 5
+// views of 2^20 slots, 381 us for 8 views of 500k); this form has 6 blocks of
+// two warps with 165 registers (427, 316 us).  Where the staged form has 8 blocks
+// of one warp (one view, lower degrees) or the map is in L2 it is the faster one
+// (staged / this form: one view of 300k 91 / 96 us; degree 1, 5 views of 300k 94 /
+// 113; degree 3, 5 views of 60k 45 / 51, 100k 66 / 64, 300k 179 / 157; 2 views of
+// 150k 64 / 66, 220k 87 / 84).
+constexpr int kMultiN = 200000;  // Gaussians from which it is taken
 constexpr int kMultiB = 64;  // Gaussians and threads of a block
 
 // The SH slice of a block in pieces of four floats aligned in the global
 // array: piece c holds the slice's floats 4 c - shift .. 4 c - shift + 3, shift
-// = the slice's place within 16 bytes.  Rows whose length is a multiple of 4
-// floats are kept 4 floats apart in shared memory (a thread reads its own row:
-// 4-way bank conflicts instead of 16-way); pieces keep their 16-byte alignment.
+// = the slice's place within 16 bytes.  Rows are kept 4 floats apart in shared
+// memory (a thread reads its own row: 4-way bank conflicts instead of 16-way);
+// pieces keep their 16-byte alignment.
 template <int D>
 struct ShRows {
   static constexpr int K = (D + 1) * (D + 1);
   static constexpr int NS = 3 * K;
-  static constexpr bool kPad = NS % 4 == 0;
-  static constexpr int RS = kPad ? NS + 4 : NS;
+  static constexpr int RS = NS + 4;
   static constexpr int WORDS = (kMultiB + 1) * RS + 8;
+  static_assert(NS % 4 == 0, "a row is whole pieces");
   // shared-memory word of piece c's first float
-  static __device__ __forceinline__ int piece(int c) {
-    return kPad ? (c / (NS / 4)) * RS + 4 * (c % (NS / 4)) : 4 * c;
-  }
+  static __device__ __forceinline__ int piece(int c) { return (c / (NS / 4)) * RS + 4 * (c % (NS / 4)); }
   // shared-memory word of float rr of row t
   static __device__ __forceinline__ int word(int t, int rr, int shift) {
-    if constexpr (!kPad) return t * NS + rr + shift;
     const int q = rr + shift;
     return q < NS ? t * RS + q : (t + 1) * RS + q - NS;
   }
@@ -1275,42 +1339,41 @@ int launch_project_bwd(const ProjectArgs& a, float4* g2d, float* g_means, float*
 int launch_project_bwd_adam(const ProjectArgs& a, float4* g2d, float* params, float* m, float* v,
                             const AdamArgs& ad, float* pose_partials, cudaStream_t s, const LossFoldArgs* loss) {
   if (a.n <= 0) return 0;
-  const int bt = a.views == 1 ? kFusedThreads : kMultiB;
+  const bool wide = a.views > 1 && a.sh_degree == 3 && a.n >= kMultiN;
+  const int bt = wide ? kMultiB : fused_threads<false>();
   const int nb = (a.n + bt - 1) / bt;
   LossFoldArgs L{};
   if (loss) L = *loss;
-#define GS_FUSED(K_, D_, S_) \
-  launch_pdl(K_<D_>, nb, bt, sizeof(S_<D_>), s, a, g2d, params, m, v, ad, pose_partials, L)
-  if (a.views == 1) {
-    switch (a.sh_degree) {
-      case 0: GS_FUSED(project_bwd_adam_kernel, 0, FusedSmem); break;
-      case 1: GS_FUSED(project_bwd_adam_kernel, 1, FusedSmem); break;
-      case 2: GS_FUSED(project_bwd_adam_kernel, 2, FusedSmem); break;
-      default: GS_FUSED(project_bwd_adam_kernel, 3, FusedSmem); break;
-    }
-  } else {
-    switch (a.sh_degree) {
-      case 0: GS_FUSED(project_bwd_adam_multi_kernel, 0, MultiSmem); break;
-      case 1: GS_FUSED(project_bwd_adam_multi_kernel, 1, MultiSmem); break;
-      case 2: GS_FUSED(project_bwd_adam_multi_kernel, 2, MultiSmem); break;
-      default: GS_FUSED(project_bwd_adam_multi_kernel, 3, MultiSmem); break;
-    }
+#define GS_FUSED(K_, S_) launch_pdl(K_, nb, bt, sizeof(S_), s, a, g2d, params, m, v, ad, pose_partials, L)
+#define GS_FUSED_DEG(M_, S_)                                                       \
+  switch (a.sh_degree) {                                                           \
+    case 0: GS_FUSED((project_bwd_adam_kernel<0, M_>), S_<0>); break;              \
+    case 1: GS_FUSED((project_bwd_adam_kernel<1, M_>), S_<1>); break;              \
+    case 2: GS_FUSED((project_bwd_adam_kernel<2, M_>), S_<2>); break;              \
+    default: GS_FUSED((project_bwd_adam_kernel<3, M_>), S_<3>); break;             \
   }
+  if (wide) GS_FUSED(project_bwd_adam_multi_kernel<3>, MultiSmem<3>);
+  else if (a.views == 1) GS_FUSED_DEG(false, FusedSmem)
+  else GS_FUSED_DEG(true, FusedSmemMulti)
+#undef GS_FUSED_DEG
 #undef GS_FUSED
   return nb;
 }
 
 void init_project_kernels() {
-#define GS_ATTR(K_, D_, S_) \
-  cudaFuncSetAttribute(K_<D_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(S_<D_>))
-  GS_ATTR(project_bwd_adam_kernel, 0, FusedSmem);
-  GS_ATTR(project_bwd_adam_kernel, 1, FusedSmem);
-  GS_ATTR(project_bwd_adam_kernel, 2, FusedSmem);
-  GS_ATTR(project_bwd_adam_kernel, 3, FusedSmem);
-  GS_ATTR(project_bwd_adam_multi_kernel, 0, MultiSmem);
-  GS_ATTR(project_bwd_adam_multi_kernel, 1, MultiSmem);
-  GS_ATTR(project_bwd_adam_multi_kernel, 2, MultiSmem);
-  GS_ATTR(project_bwd_adam_multi_kernel, 3, MultiSmem);
+#define GS_ATTR(D_, M_, S_)                                                                           \
+  cudaFuncSetAttribute(project_bwd_adam_kernel<D_, M_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       (int)sizeof(S_<D_>))
+  GS_ATTR(0, false, FusedSmem);
+  GS_ATTR(1, false, FusedSmem);
+  GS_ATTR(2, false, FusedSmem);
+  GS_ATTR(3, false, FusedSmem);
+  GS_ATTR(0, true, FusedSmemMulti);
+  GS_ATTR(1, true, FusedSmemMulti);
+  GS_ATTR(2, true, FusedSmemMulti);
+  GS_ATTR(3, true, FusedSmemMulti);
+  cudaFuncSetAttribute(project_bwd_adam_multi_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)sizeof(MultiSmem<3>));
 #undef GS_ATTR
 }
 
