@@ -1093,10 +1093,12 @@ int raster_px_per_lane(uint32_t n_tiles, int num_sms, int64_t pairs, int64_t lon
   int ppl = n_tiles >= 6 * sms ? 4 : n_tiles >= sms ? 2 : 1;
   // A warp walks its list alone: where the longest is several times a warp's
   // share of all (a few tiles whose pixels do not stop), the pass takes as long
-  // as that walk, and smaller regions make it shorter: 8 views of 234k Gaussians
-  // with lists of 334 and one of 15804, forward + backward 2782 -> 1919 us.
-  // Lists below 1024 end soon enough.
-  while (ppl > 1 && longest >= 1024 && longest * warps > 4 * pairs * (8 / ppl)) ppl /= 2;
+  // as that walk, and smaller regions make it shorter.  Lists below 1024 end
+  // soon enough.  Not down to one pixel per lane: that has twice the additions
+  // to each gradient record, and a larger rounding error for it.  8 views of
+  // 234k Gaussians with lists of 334 and one of 15804, forward + backward: 2782
+  // us with four pixels per lane, 2237 with two.
+  if (ppl == 4 && longest >= 1024 && longest * warps > 8 * pairs) ppl = 2;
   return ppl;
 }
 
