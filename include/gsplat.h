@@ -171,9 +171,9 @@ gs_status gs_ctx_set_adam_step(gs_ctx *ctx, int64_t step);
 gs_status gs_ctx_set_tile_order(gs_ctx *ctx, int on);
 
 /* on = 1 (default): each raster pass is one persistent launch of as many
- * CTAs as the GPU holds at once, whose warps pull (tile, 8 x 8 pixel block)
- * jobs from a device counter in the visit order above, for all views of a
- * batch.  on = 0: one CTA per tile.  Results do not depend on it. */
+ * CTAs as the GPU holds at once, whose warps pull (tile, pixel region) jobs
+ * from a device counter in the visit order above, for all views of a batch.
+ * on = 0: a grid of one warp per job.  Results do not depend on it. */
 gs_status gs_ctx_set_persistent(gs_ctx *ctx, int on);
 
 /* Synchronise the stream, then report GS_ERR_BOUNDS if the bounds-checked
@@ -226,8 +226,8 @@ gs_status gs_render_fwd(gs_ctx *ctx, const gs_gaussians *g, const gs_camera *cam
  * (e.g. two renders at two poses followed by the backward pass of the first).
  * The parameter VALUES are not compared: changing them in place between the
  * forward and the backward pass is the caller's error.  Walks every tile list back to
- * front from the stored last contributor, recomputing transmittance from the
- * stored final T.  dL_dcolor [3, H, W] and dL_ddepth [H, W] are required,
+ * front from the pixel's stored last list entry, recomputing transmittance
+ * from the stored final T.  dL_dcolor [3, H, W] and dL_ddepth [H, W] are required,
  * dL_dalpha [H, W] may be NULL.  Gradients w.r.t. every parameter array are
  * ADDED to `grads` (the caller zeroes them).  dL_dpose (device float[6],
  * nullable) receives += the gradient w.r.t. xi = (rho, phi) of the left
@@ -623,7 +623,8 @@ gs_status gs_get_tile_ranges(gs_ctx *ctx, uint32_t *ranges, int64_t n_tiles, gs_
  * empty list, else 4 floor(log2 len) + the two bits after len's leading one
  * + 1); n_tiles must be the forward pass's tile count.  GS_ERR_STATE when
  * that pass visited the tiles in index order (gs_ctx_set_tile_order(0), or
- * the radix binning of very long lists).  For checks of the binning. */
+ * the radix binning of very long lists, or lists cut to their nearest entries
+ * by a sync-mode pass).  For checks of the binning. */
 gs_status gs_get_tile_order(gs_ctx *ctx, uint32_t *order, int64_t n_tiles, gs_stream_t stream);
 
 #ifdef __cplusplus
