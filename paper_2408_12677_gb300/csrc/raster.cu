@@ -100,6 +100,10 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 // about 5 ns an addition (32 per tile).
 constexpr float kWide = 512.f * 256.f / 4.f;
 
+// log2 opacity in place of a NaN (others are at most 0): alpha is over alpha_max
+// up to the support's edge, where q' = 6.5.
+constexpr float kNanOpacity = 64.f;
+
 // Converts a gathered record to tile-local coordinates and tests the splat's
 // support bounding box against the blocks of the warp's region, whose first
 // pixel is (bx, by): bit l of the result is set when the box meets the pixel
@@ -108,7 +112,9 @@ constexpr float kWide = 512.f * 256.f / 4.f;
 // (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents sqrt(R2) / i0 and
 // sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2); the widening covers float32 rounding
 // of the test and of the hardware square roots and reciprocals.  `wide`: the
-// box has more than 4 kWide pixels.
+// box has more than 4 kWide pixels.  A NaN opacity (fminf passes it over in R2
+// and here) becomes one that is clamped wherever the splat reaches: the raster
+// loops multiply alpha by 0 outside the support, which a NaN would survive.
 template <class M>
 __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, float ox, float oy, float bx, float by,
                                                const RasterParams& rp, uint32_t id, Entry& e, bool& wide) {
@@ -117,7 +123,7 @@ __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, 
   const float mly = __fadd_rn(__fsub_rn(f0.y, oy), f0.w);
   const float R2 = fminf(rp.qmax_s, __fsub_rn(f1.w, rp.log2_alpha_min));
   e.a = make_float4(mlx, mly, f1.x, -f1.y);
-  e.b = make_float4(f1.z, f1.w, f2.w, R2);
+  e.b = make_float4(f1.z, fminf(f1.w, kNanOpacity), f2.w, R2);
   e.c = make_float4(f2.x, f2.y, f2.z, __uint_as_float(id));
   if (!(R2 > 0.f && f1.x > 0.f && f1.z > 0.f)) return 0u;
   const float Rr = sqrt_approx(R2) * 1.0001f + 1e-4f;
