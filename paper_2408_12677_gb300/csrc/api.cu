@@ -160,7 +160,7 @@ struct gs_ctx {
   const uint32_t* pfx_sorted = nullptr;  // items by depth (of the current pass)
   bool st_cut = false;            // the last forward pass's lists are cut (tcount, toffset: the full ones)
   int* big_diff = nullptr;        // difference grids of the projection's large rectangles, 0 between passes
-  int64_t cap_big = 0;
+                                  // (part of tcount's allocation)
   bool order_tiles = true;  // compute and use the visit order
   bool persistent = true;   // raster passes as persistent grids pulling (tile, quadrant) jobs
   int st_sh = 0;
@@ -308,25 +308,6 @@ gs_status ensure_buckets(gs_ctx* c, int64_t t, uint32_t entries) {
   return GS_OK;
 }
 
-gs_status ensure_tiles(gs_ctx* c, int64_t t) {
-  if (t <= c->cap_t) return GS_OK;
-  if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
-  GS_CUDA(c, cudaDeviceSynchronize());
-  const int64_t cap = grow_target(t, c->cap_t);
-  GS_GROW(c, cap_t, regrow(&c->ranges, cap));
-  GS_GROW(c, cap_t, regrow(&c->tcount, cap));
-  c->counts_zero = false;
-  GS_GROW(c, cap_t, regrow(&c->toffset, cap));
-  GS_GROW(c, cap_t, regrow(&c->tcursor, cap));
-  GS_GROW(c, cap_t, regrow(&c->torder, cap));
-  GS_GROW(c, cap_t, regrow(&c->tlong, cap));
-  GS_GROW(c, cap_t, regrow(&c->scan_aux, tile_scan_aux_size(cap)));
-  GS_GROW(c, cap_t, regrow(&c->tile_loss, 3 * kMaxTileJobs * cap));
-  c->cap_t = cap;
-  c->have_state = false;
-  return GS_OK;
-}
-
 // Cells of the views' difference grids ((tiles_x + 1) x (tiles_y + 1) each, end
 // to end), their first cells in base[].
 int64_t grid_layout(const TileMap& map, const int* tiles_y, uint32_t* base) {
@@ -338,14 +319,30 @@ int64_t grid_layout(const TileMap& map, const int* tiles_y, uint32_t* base) {
   return cells;
 }
 
-gs_status ensure_big(gs_ctx* c, int64_t cells) {
-  if (cells <= c->cap_big) return GS_OK;
+// The most cells that the grids of up to kMaxViews views of `tiles` tiles in
+// all can have: (x + 1) (y + 1) <= 2 x y + 2.  The grids thus grow with the
+// tiles only, never in a pass whose tiles fit (a captured graph may use them).
+int64_t big_cells(int64_t tiles) { return 2 * (tiles + kMaxViews); }
+
+gs_status ensure_tiles(gs_ctx* c, int64_t t) {
+  if (t <= c->cap_t) return GS_OK;
   if (injected_alloc_failure(c)) return fail(c, GS_ERR_OOM, "injected allocation failure");
   GS_CUDA(c, cudaDeviceSynchronize());
-  const int64_t cap = grow_target(cells, c->cap_big);
-  GS_GROW(c, cap_big, regrow(&c->big_diff, cap));
-  GS_GROW(c, cap_big, cudaMemset(c->big_diff, 0, sizeof(int) * (size_t)cap));
-  c->cap_big = cap;
+  const int64_t cap = grow_target(t, c->cap_t);
+  GS_GROW(c, cap_t, regrow(&c->ranges, cap));
+  // the counters and the difference grids behind them, which the next pass
+  // clears on its own stream
+  GS_GROW(c, cap_t, regrow(&c->tcount, cap + big_cells(cap)));
+  c->big_diff = (int*)(c->tcount + cap);
+  c->counts_zero = false;
+  GS_GROW(c, cap_t, regrow(&c->toffset, cap));
+  GS_GROW(c, cap_t, regrow(&c->tcursor, cap));
+  GS_GROW(c, cap_t, regrow(&c->torder, cap));
+  GS_GROW(c, cap_t, regrow(&c->tlong, cap));
+  GS_GROW(c, cap_t, regrow(&c->scan_aux, tile_scan_aux_size(cap)));
+  GS_GROW(c, cap_t, regrow(&c->tile_loss, 3 * kMaxTileJobs * cap));
+  c->cap_t = cap;
+  c->have_state = false;
   return GS_OK;
 }
 
@@ -931,7 +928,6 @@ gs_status gs_ctx_destroy(gs_ctx* c) {
   cudaFree(c->pfx_gather);
   cudaFree(c->pfx_rects);
   cudaFree(c->pfx_diff);
-  cudaFree(c->big_diff);
   cudaFree(c->qt_cells[0]);
   cudaFree(c->qt_cells[1]);
   cudaFree(c->qt_leaves);
@@ -1240,7 +1236,7 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   uint32_t grid_base[kMaxViews] = {};
   if (c->sync) {
     if ((st = ensure_n(c, std::max(n_items, 1))) != GS_OK || (st = ensure_px(c, L.pixels)) != GS_OK ||
-        (st = ensure_tiles(c, L.tiles)) != GS_OK || (st = ensure_big(c, grid_layout(L.map, L.tiles_y, grid_base))) != GS_OK)
+        (st = ensure_tiles(c, L.tiles)) != GS_OK)
       return st;
   } else if (n_items > c->cap_n || L.pixels > c->cap_px || L.tiles > c->cap_t) {
     return fail(c, GS_ERR_CAPACITY, "no-sync mode: reserve items/pixels first (gs_ctx_reserve)");
@@ -1256,10 +1252,10 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   pa.nvalid = fl ? c->d_nvalid : nullptr;  // zeroed by the projection for the fused loss's count
   pa.step_inc = fl ? fl->step : nullptr;
   const bool buckets = !c->sync && c->bucket_ok && (int64_t)L.tiles <= c->cap_bt;
-  // large rectangles go to the difference grids (no-sync passes count tile by
-  // tile where no sync pass has sized the grids)
-  const bool grids = !buckets && grid_layout(L.map, L.tiles_y, grid_base) <= c->cap_big;
+  // large rectangles go to the difference grids
+  const bool grids = !buckets;
   if (grids) {
+    grid_layout(L.map, L.tiles_y, grid_base);
     pa.big_diff = c->big_diff;
     for (int v = 0; v < V; ++v) pa.big_base[v] = grid_base[v];
   }
@@ -1274,8 +1270,7 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
     // also starts from zeros
     GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta, 0, sizeof(uint32_t), s));
     GS_CUDA(c, cudaMemsetAsync(c->d_bigmeta + kHugeFlag, 0, sizeof(uint32_t), s));
-    GS_CUDA(c, cudaMemsetAsync(c->tcount, 0, sizeof(uint32_t) * (size_t)c->cap_t, s));
-    if (c->big_diff) GS_CUDA(c, cudaMemsetAsync(c->big_diff, 0, sizeof(int) * (size_t)c->cap_big, s));
+    GS_CUDA(c, cudaMemsetAsync(c->tcount, 0, sizeof(uint32_t) * (size_t)(c->cap_t + big_cells(c->cap_t)), s));
   }
   c->counts_zero = false;
   {
