@@ -917,7 +917,8 @@ __device__ __forceinline__ void cta_sort_list64(uint32_t* __restrict__ ids, cons
 // sorted by that warp in registers (no barriers), the few of those whose 32-bit
 // keys do not suffice by the whole CTA; longer ones go to long_list, which
 // tile_sort_long_kernel sorts.  The kernel also zeroes each tile's counter (and
-// block 0 the large-splat queue length, and the two raster job counters),
+// block 0 the large-splat queue length, the flag of the difference grids and
+// the two raster job counters),
 // leaving them zero for the next passes.  In bucket mode each warp also files
 // its tile under its length class (see TileBinArgs).
 //
@@ -951,7 +952,7 @@ __global__ void __launch_bounds__(kSortThreads, 6) tile_sort_kernel(const uint32
   if (threadIdx.x == 0) {
     s_nlong = 0u;
     if (blockIdx.x == 0) {
-      *big_len = 0u;
+      big_len[0] = big_len[kHugeFlag] = 0u;  // (the scan has used the grids up)
       raster_work[0] = raster_work[1] = 0u;  // the raster passes' job counters
     }
   }
