@@ -54,8 +54,8 @@ struct gs_ctx {
   uint32_t* tcount = nullptr;   // per-tile pair counts
   uint32_t* toffset = nullptr;  // per-tile list offsets
   uint32_t* tcursor = nullptr;  // per-tile scatter cursors
-  uint32_t* torder = nullptr;   // raster visit order of the tiles (longest lists first)
   uint2* tlong = nullptr;       // lists for the per-tile sort's second kernel
+  uint32_t* torder = nullptr;   // raster visit order of the tiles (longest lists first; behind tlong)
   uint32_t* scan_aux = nullptr;  // multi-block tile scan scratch
   uint32_t* bigq = nullptr;     // ids of Gaussians covering more than kBigTiles tiles
   uint32_t* d_bigmeta = nullptr;  // [0] length of the large-splat queue, [1] / [2] forward / backward raster
@@ -337,8 +337,8 @@ gs_status ensure_tiles(gs_ctx* c, int64_t t) {
   c->counts_zero = false;
   GS_GROW(c, cap_t, regrow(&c->toffset, cap));
   GS_GROW(c, cap_t, regrow(&c->tcursor, cap));
-  GS_GROW(c, cap_t, regrow(&c->torder, cap));
-  GS_GROW(c, cap_t, regrow(&c->tlong, cap));
+  GS_GROW(c, cap_t, regrow(&c->tlong, cap + (cap + 1) / 2));
+  c->torder = (uint32_t*)(c->tlong + cap);
   GS_GROW(c, cap_t, regrow(&c->scan_aux, tile_scan_aux_size(cap)));
   GS_GROW(c, cap_t, regrow(&c->tile_loss, 3 * kMaxTileJobs * cap));
   c->cap_t = cap;
@@ -710,9 +710,9 @@ gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, c
 // some tile list is longer than the per-tile sort holds, by way of the lists'
 // nearest entries (bin_prefix) where tiles_y is given.  counted: the
 // projection already added every item's tiles to the (zeroed) tile
-// counters, the large rectangles' (with tiles_y) to the difference grids.
+// counters, the large rectangles' (with grids) to the difference grids.
 gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, bool counted,
-                       const int* tiles_y = nullptr) {
+                       const int* tiles_y = nullptr, bool grids = false) {
   const int64_t T = (int64_t)map.tile_base[map.views];
   c->st_cut = false;
   if (c->sync) GS_CUDA(c, cudaMemsetAsync(c->d_overflow, 0, sizeof(uint32_t), s));
@@ -740,7 +740,7 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
   tb.order = c->order_tiles ? c->torder : nullptr;
   tb.counted = counted;
   tb.scan_aux = c->scan_aux;
-  if (tiles_y) {
+  if (grids) {
     tb.big_diff = c->big_diff;
     grid_layout(map, tiles_y, tb.big_base);
     for (int v = 0; v < map.views; ++v) tb.tiles_y[v] = tiles_y[v];
@@ -900,7 +900,6 @@ gs_status gs_ctx_destroy(gs_ctx* c) {
   cudaFree(c->tcount);
   cudaFree(c->toffset);
   cudaFree(c->tcursor);
-  cudaFree(c->torder);
   cudaFree(c->tlong);
   cudaFree(c->scan_aux);
   cudaFree(c->bigq);
@@ -1252,8 +1251,9 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   pa.nvalid = fl ? c->d_nvalid : nullptr;  // zeroed by the projection for the fused loss's count
   pa.step_inc = fl ? fl->step : nullptr;
   const bool buckets = !c->sync && c->bucket_ok && (int64_t)L.tiles <= c->cap_bt;
-  // large rectangles go to the difference grids
-  const bool grids = !buckets;
+  // rectangles of more than kHugeTiles tiles go to the difference grids
+  bool grids = false;
+  for (int v = 0; v < V; ++v) grids = grids || (!buckets && (int64_t)L.map.tiles_x[v] * L.tiles_y[v] > (int64_t)kHugeTiles);
   if (grids) {
     grid_layout(L.map, L.tiles_y, grid_base);
     pa.big_diff = c->big_diff;
@@ -1284,7 +1284,7 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   if (c->counting)  // (a pass over cut lists may be repeated)
     GS_CUDA(c, cudaMemcpyAsync(c->d_evals + 2, c->d_evals, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
   if ((st = buckets ? bin_buckets(c, n_items, L.map, s)
-                    : bin_and_sort(c, n_items, L.map, s, true, grids ? L.tiles_y : nullptr)) != GS_OK)
+                    : bin_and_sort(c, n_items, L.map, s, true, L.tiles_y, grids)) != GS_OK)
     return st;
 
   c->st_n = g->n;

@@ -45,3 +45,21 @@ def test_grids_are_integrated_only_when_used():
     after = passes(small, 60)
     assert after <= before + 3.0, (before, after)
     ctx.close()
+
+
+def test_no_grids_for_views_of_few_tiles():
+    """Views of at most 1024 tiles hold no such rectangle: 5000 tiles of eight views are scanned in three launches,
+    with the projection, the scatter, the sort and the raster pass seven."""
+    ensure_built()
+    from paper_2408_12677_gb300 import abi
+    from paper_2408_12677_gb300.torch_api import Context, camera_struct
+    cam, pose = Camera(400.0, 400.0, 200.0, 200.0, 400, 400), look_at([0.1, 0.2, -0.1], [0.7, 3.0, 0.2])
+    P = workloads.random_gaussians(np.random.default_rng(8), 3000, cam, pose, 0, log_scale_range=(-6.0, -5.0))
+    ctx, model = Context(0), to_gpu_model(P)
+    img = [[torch.empty(c + (400, 400), device="cuda") for _ in range(8)] for c in ((3,), (), ())]
+    args = model.gaussians(), [camera_struct(cam)] * 8, [abi.make_viewmat(pose.R, pose.t)] * 8, abi.raster_cfg(), *img
+    abi.gs_render_fwd_batched(ctx.handle, *args)
+    before = ctx.stats()["kernel_launches"]
+    abi.gs_render_fwd_batched(ctx.handle, *args)
+    assert ctx.stats()["kernel_launches"] - before == 7
+    ctx.close()
