@@ -20,6 +20,12 @@
 // 1.96 (backward), and one reduction serves 16 Gaussians: 85 -> 64 us and
 // 168 -> 100 us at 1200 x 680 with 300k Gaussians, 811 -> 654 us and 1759 ->
 // 1110 us for five such views.
+#ifndef BWDP
+#define BWDP 4
+#endif
+#ifndef FWDP
+#define FWDP 4
+#endif
 #include <algorithm>
 #include <type_traits>
 
@@ -221,11 +227,12 @@ struct Walk {
     __syncwarp();  // the entries are stored before any lane reads them
     return warp_transpose(m, lane);
   }
-  __device__ __forceinline__ void push(unsigned mine) {  // the staged chunk's entries
+  __device__ __forceinline__ void push(unsigned mine, bool take = true) {  // the staged chunk's entries
     if (DIR > 0) {
       if (mine) met = top + 32 - __clz(mine);
       mine = __brev(mine);
     }
+    if (!take) mine = 0u;
     const int r = top - off;
     cur = r == 0 ? mine : cur;
     w1 = r == 32 ? mine : w1;
@@ -271,6 +278,27 @@ struct Walk {
     return slot;
   }
 };
+
+// Passes with one or two pixels per lane take a chunk by all lanes together where
+// most of its entries that meet the warp's region (meet) meet every block of it
+// (whole): the lanes' lists would be nearly the same, and the backward pass makes
+// one addition to a Gaussian's record per region instead of one per block.  With
+// four pixels an addition the gradients' errors against 64 bits were up to 1.75
+// times those with 64 (200 x 150, 2000 large splats; 1.03 to 1.07 for a seeded
+// map; means over 24 maps); now they are 0.97 to 1.02 times.  With one pixel per
+// lane the backward pass takes every chunk so, two entries at a time, since the
+// few warps wait for each other's exchanges: forward + backward 24 + 45 -> 24 + 40
+// us for the former, 36 + 64 -> 34 + 57 us for 5000 at 320 x 240.  Three quarters
+// or half of the entries with two pixels per lane took 75 and 80 instead of 74 us
+// an iteration on a seeded map of 20000.  Not with four, whose additions are of
+// eight pixels in large images (errors as with 64 pixels): 294 -> 295 us for 300k
+// Gaussians, 1327 -> 1340 for five views.
+template <int PPL>
+constexpr bool kTogether = PPL <= 2;
+template <int PPL>
+__device__ __forceinline__ bool together(unsigned meet, unsigned whole) {
+  return PPL == 1 ? 2 * __popc(whole) >= __popc(meet) : 8 * __popc(whole) >= 7 * __popc(meet);
+}
 
 // Slot kRing of a warp's entries: support radius -1, accepted by no pixel.
 __device__ __forceinline__ void init_warp_smem(WarpSmem& sm) {
@@ -459,12 +487,74 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
   }
   uint32_t n_blend = 0, n_visit = 0;
 
+  // one entry (each lane its own, or the same one for all), at place idx of the list
+  auto blend = [&](const Entry& en, int idx) {
+    const float4 ea = en.a, eb = en.b, ec = en.c;
+    const float dx = __fsub_rn(plx, ea.x);
+    const float t0 = __fmul_rn(ea.z, dx);
+    float al[2 * NP], in[2 * NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const f2x DY = f2_sub(f2_pack(ply[2 * p], ply[2 * p + 1]), f2_bcast(ea.y));
+      const f2x WQ = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
+      const f2x TQ = f2_mul(WQ, f2_bcast(eb.x));
+      const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ, TQ));
+      const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
+      al[2 * p] = ex2_approx(f2_lo(ARG));
+      al[2 * p + 1] = ex2_approx(f2_hi(ARG));
+      in[2 * p] = one_if_le(f2_lo(Q), eb.w);
+      in[2 * p + 1] = one_if_le(f2_hi(Q), eb.w);
+    }
+    if (eb.y > rp.log2_clamp) {
+#pragma unroll
+      for (int s = 0; s < 2 * NP; ++s) al[s] = fminf(rp.alpha_max, al[s]);
+    }
+    f2x AL[NP], TEST[NP];
+    float low = 1.f;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      // alpha, exactly 0 (so that T, R, G, B and D stay as they are) outside the support
+      AL[p] = f2_mul(f2_pack(al[2 * p], al[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
+      TEST[p] = f2_mul(T[p], f2_sub(ONE2, AL[p]));
+      low = fminf(low, fminf(f2_lo(TEST[p]), f2_hi(TEST[p])));
+    }
+    if (COUNT) {
+#pragma unroll
+      for (int s = 0; s < PPL; ++s) {
+        n_visit += eb.w > 0.f && ply[s] != kInf ? 1u : 0u;
+        n_blend += in[s] > 0.f && (s & 1 ? f2_hi(TEST[s / 2]) : f2_lo(TEST[s / 2])) >= rp.t_eps ? 1u : 0u;
+      }
+    }
+    if (low < rp.t_eps) {  // a pixel stops in front of this entry
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const bool s0 = f2_lo(TEST[p]) < rp.t_eps, s1 = f2_hi(TEST[p]) < rp.t_eps;
+        AL[p] = f2_pack(s0 ? 0.f : f2_lo(AL[p]), s1 ? 0.f : f2_hi(AL[p]));
+        TEST[p] = f2_pack(s0 ? f2_lo(T[p]) : f2_lo(TEST[p]), s1 ? f2_hi(T[p]) : f2_hi(TEST[p]));
+        ply[2 * p] = s0 ? kInf : ply[2 * p];
+        ply[2 * p + 1] = s1 ? kInf : ply[2 * p + 1];
+        stop[2 * p] = s0 ? idx : stop[2 * p];
+        stop[2 * p + 1] = s1 ? idx : stop[2 * p + 1];
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const f2x W = f2_mul(AL[p], T[p]);
+      T[p] = TEST[p];
+      R[p] = f2_fma_s(W, ec.x, R[p]);
+      G[p] = f2_fma_s(W, ec.y, G[p]);
+      B[p] = f2_fma_s(W, ec.z, B[p]);
+      D[p] = f2_fma_s(W, eb.z, D[p]);
+    }
+  };
+
   if (walk.n > 0) {
     walk.begin();
     unsigned gone = 0u;  // 1: every pixel of the lane is done
+    unsigned held = 0u;  // a chunk whose entries all lanes take together
     for (;;) {
       while (__any_sync(kFull, walk.cur == 0u && walk.off < walk.top)) walk.step();
-      const bool can = walk.can_stage();
+      const bool can = walk.can_stage() && !held;
       if (can && __any_sync(kFull, (walk.cur | gone) == 0u)) {  // a lane is dry
         bool out = true;
 #pragma unroll
@@ -474,73 +564,35 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
         gone = out ? 1u : 0u;
         unsigned m;
         bool wide;
-        walk.push(walk.stage(rp, m, wide));
+        const unsigned mine = walk.stage(rp, m, wide);
+        if constexpr (kTogether<PPL>) {
+          const unsigned whole = __ballot_sync(kFull, m == kFull);
+          if (whole) {
+            const unsigned meet = __ballot_sync(kFull, m != 0u);
+            if (together<PPL>(meet, whole)) held = meet;
+          }
+        }
+        walk.push(mine, !held);
         if (out) walk.drop();
         continue;
       }
-      const int lim = walk.limit(can);
-      if (lim == walk.kEnd) break;
-      if (lim == walk.kAgain) continue;
+      int lim = walk.end;
+      if (!held) {
+        lim = walk.limit(can);
+        if (lim == walk.kEnd) break;
+        if (lim == walk.kAgain) continue;
+      } else if (!__any_sync(kFull, walk.cur != 0u)) {
+        const Entry* e = sm.e + ((walk.top - 32) & (kRing - 1));
+        for (; held; held &= held - 1u) {
+          const int j = __ffs(held) - 1;
+          blend(e[j], walk.top - 32 + j);
+        }
+        continue;
+      }
       do {
         int idx;
         const Entry& en = sm.e[walk.take(idx)];
-        const float4 ea = en.a, eb = en.b, ec = en.c;
-        const float dx = __fsub_rn(plx, ea.x);
-        const float t0 = __fmul_rn(ea.z, dx);
-        float al[2 * NP], in[2 * NP];
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          const f2x DY = f2_sub(f2_pack(ply[2 * p], ply[2 * p + 1]), f2_bcast(ea.y));
-          const f2x WQ = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
-          const f2x TQ = f2_mul(WQ, f2_bcast(eb.x));
-          const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ, TQ));
-          const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
-          al[2 * p] = ex2_approx(f2_lo(ARG));
-          al[2 * p + 1] = ex2_approx(f2_hi(ARG));
-          in[2 * p] = one_if_le(f2_lo(Q), eb.w);
-          in[2 * p + 1] = one_if_le(f2_hi(Q), eb.w);
-        }
-        if (eb.y > rp.log2_clamp) {
-#pragma unroll
-          for (int s = 0; s < 2 * NP; ++s) al[s] = fminf(rp.alpha_max, al[s]);
-        }
-        f2x AL[NP], TEST[NP];
-        float low = 1.f;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          // alpha, exactly 0 (so that T, R, G, B and D stay as they are) outside the support
-          AL[p] = f2_mul(f2_pack(al[2 * p], al[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
-          TEST[p] = f2_mul(T[p], f2_sub(ONE2, AL[p]));
-          low = fminf(low, fminf(f2_lo(TEST[p]), f2_hi(TEST[p])));
-        }
-        if (COUNT) {
-#pragma unroll
-          for (int s = 0; s < PPL; ++s) {
-            n_visit += eb.w > 0.f && ply[s] != kInf ? 1u : 0u;
-            n_blend += in[s] > 0.f && (s & 1 ? f2_hi(TEST[s / 2]) : f2_lo(TEST[s / 2])) >= rp.t_eps ? 1u : 0u;
-          }
-        }
-        if (low < rp.t_eps) {  // a pixel stops in front of this entry
-#pragma unroll
-          for (int p = 0; p < NP; ++p) {
-            const bool s0 = f2_lo(TEST[p]) < rp.t_eps, s1 = f2_hi(TEST[p]) < rp.t_eps;
-            AL[p] = f2_pack(s0 ? 0.f : f2_lo(AL[p]), s1 ? 0.f : f2_hi(AL[p]));
-            TEST[p] = f2_pack(s0 ? f2_lo(T[p]) : f2_lo(TEST[p]), s1 ? f2_hi(T[p]) : f2_hi(TEST[p]));
-            ply[2 * p] = s0 ? kInf : ply[2 * p];
-            ply[2 * p + 1] = s1 ? kInf : ply[2 * p + 1];
-            stop[2 * p] = s0 ? idx : stop[2 * p];
-            stop[2 * p + 1] = s1 ? idx : stop[2 * p + 1];
-          }
-        }
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          const f2x W = f2_mul(AL[p], T[p]);
-          T[p] = TEST[p];
-          R[p] = f2_fma_s(W, ec.x, R[p]);
-          G[p] = f2_fma_s(W, ec.y, G[p]);
-          B[p] = f2_fma_s(W, ec.z, B[p]);
-          D[p] = f2_fma_s(W, eb.z, D[p]);
-        }
+        blend(en, idx);
       } while (can ? !__any_sync(kFull, (walk.cur | gone) == 0u) : walk.any_up_to(lim));
     }
     cp_wait_all();
@@ -708,7 +760,11 @@ __device__ __forceinline__ int rec_off(int k) { return k < 7 ? k : k + 1; }
 // -> 1) and a final xor-1 step (12 shuffles instead of 50), then adds the
 // totals to the record: even lanes hold distinct values, so this is one
 // warp-wide scalar atomic add.
-__device__ __forceinline__ void warp_reduce_add10(const float (&v)[10], int lane, float* __restrict__ rec) {
+struct WarpSum {
+  float x;   // the lane's total
+  int off;   // its float of the record, -1: none
+};
+__device__ __forceinline__ WarpSum warp_sum10(const float (&v)[10], int lane) {
   const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
   float u[5];
 #pragma unroll
@@ -732,7 +788,18 @@ __device__ __forceinline__ void warp_reduce_add10(const float (&v)[10], int lane
   // xor 16; lanes with b2 and (b3 or b1) hold the zero pads
   const int i3 = (b3 ? 3 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
   const bool valid = !(b2 && (b3 || b1));
-  if (!(lane & 1) && valid && x != 0.f) atomicAdd(&rec[rec_off((b4 ? 5 : 0) + i3)], x);
+  return WarpSum{x, !(lane & 1) && valid ? rec_off((b4 ? 5 : 0) + i3) : -1};
+}
+__device__ __forceinline__ void warp_reduce_add10(const float (&v)[10], int lane, float* __restrict__ rec) {
+  const WarpSum s = warp_sum10(v, lane);
+  if (s.off >= 0 && s.x != 0.f) atomicAdd(&rec[s.off], s.x);
+}
+// ... of two entries, whose exchanges do not wait for one another
+__device__ __forceinline__ void warp_reduce_add10(const float (&v)[10], const float (&u)[10], int lane,
+                                                  float* __restrict__ rec_v, float* __restrict__ rec_u) {
+  const WarpSum s = warp_sum10(v, lane), t = warp_sum10(u, lane);
+  if (s.off >= 0 && s.x != 0.f) atomicAdd(&rec_v[s.off], s.x);
+  if (t.off >= 0 && t.x != 0.f) atomicAdd(&rec_u[t.off], t.x);
 }
 
 // Backward pass of region `quad` of the tile of visit k by one warp: back to
@@ -825,132 +892,167 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
   walk.by = (float)byi;
   walk.begin();
   const f2x ONE2 = f2_pack(1.f, 1.f);
-  // every group's next entry
-  auto entry = [&](auto whole_warp) {
-          int idx;
-          const Entry& en = sm.e[walk.take(idx)];
-          const float4 ea = en.a, eb = en.b, ec = en.c;
-          const float dx = __fsub_rn(plx, ea.x);
-          const float t0 = __fmul_rn(ea.z, dx);
-          f2x TQ[NP], WQ[NP];
-          float ar[2 * NP], in[2 * NP];
-    #pragma unroll
-          for (int p = 0; p < NP; ++p) {
-            const f2x DY = f2_sub(PLY[p], f2_bcast(ea.y));
-            WQ[p] = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
-            TQ[p] = f2_mul(WQ[p], f2_bcast(eb.x));
-            const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ[p], TQ[p]));
-            const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
-            ar[2 * p] = ex2_approx(f2_lo(ARG));
-            ar[2 * p + 1] = ex2_approx(f2_hi(ARG));
-            in[2 * p] = one_if_le_and(f2_lo(Q), eb.w, idx, last[2 * p]);
-            in[2 * p + 1] = one_if_le_and(f2_hi(Q), eb.w, idx, last[2 * p + 1]);
-          }
-          f2x AL[NP], AG[NP];  // alpha, and alpha where it is not clamped: 0 where the pixel takes no part
-    #pragma unroll
-          for (int p = 0; p < NP; ++p) AL[p] = AG[p] = f2_mul(f2_pack(ar[2 * p], ar[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
-          if (eb.y > rp.log2_clamp) {  // the 0.99 clamp has zero gradient
-    #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-              const bool c0 = f2_lo(AL[p]) > rp.alpha_max, c1 = f2_hi(AL[p]) > rp.alpha_max;
-              AG[p] = f2_pack(c0 ? 0.f : f2_lo(AL[p]), c1 ? 0.f : f2_hi(AL[p]));
-              AL[p] = f2_pack(c0 ? rp.alpha_max : f2_lo(AL[p]), c1 ? rp.alpha_max : f2_hi(AL[p]));
-            }
-          }
-          f2x GA = 0, GT = 0, GW = 0, V6 = 0, V7 = 0, V8 = 0, V9 = 0;  // sums over the lane's pairs
-    #pragma unroll
-          for (int p = 0; p < NP; ++p) {
-            const f2x OM = f2_sub(ONE2, AL[p]);  // in [0.01, 1]; 1 where the pixel takes no part: T, U unchanged
-            const f2x INV = f2_pack(rcp_approx(f2_lo(OM)), rcp_approx(f2_hi(OM)));
-            T[p] = f2_mul(T[p], INV);  // transmittance in front of this Gaussian
-            const f2x W = f2_mul(AL[p], T[p]);
-            const f2x CD = f2_fma_s(C0[p], ec.x, f2_fma_s(C1[p], ec.y, f2_fma_s(C2[p], ec.z, f2_mul(DD[p], f2_bcast(eb.z)))));
-            // d/d alpha_i: colour/depth T_i c_i - (sum behind)/(1 - alpha_i); alpha image + T_final/(1 - alpha_i)
-            const f2x GAL = f2_sub(f2_mul(T[p], CD), f2_mul(U[p], INV));
-            U[p] = f2_fma(W, CD, U[p]);
-            const f2x g = f2_mul(GAL, AG[p]);
-            const f2x gt = f2_mul(g, TQ[p]);
-            if (p == 0) {
-              GA = g;
-              GT = gt;
-              GW = f2_mul(gt, WQ[p]);
-              V6 = f2_mul(W, DD[p]);
-              V7 = f2_mul(W, C0[p]);
-              V8 = f2_mul(W, C1[p]);
-              V9 = f2_mul(W, C2[p]);
-            } else {
-              GA = f2_add(GA, g);
-              GT = f2_add(GT, gt);
-              GW = f2_fma(gt, WQ[p], GW);
-              V6 = f2_fma(W, DD[p], V6);
-              V7 = f2_fma(W, C0[p], V7);
-              V8 = f2_fma(W, C1[p], V8);
-              V9 = f2_fma(W, C2[p], V9);
-            }
-          }
-          float v[10];
-          v[5] = f2_lo(GA) + f2_hi(GA);
-          v[1] = f2_lo(GT) + f2_hi(GT);
-          v[4] = f2_lo(GW) + f2_hi(GW);
-          v[6] = f2_lo(V6) + f2_hi(V6);
-          v[7] = f2_lo(V7) + f2_hi(V7);
-          v[8] = f2_lo(V8) + f2_hi(V8);
-          v[9] = f2_lo(V9) + f2_hi(V9);
-          v[0] = v[5] * t0;
-          v[2] = v[0] * dx;
-          v[3] = v[1] * dx;
-          float* rec = g2d + 12 * (size_t)__float_as_uint(ec.w);
-          if constexpr (decltype(whole_warp)::value)
-            warp_reduce_add10(v, lane, rec);
-          else
-            group_reduce_add10<M::LPG>(v, lane, rec);
+  // one entry (each group its own, or the same one for all) at place idx of the
+  // list: the lane's sums; returns the Gaussian's record
+  auto sums = [&](const Entry& en, int idx, float (&v)[10]) -> float* {
+    const float4 ea = en.a, eb = en.b, ec = en.c;
+    const float dx = __fsub_rn(plx, ea.x);
+    const float t0 = __fmul_rn(ea.z, dx);
+    f2x TQ[NP], WQ[NP];
+    float ar[2 * NP], in[2 * NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const f2x DY = f2_sub(PLY[p], f2_bcast(ea.y));
+      WQ[p] = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
+      TQ[p] = f2_mul(WQ[p], f2_bcast(eb.x));
+      const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ[p], TQ[p]));
+      const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
+      ar[2 * p] = ex2_approx(f2_lo(ARG));
+      ar[2 * p + 1] = ex2_approx(f2_hi(ARG));
+      in[2 * p] = one_if_le_and(f2_lo(Q), eb.w, idx, last[2 * p]);
+      in[2 * p + 1] = one_if_le_and(f2_hi(Q), eb.w, idx, last[2 * p + 1]);
+    }
+    f2x AL[NP], AG[NP];  // alpha, and alpha where it is not clamped: 0 where the pixel takes no part
+#pragma unroll
+    for (int p = 0; p < NP; ++p) AL[p] = AG[p] = f2_mul(f2_pack(ar[2 * p], ar[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
+    if (eb.y > rp.log2_clamp) {  // the 0.99 clamp has zero gradient
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const bool c0 = f2_lo(AL[p]) > rp.alpha_max, c1 = f2_hi(AL[p]) > rp.alpha_max;
+        AG[p] = f2_pack(c0 ? 0.f : f2_lo(AL[p]), c1 ? 0.f : f2_hi(AL[p]));
+        AL[p] = f2_pack(c0 ? rp.alpha_max : f2_lo(AL[p]), c1 ? rp.alpha_max : f2_hi(AL[p]));
+      }
+    }
+    f2x GA = 0, GT = 0, GW = 0, V6 = 0, V7 = 0, V8 = 0, V9 = 0;  // sums over the lane's pairs
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const f2x OM = f2_sub(ONE2, AL[p]);  // in [0.01, 1]; 1 where the pixel takes no part: T, U unchanged
+      const f2x INV = f2_pack(rcp_approx(f2_lo(OM)), rcp_approx(f2_hi(OM)));
+      T[p] = f2_mul(T[p], INV);  // transmittance in front of this Gaussian
+      const f2x W = f2_mul(AL[p], T[p]);
+      const f2x CD = f2_fma_s(C0[p], ec.x, f2_fma_s(C1[p], ec.y, f2_fma_s(C2[p], ec.z, f2_mul(DD[p], f2_bcast(eb.z)))));
+      // d/d alpha_i: colour/depth T_i c_i - (sum behind)/(1 - alpha_i); alpha image + T_final/(1 - alpha_i)
+      const f2x GAL = f2_sub(f2_mul(T[p], CD), f2_mul(U[p], INV));
+      U[p] = f2_fma(W, CD, U[p]);
+      const f2x g = f2_mul(GAL, AG[p]);
+      const f2x gt = f2_mul(g, TQ[p]);
+      if (p == 0) {
+        GA = g;
+        GT = gt;
+        GW = f2_mul(gt, WQ[p]);
+        V6 = f2_mul(W, DD[p]);
+        V7 = f2_mul(W, C0[p]);
+        V8 = f2_mul(W, C1[p]);
+        V9 = f2_mul(W, C2[p]);
+      } else {
+        GA = f2_add(GA, g);
+        GT = f2_add(GT, gt);
+        GW = f2_fma(gt, WQ[p], GW);
+        V6 = f2_fma(W, DD[p], V6);
+        V7 = f2_fma(W, C0[p], V7);
+        V8 = f2_fma(W, C1[p], V8);
+        V9 = f2_fma(W, C2[p], V9);
+      }
+    }
+    v[5] = f2_lo(GA) + f2_hi(GA);
+    v[1] = f2_lo(GT) + f2_hi(GT);
+    v[4] = f2_lo(GW) + f2_hi(GW);
+    v[6] = f2_lo(V6) + f2_hi(V6);
+    v[7] = f2_lo(V7) + f2_hi(V7);
+    v[8] = f2_lo(V8) + f2_hi(V8);
+    v[9] = f2_lo(V9) + f2_hi(V9);
+    v[0] = v[5] * t0;
+    v[2] = v[0] * dx;
+    v[3] = v[1] * dx;
+    return g2d + 12 * (size_t)__float_as_uint(ec.w);
   };
-  // The entries of a chunk from its first to its last wide one are held back
-  // until the groups are done with what comes before, and then walked by all
-  // groups together, every entry on every block: each Gaussian's sums go over
-  // the whole warp and to its record once, not once per block (the nearest
-  // splats of a map of large ones cover the image: 257k additions to one
-  // record took 1.30 ms where the pass now takes 0.13).
-  unsigned held = 0u, rest = 0u;  // the wide entries; the group's entries of the chunk after them
-  bool together = false;
+  // A chunk taken together, and the entries of another from its first to its last
+  // wide one, are held back until the groups are
+  // done with what comes before, and then walked by all groups together, every
+  // entry on every block: each Gaussian's sums go over the whole warp and to its
+  // record once, not once per block (the nearest splats of a map of large ones
+  // cover the image: 257k additions to one record took 1.30 ms where the pass
+  // now takes 0.13).
+  unsigned held = 0u, rest = 0u;  // these entries; the group's entries of the chunk after them
+  bool all = false;               // the groups have them as their own lists (four pixels per lane; a loop over
+                                  // them made the pass 1.3 us slower, 106 -> 107.4)
   for (;;) {
     while (__any_sync(kFull, walk.cur == 0u && walk.off < walk.top)) walk.step();
-    const bool can = walk.can_stage() && !together && !held;
+    const bool can = walk.can_stage() && !held && !all;
     if (can && __any_sync(kFull, walk.cur == 0u)) {  // a group is dry
       unsigned m;
       bool wide;
       unsigned mine = walk.stage(rp, m, wide);
       const int over = walk.chunk(walk.top) + 32 - glast;  // entries behind every pixel of the group
       if (over > 0) mine = over < 32 ? mine & (kFull >> over) : 0u;
-      const unsigned w = __ballot_sync(kFull, m != 0u && wide);
-      if (w) {  // (entry 31 comes first)
-        const unsigned behind = kFull << (31 - __clz(w)) << 1, front = (1u << (__ffs(w) - 1)) - 1u;
-        held = __ballot_sync(kFull, m != 0u) & ~behind & ~front;
-        rest = mine & front;
-        mine &= behind;
+      const unsigned whole = __ballot_sync(kFull, PPL == 1 ? m != 0u : kTogether<PPL> ? m == kFull : m != 0u && wide);
+      rest = 0u;
+      if (whole) {
+        const unsigned meet = __ballot_sync(kFull, m != 0u);
+        const unsigned w = kTogether<PPL> ? __ballot_sync(kFull, m != 0u && wide) : whole;
+        if (kTogether<PPL> && (PPL == 1 || together<PPL>(meet, whole))) {
+          held = meet;
+          mine = 0u;
+        } else if (w) {  // (entry 31 comes first)
+          const unsigned behind = kFull << (31 - __clz(w)) << 1, front = (1u << (__ffs(w) - 1)) - 1u;
+          held = meet & ~behind & ~front;
+          rest = mine & front;
+          mine &= behind;
+        }
       }
       walk.push(mine);
       continue;
     }
     int lim = walk.end;
-    if (!together && !held) {
+    if (!held && !all) {
       lim = walk.limit(can);
       if (lim == walk.kEnd) break;
       if (lim == walk.kAgain) continue;
-    } else if (!__any_sync(kFull, walk.cur != 0u)) {  // the wide entries' turn, or they are done
+    } else if (!__any_sync(kFull, walk.cur != 0u)) {  // the held entries' turn, or they are done
+      if constexpr (kTogether<PPL>) {
+        const Entry* e = sm.e + ((walk.top - 32) & (kRing - 1));
+        const int i0 = walk.chunk(walk.top - 32);
+        while (held) {
+          const int j = 31 - __clz(held);
+          held ^= 1u << j;
+          float v[10];
+          float* rec = sums(e[j], i0 + j, v);
+          if (held) {
+            const int k = 31 - __clz(held);
+            held ^= 1u << k;
+            float u[10];
+            float* rec_u = sums(e[k], i0 + k, u);
+            warp_reduce_add10(v, u, lane, rec, rec_u);
+          } else {
+            warp_reduce_add10(v, lane, rec);
+          }
+        }
+        walk.cur = rest;
+      } else {
+        walk.cur = all ? rest : held;
+        all = !all;
+        held = 0u;
+      }
       walk.base = walk.off = walk.top - 32;
-      walk.cur = together ? rest : held;
-      together = !together;
-      held = 0u;
       continue;
     }
-    if (together) {
-      do entry(std::true_type());
-      while (__any_sync(kFull, walk.cur != 0u));
-    } else {
-      do entry(std::false_type());
-      while (can ? !__any_sync(kFull, walk.cur == 0u) : walk.any_up_to(lim));
+    if (all) {
+      do {
+        int idx;
+        const Entry& en = sm.e[walk.take(idx)];
+        float v[10];
+        float* rec = sums(en, idx, v);
+        warp_reduce_add10(v, lane, rec);
+      } while (__any_sync(kFull, walk.cur != 0u));
+      continue;
     }
+    do {
+      int idx;
+      const Entry& en = sm.e[walk.take(idx)];
+      float v[10];
+      float* rec = sums(en, idx, v);
+      group_reduce_add10<M::LPG>(v, lane, rec);
+    } while (can ? !__any_sync(kFull, walk.cur == 0u) : walk.any_up_to(lim));
   }
   cp_wait_all();
 }
