@@ -378,8 +378,12 @@ gs_status ensure_px(gs_ctx* c, int64_t npx) {
   GS_GROW(c, cap_px, regrow(&c->T_final, cap));
   GS_GROW(c, cap_px, regrow(&c->last, cap));
   GS_GROW(c, cap_px, regrow(&c->dl_img, 4 * cap));
-  // per-block partials (blocks of every view: <= blocks(total) + views) and per-view scales
-  const int64_t lb = loss_blocks_max(cap);
+  // per-block partials (blocks of every view: <= blocks(total) + views) and
+  // per-view scales; also the fused loss's: images of one column have a tile
+  // per 8 pixels, with at most 4 warp jobs when they are many (8 when below one
+  // per SM)
+  static_assert(kLossChunk == 512, "cap / 1024 blocks of 512 of 4 jobs per 8 pixels");
+  const int64_t lb = std::max(loss_blocks_max(cap), cap / 1024 + kMaxViews);
   GS_GROW(c, cap_px, regrow(&c->loss_partials, 3 * (lb + kMaxViews) + kMaxViews + 4));
   c->cap_px = cap;
   c->have_state = false;
