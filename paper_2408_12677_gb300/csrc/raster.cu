@@ -116,7 +116,11 @@ constexpr float kNanOpacity = 64.f;
 // centres of lane l's block.  The box holds every pixel the per-pixel test can
 // accept: q' <= min(qmax, log2 o - log2 alpha_min) is the ellipse
 // (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents sqrt(R2) / i0 and
-// sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2); the widening covers float32 rounding
+// sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2), and per row of blocks only the ellipse's
+// extent over its pixel centres counts: the box of a thin slanted splat holds
+// many times the pixels that it reaches (300k needles of 100 px, forward 4.5 -> 0.8
+// ms, backward 23 -> 4.9 ms; 20000 random splats of up to 20:1 179 -> 150 and 291
+// -> 236 us; 300k seeded ones as before).  The widening covers float32 rounding
 // of the test and of the hardware square roots and reciprocals.  `wide`: the
 // box has more than 4 kWide pixels.  A NaN opacity (fminf passes it over in R2
 // and here) becomes one that is clamped wherever the splat reaches: the raster
@@ -134,22 +138,28 @@ __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, 
   if (!(R2 > 0.f && f1.x > 0.f && f1.z > 0.f)) return 0u;
   const float Rr = sqrt_approx(R2) * 1.0001f + 1e-4f;
   const float inv0 = rcp_approx(f1.x), inv1 = rcp_approx(f1.z);
-  const float ex = Rr * inv0 + 1e-3f;
-  const float ey = Rr * sqrt_approx(f1.y * f1.y * inv0 * inv0 + inv1 * inv1) + 1e-3f;
+  const float ex0 = Rr * inv0, ey0 = Rr * sqrt_approx(f1.y * f1.y * inv0 * inv0 + inv1 * inv1);
+  const float ex = ex0 + 1e-3f, ey = ey0 + 1e-3f;
   wide = ex * ey > kWide;
-  // first and last block column and row whose centres lie within the box
-  constexpr float BW = M::LPG, BH = M::ROWS, NC = M::RW / M::LPG, NR = M::RH / M::ROWS;
-  const float rx = mlx - bx, ry = mly - by;
-  const int c0 = __float2int_ru(fmaxf((rx - ex + 0.5f) / BW - 1.f, 0.f));
-  const int c1 = __float2int_rd(fminf((rx + ex - 0.5f) / BW, NC - 1.f));
-  const int r0 = __float2int_ru(fmaxf((ry - ey + 0.5f) / BH - 1.f, 0.f));
-  const int r1 = __float2int_rd(fminf((ry + ey - 0.5f) / BH, NR - 1.f));
-  if (c1 < c0 || r1 < r0) return 0u;
+  // at height y from its centre the ellipse's x is within kx y +- hx
+  const float u = ex0 * rcp_approx(ey0);
+  const float kx = f1.y * u * u, hx = u * Rr * inv1 + 1e-3f + 4e-6f * ex;
+  // per row of blocks, the first and last column with centres in that range and
+  // in the box (fmaxf and fminf pass a NaN of extreme ratios over: the box alone)
+  constexpr float BW = M::LPG, BH = M::ROWS, NC = M::RW / M::LPG;
   constexpr unsigned kRow = M::RW == 32 ? kFull : (1u << M::RW) - 1u;
-  const unsigned xm = (kRow >> (M::RW - M::LPG * (c1 - c0 + 1))) << (M::LPG * c0);
+  const float rx = mlx - bx, ry = mly - by;
+  const float box0 = fmaxf((rx - ex + 0.5f) / BW - 1.f, 0.f), box1 = fminf((rx + ex - 0.5f) / BW, NC - 1.f);
+  const float mid = rx + kx * (0.5f - ry), span = kx * (BH - 1.f), step = kx * (BH / BW);
+  const float lo = (mid + fminf(span, 0.f) - hx + 0.5f) / BW - 1.f, hi = (mid + fmaxf(span, 0.f) + hx - 0.5f) / BW;
+  const float row0 = (ry - ey + 0.5f) / BH - 1.f, row1 = (ry + ey - 0.5f) / BH;
   unsigned m = 0u;
 #pragma unroll
-  for (int r = 0; r < M::RH / M::ROWS; ++r) m |= r0 <= r && r <= r1 ? xm << (M::RW * r) : 0u;
+  for (int r = 0; r < M::RH / M::ROWS; ++r) {
+    const int c0 = __float2int_ru(fmaxf(lo + r * step, box0)), c1 = __float2int_rd(fminf(hi + r * step, box1));
+    const unsigned xm = (kRow >> (M::RW - M::LPG * (c1 - c0 + 1))) << (M::LPG * c0);
+    m |= row0 <= r && r <= row1 && c0 <= c1 ? xm << (M::RW * r) : 0u;
+  }
   return m;
 }
 
