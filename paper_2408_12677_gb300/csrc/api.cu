@@ -67,7 +67,8 @@ struct gs_ctx {
   bool bwd_work_zero = false;     // both; a raster launch uses its counter up)
   bool g2d_zero = false;          // the gradient records are all 0 (their consumers clear what they read)
   unsigned long long* d_binstats = nullptr;  // [0] total pairs, [1] longest tile list; of cut lists also [2] the
-                                             // largest kept rank, [3] level-2 tiles, [4] a pixel did not stop
+                                             // largest kept rank, [3] level-2 tiles, [4] tiles whose pixels did
+                                             // not all stop
   long long* d_step = nullptr;               // device Adam step counter (step = 0 calls)
   int64_t cap_px = 0;
   float* T_final = nullptr;
@@ -158,6 +159,7 @@ struct gs_ctx {
   int64_t cap_pfx_diff = 0;
   int* pfx_diff = nullptr;
   const uint32_t* pfx_sorted = nullptr;  // items by depth (of the current pass)
+  int cut_wait = 0;               // passes of long lists to bin in full before their lists are cut again
   bool st_cut = false;            // the last forward pass's lists are cut (tcount, toffset: the full ones)
   int* big_diff = nullptr;        // difference grids of the projection's large rectangles, 0 between passes
                                   // (part of tcount's allocation)
@@ -455,10 +457,11 @@ gs_status ensure_hist(gs_ctx* c) {
 }
 
 // Radix binning (used when a tile list is longer than the per-tile sort holds):
-// depth sort of the n items (keys in zkey, ids implicit), duplication into
-// pairs, pair sort by global tile, tile ranges.  On success c->st_pairs /
-// st_pair_buf describe the sorted pair list.
-gs_status bin_and_sort_radix(gs_ctx* c, int n, const TileMap& map, cudaStream_t s) {
+// depth sort of the n items (keys in zkey, ids implicit; `sorted_ids` when they
+// are in order already), duplication into pairs, pair sort by global tile, tile
+// ranges.  On success c->st_pairs / st_pair_buf describe the sorted pair list.
+gs_status bin_and_sort_radix(gs_ctx* c, int n, const TileMap& map, cudaStream_t s,
+                             const uint32_t* sorted_ids = nullptr) {
   const int64_t T = (int64_t)map.tile_base[map.views];
   if (c->sync) GS_CUDA(c, cudaMemsetAsync(c->d_overflow, 0, sizeof(uint32_t), s));
   SortBuffers sb;
@@ -468,12 +471,11 @@ gs_status bin_and_sort_radix(gs_ctx* c, int n, const TileMap& map, cudaStream_t 
   sb.vals[1] = c->dval[1];
   sb.hist = c->hist;
   sb.max_blocks = c->hist_blocks;
-  int dcur;
-  {
+  if (!sorted_ids) {
     StageTimer t(c, GS_STAGE_DEPTH_SORT, s);
-    dcur = radix_sort_pairs(sb, c->zkey, nullptr, (uint32_t)n, nullptr, 32, c->num_sms, s, &c->launches);
+    const int dcur = radix_sort_pairs(sb, c->zkey, nullptr, (uint32_t)n, nullptr, 32, c->num_sms, s, &c->launches);
+    sorted_ids = dcur >= 0 ? c->dval[dcur] : c->dval[0];
   }
-  const uint32_t* sorted_ids = dcur >= 0 ? c->dval[dcur] : c->dval[0];
 
   DupArgs da;
   da.n = n;
@@ -598,12 +600,20 @@ gs_status bin_buckets(gs_ctx* c, int n, const TileMap& map, cudaStream_t s) {
 constexpr uint32_t kPrefixTarget = 256, kPrefixRanks = 32768;
 // Only where the mean list is that long.  A few long lists in a scene of short
 // ones are long because their pixels do not stop (grazing views of distant
-// surfaces): they are gathered whole and the pass is rastered again, 9.5 ms for
-// 8 views of 500k Gaussians (lists of 403, 33 of 31360 above 4096) against 4.3
-// ms binned in full.  Where large splats cover the tiles the nearest entries
-// are cheaper: 0.90 against 2.24 ms for lists of 3266 (1752 x 1168, 1M), 0.37
-// against 0.52 ms for 2916 (640 x 480, 200k).
-constexpr int64_t kPrefixMean = 768;
+// surfaces): they are gathered whole and the pass is rastered again.  Lists of
+// 1000 to 2000 entries are binned in full in the time of a second attempt, which
+// faint splats always need (training steps, cut / in full: 1752 x 1168, 1M
+// Gaussians, lists of 1191, opaque 1.88 / 1.35 ms; 1451, a tenth of the image
+// faint 1.95 / 1.64; 920, faint 6.1 / 3.4; 8 views of 640 x 480, 1031, faint 8.7 /
+// 4.8; 1955, opaque 1.83 / 1.75; 2452, opaque 0.98 / about 2.2).
+constexpr int64_t kPrefixMean = 2048;
+// A level-2 list costs a look at every item.  Where so many tiles are still open
+// after the second attempt that this takes longer than binning all pairs (kLooks
+// looks, at 1.9 to 2.2 ps, against a pair's 73 ps: faint needles of 100 px), the
+// pass is binned in full, and so are the context's next kCutWait passes that
+// would be cut.
+constexpr int64_t kLooks = 32;
+constexpr int kCutWait = 15;
 gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, cudaStream_t s, int attempt,
                      bool* done) {
   const int64_t T = (int64_t)map.tile_base[map.views];
@@ -774,7 +784,10 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
                    ensure_buckets(c, T, (uint32_t)entries) == GS_OK &&
                    c->cap_bt * (int64_t)kLenClasses < ((int64_t)1 << 32);
     if (longest > tile_sort_capacity()) {
-      if (tiles_y && P <= 0xFFFFFFF0ll && P >= kPrefixMean * T) {  // (more pairs than that are refused by the full binning)
+      const bool cut = tiles_y && P <= 0xFFFFFFF0ll && P >= kPrefixMean * T;  // (more pairs are refused by the full binning)
+      if (cut && c->cut_wait > 0) {
+        c->cut_wait -= 1;
+      } else if (cut) {
         bool done = false;
         const gs_status ps = bin_prefix(c, n, map, tiles_y, s, 0, &done);
         if (ps != GS_OK) return ps;
@@ -1346,16 +1359,19 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   GS_CHECK_LAUNCH(c, "raster_open");
   GS_CUDA(c, cudaMemcpyAsync(c->h_pinned, c->d_binstats + 4, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   GS_CUDA(c, cudaStreamSynchronize(s));
-  if (c->h_pinned[0] == 0) break;
+  const int64_t open_tiles = (int64_t)c->h_pinned[0];
+  if (open_tiles == 0) break;
   // some list was cut too short: bin again with longer ones (the third time
-  // in full, which no pixel can exhaust)
+  // the open tiles' in full, which no pixel can exhaust), or all in full
   if (attempt == 2) return fail(c, GS_ERR_CUDA, "a full list left a pixel open");
   if (c->counting)
     GS_CUDA(c, cudaMemcpyAsync(c->d_evals, c->d_evals + 2, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
   if (fl) GS_CUDA(c, cudaMemsetAsync(c->d_nvalid, 0, kMaxViews * sizeof(uint32_t), s));
   bool done = false;
-  if ((st = bin_prefix(c, n_items, L.map, L.tiles_y, s, attempt + 1, &done)) != GS_OK) return st;
-  if (!done && (st = bin_and_sort_radix(c, n_items, L.map, s)) != GS_OK) return st;
+  const bool in_full = attempt == 1 && open_tiles * n_items > kLooks * c->st_pairs;
+  if (in_full) c->cut_wait = kCutWait;
+  else if ((st = bin_prefix(c, n_items, L.map, L.tiles_y, s, attempt + 1, &done)) != GS_OK) return st;
+  if (!done && (st = bin_and_sort_radix(c, n_items, L.map, s, c->pfx_sorted)) != GS_OK) return st;
   }
   c->st_g = *g;
   for (int v = 0; v < V; ++v) {

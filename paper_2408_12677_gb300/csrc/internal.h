@@ -364,8 +364,9 @@ void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsig
 void launch_loss_tiles_finalize(const RasterArgs& a, float w_depth, float* loss, float* depth_scale,
                                 float* partials, uint32_t* ticket, long long* step, cudaStream_t s,
                                 int64_t* launches);
-// after a forward pass over cut lists: level[t] is raised and *open set for a
-// tile with cut[t] whose list ends before all of its pixels have stopped
+// after a forward pass over cut lists: level[t] is raised for each tile with
+// cut[t] whose list ends before all of its pixels have stopped, and these are
+// added to *open
 void launch_raster_open(const RasterArgs& a, const int32_t* last, const uint8_t* cut, uint8_t* level,
                         unsigned long long* open, cudaStream_t s);
 void launch_raster_bwd(const RasterArgs& a, const float* T_final, const int32_t* last, float4* g2d, cudaStream_t s);

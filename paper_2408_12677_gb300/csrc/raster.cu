@@ -1088,10 +1088,11 @@ __global__ void __launch_bounds__(kThreads, kBwdCtas) raster_bwd_kernel(const __
 }
 
 // Marks the tiles whose list is cut and holds a pixel that did not stop (one
-// CTA of 256 threads per tile).
+// CTA of 256 threads per tile) and counts them.
 __global__ void __launch_bounds__(256) raster_open_kernel(const __grid_constant__ RasterArgs a,
                                                           const int32_t* __restrict__ last_all,
-                                                          const uint8_t* __restrict__ cut, uint8_t* __restrict__ level,
+                                                          const uint8_t* __restrict__ cut,
+                                                          uint8_t* __restrict__ level,
                                                           unsigned long long* __restrict__ open) {
   const uint32_t tile = blockIdx.x;
   if (!cut[tile]) return;
@@ -1105,7 +1106,7 @@ __global__ void __launch_bounds__(256) raster_open_kernel(const __grid_constant_
   const bool mine = in && (last_all[a.v[v].pix_base + (size_t)py * a.v[v].width + px] & kOpen);
   if (__syncthreads_or(mine) && threadIdx.x == 0) {
     level[tile] += 1;
-    atomicOr(open, 1ull);
+    atomicAdd(open, 1ull);
   }
 }
 
