@@ -627,6 +627,7 @@ gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, c
   if (st != GS_OK) return st;
   for (int v = 0; v < map.views; ++v) a.tiles_y[v] = tiles_y[v];
   a.grid_cells = (uint32_t)cells;
+  a.n = (uint32_t)n;
   a.target = kPrefixTarget;
   if (attempt == 0) {
     SortBuffers sb;
@@ -703,7 +704,7 @@ gs_status bin_prefix(gs_ctx* c, int n, const TileMap& map, const int* tiles_y, c
   {
     StageTimer t(c, GS_STAGE_DUPLICATE, s);
     launch_prefix_scatter(a, max_lim, c->pfx_cur, c->pv[0], tb.capacity, s, &c->launches);
-    launch_prefix_gather(a, n_gather, (uint32_t)n, c->pfx_rects, c->pfx_off, c->pv[0], tb.capacity, s, &c->launches);
+    launch_prefix_gather(a, n_gather, c->pfx_rects, c->pfx_off, c->pv[0], tb.capacity, s, &c->launches);
   }
   {
     StageTimer t(c, GS_STAGE_PAIR_SORT, s);
@@ -882,6 +883,7 @@ gs_status gs_ctx_create(gs_ctx** out, int device, int64_t pair_capacity) {
   if (e == cudaSuccess) e = cudaMemset(c->d_bounds, 0, sizeof(uint32_t));
   if (e == cudaSuccess) e = raster_bind_bounds(c->d_bounds);
   if (e == cudaSuccess) e = tilebin_bind_bounds(c->d_bounds);
+  if (e == cudaSuccess) e = prefix_bind_bounds(c->d_bounds);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_pinned, 4 * sizeof(unsigned long long));
   if (e != cudaSuccess) {
     gs_ctx_destroy(c);

@@ -261,6 +261,7 @@ struct PrefixArgs {
   int tiles_y[kMaxViews];
   uint32_t grid_base[kMaxViews];  // first cell of each view's (tiles_x + 1) x (tiles_y + 1) grid
   uint32_t grid_cells;            // cells of a slab's grids
+  uint32_t n;                     // items
   uint32_t ranks;                 // items looked at, nearest first
   int slabs;
   uint32_t bound[kPrefixSlabs];   // first rank behind each slab
@@ -281,8 +282,8 @@ void prefix_slabs(PrefixArgs& a, uint32_t ranks);  // sets ranks, slabs, bound
 void launch_prefix_choose(const PrefixArgs& a, cudaStream_t s, int64_t* launches);
 void launch_prefix_scatter(const PrefixArgs& a, uint32_t max_lim, uint32_t* cursors, uint32_t* ids, uint32_t capacity,
                            cudaStream_t s, int64_t* launches);
-// the level-2 tiles' lists out of all n items; srects: scratch of n rectangles
-void launch_prefix_gather(const PrefixArgs& a, uint32_t n_gather, uint32_t n, ushort4* srects, const uint32_t* offsets,
+// the level-2 tiles' lists out of all items; srects: scratch of a rectangle per item
+void launch_prefix_gather(const PrefixArgs& a, uint32_t n_gather, ushort4* srects, const uint32_t* offsets,
                           uint32_t* ids, uint32_t capacity, cudaStream_t s, int64_t* launches);
 // out[t] = tile t's range in the full (virtual) pair list
 void launch_full_ranges(const uint32_t* offsets, const uint32_t* full, int n, uint2* out, cudaStream_t s);
@@ -352,6 +353,7 @@ constexpr int kMaxTileJobs = 8;
 // context's bounds word (no-op in the normal build)
 cudaError_t raster_bind_bounds(uint32_t* word);
 cudaError_t tilebin_bind_bounds(uint32_t* word);
+cudaError_t prefix_bind_bounds(uint32_t* word);
 void launch_raster_fwd(const RasterArgs& a, float* T_final, int32_t* last, unsigned long long* counters,
                        cudaStream_t s);
 // loss from the forward pass's per-block partials: loss = sum over views of

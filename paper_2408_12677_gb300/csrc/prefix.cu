@@ -31,16 +31,23 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// An item's id and rectangle, checked in the bounds-checked build.
+__device__ __forceinline__ bool item_ok(const PrefixArgs& a, uint32_t id) { return in_bounds(id < a.n); }
+__device__ __forceinline__ bool rect_ok(const PrefixArgs& a, int v, ushort4 q) {
+  return in_bounds(q.x <= q.z && q.y <= q.w && (int)q.z <= a.map.tiles_x[v] && (int)q.w <= a.tiles_y[v]);
+}
+
 __global__ void __launch_bounds__(kThreads) slab_count_kernel(const __grid_constant__ PrefixArgs a) {
   const uint32_t r = blockIdx.x * kThreads + threadIdx.x;
   const uint32_t id = r < a.ranks ? a.sorted[r] : 0u;
-  const bool live = r < a.ranks && a.tiles[id] != 0u;
+  bool live = r < a.ranks && item_ok(a, id) && a.tiles[id] != 0u;
+  const int v = a.map.views == 1 || !live ? 0 : (int)(id / (uint32_t)a.map.n_per_view);
+  const ushort4 q = live ? a.rects[id] : make_ushort4(0, 0, 0, 0);
+  live = live && rect_ok(a, v, q);
   const unsigned act = __ballot_sync(0xFFFFFFFFu, live);
   if (!live) return;
   int s = 0;
   while (r >= a.bound[s]) ++s;
-  const int v = a.map.views == 1 ? 0 : (int)(id / (uint32_t)a.map.n_per_view);
-  const ushort4 q = a.rects[id];
   const int w = a.map.tiles_x[v] + 1;
   int* g = a.diff + (size_t)s * a.grid_cells + a.grid_base[v];
   warp_agg_add(g + q.y * w + q.x, 1, act);
@@ -92,35 +99,39 @@ __global__ void __launch_bounds__(128) prefix_scatter_kernel(const __grid_consta
                                                              uint32_t* __restrict__ cursors,
                                                              uint32_t* __restrict__ ids, uint32_t capacity) {
   const uint32_t r = blockIdx.x;
-  const uint32_t id = a.sorted[r], n = a.tiles[id];
+  const uint32_t id = a.sorted[r];
+  if (!item_ok(a, id)) return;
+  const uint32_t n = a.tiles[id];
   if (n == 0u) return;
   const int v = a.map.views == 1 ? 0 : (int)(id / (uint32_t)a.map.n_per_view);
   const ushort4 q = a.rects[id];
   const uint32_t w = (uint32_t)(q.z - q.x);
   for (uint32_t k = threadIdx.x; k < n; k += 128) {
     const uint32_t t = a.map.tile_base[v] + (q.y + k / w) * (uint32_t)a.map.tiles_x[v] + q.x + k % w;
-    if (r >= a.lim[t]) continue;
+    if (!in_bounds(t < a.map.tile_base[a.map.views]) || r >= a.lim[t]) continue;
     const uint32_t pos = atomicAdd(&cursors[t], 1u);
     if (pos < capacity) ids[pos] = id;
   }
 }
 
-__global__ void __launch_bounds__(kThreads) sort_rects_kernel(uint32_t n, const uint32_t* __restrict__ sorted,
-                                                              const ushort4* __restrict__ rects,
+__global__ void __launch_bounds__(kThreads) sort_rects_kernel(const __grid_constant__ PrefixArgs a,
                                                               ushort4* __restrict__ out) {
   const uint32_t r = blockIdx.x * kThreads + threadIdx.x;
-  if (r < n) out[r] = rects[sorted[r]];
+  if (r >= a.n) return;
+  const uint32_t id = a.sorted[r];
+  out[r] = item_ok(a, id) ? a.rects[id] : make_ushort4(0, 0, 0, 0);
 }
 
 // One block per level-2 tile: its items in depth order, kGatherItems
 // consecutive ranks per thread and round, their places by a block scan.
 constexpr int kGatherThreads = 512, kGatherItems = 4;
-__global__ void __launch_bounds__(kGatherThreads) prefix_gather_kernel(const __grid_constant__ PrefixArgs a, uint32_t n,
+__global__ void __launch_bounds__(kGatherThreads) prefix_gather_kernel(const __grid_constant__ PrefixArgs a,
                                                                        const ushort4* __restrict__ srects,
                                                                        const uint32_t* __restrict__ offsets,
                                                                        uint32_t* __restrict__ ids, uint32_t capacity) {
   __shared__ uint32_t s_w[2][kGatherThreads / 32];
-  const uint32_t t = a.gather[blockIdx.x];
+  const uint32_t t = a.gather[blockIdx.x], n = a.n;
+  if (!in_bounds(t < a.map.tile_base[a.map.views])) return;
   int v = 0;
   for (int k = 1; k < a.map.views; ++k)
     if (t >= a.map.tile_base[k]) v = k;
@@ -207,16 +218,18 @@ void launch_prefix_scatter(const PrefixArgs& a, uint32_t max_lim, uint32_t* curs
   if (launches) *launches += 1;
 }
 
-void launch_prefix_gather(const PrefixArgs& a, uint32_t n_gather, uint32_t n, ushort4* srects, const uint32_t* offsets,
+void launch_prefix_gather(const PrefixArgs& a, uint32_t n_gather, ushort4* srects, const uint32_t* offsets,
                           uint32_t* ids, uint32_t capacity, cudaStream_t s, int64_t* launches) {
-  if (n_gather == 0 || n == 0) return;
-  sort_rects_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(n, a.sorted, a.rects, srects);
-  prefix_gather_kernel<<<n_gather, kGatherThreads, 0, s>>>(a, n, srects, offsets, ids, capacity);
+  if (n_gather == 0 || a.n == 0) return;
+  sort_rects_kernel<<<(a.n + kThreads - 1) / kThreads, kThreads, 0, s>>>(a, srects);
+  prefix_gather_kernel<<<n_gather, kGatherThreads, 0, s>>>(a, srects, offsets, ids, capacity);
   if (launches) *launches += 2;
 }
 
 void launch_full_ranges(const uint32_t* offsets, const uint32_t* full, int n, uint2* out, cudaStream_t s) {
   if (n > 0) full_ranges_kernel<<<(n + 255) / 256, 256, 0, s>>>(offsets, full, n, out);
 }
+
+cudaError_t prefix_bind_bounds(uint32_t* word) { return bind_bounds_word(word); }
 
 }  // namespace gs

@@ -118,9 +118,9 @@ constexpr float kNanOpacity = 64.f;
 // (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents sqrt(R2) / i0 and
 // sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2), and per row of blocks only the ellipse's
 // extent over its pixel centres counts: the box of a thin slanted splat holds
-// many times the pixels that it reaches (300k needles of 100 px, forward 4.5 -> 0.8
-// ms, backward 23 -> 4.9 ms; 20000 random splats of up to 20:1 179 -> 150 and 291
-// -> 236 us; 300k seeded ones as before).  The widening covers float32 rounding
+// many times the pixels that it reaches (300k faint needles of 100 px: backward 23
+// -> 4.9 ms, forward 2.3, with one list per warp 13.7 and 12.4; 20000 random
+// splats of up to 20:1 179 -> 150 and 291 -> 236 us; 300k seeded ones as before).  The widening covers float32 rounding
 // of the test and of the hardware square roots and reciprocals.  `wide`: the
 // box has more than 4 kWide pixels.  A NaN opacity (fminf passes it over in R2
 // and here) becomes one that is clamped wherever the splat reaches: the raster
