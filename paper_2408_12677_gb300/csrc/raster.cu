@@ -293,21 +293,29 @@ struct Walk {
 // most of its entries that meet the warp's region (meet) meet every block of it
 // (whole): the lanes' lists would be nearly the same, and the backward pass makes
 // one addition to a Gaussian's record per region instead of one per block.  With
-// four pixels an addition the gradients' errors against 64 bits were up to 1.75
-// times those with 64 (200 x 150, 2000 large splats; 1.03 to 1.07 for a seeded
-// map; means over 24 maps); now they are 0.97 to 1.02 times.  With one pixel per
-// lane the backward pass takes every chunk so, two entries at a time, since the
-// few warps wait for each other's exchanges: forward + backward 24 + 45 -> 24 + 40
-// us for the former, 36 + 64 -> 34 + 57 us for 5000 at 320 x 240.  Three quarters
-// or half of the entries with two pixels per lane took 75 and 80 instead of 74 us
-// an iteration on a seeded map of 20000.  Not with four, whose additions are of
-// eight pixels in large images (errors as with 64 pixels): 294 -> 295 us for 300k
-// Gaussians, 1327 -> 1340 for five views.
+// four or eight pixels an addition the gradients' errors against 64 bits were up
+// to 1.75 times those with 64 (200 x 150, 2000 large splats; 1.03 to 1.07 for a
+// seeded map; means over 24 to 50 maps); now they are 0.95 to 1.05 times, with a
+// spread of 0.03 (200 x 150 to 500 x 400).  With one pixel per lane the backward
+// pass takes every chunk so, two entries at a time, since the few warps wait for
+// each other's exchanges: 97.4 -> 87.8 us an iteration for the former with the
+// ellipse's test of the rows, 150 -> 124 us for 5000 at 320 x 240.  It costs
+// small seeded maps 1 to 4% of an iteration (66 x 38, 896 Gaussians, 55.4 -> 58.4
+// us; 280 x 210, 12000, 66.0 -> 67.8).  With two pixels per lane from three
+// quarters of the entries (seven eighths: errors up to 1.25 at 280 x 210; half: 79
+// instead of 75 us for 20000 seeded ones at 320 x 240), forward from seven
+// eighths.  Not with four, whose additions are of eight pixels in large images
+// (errors as with 64): 294 -> 295 us for 300k Gaussians, 1327 -> 1340 for five
+// views.
 template <int PPL>
 constexpr bool kTogether = PPL <= 2;
 template <int PPL>
-__device__ __forceinline__ bool together(unsigned meet, unsigned whole) {
+__device__ __forceinline__ bool together_fwd(unsigned meet, unsigned whole) {
   return PPL == 1 ? 2 * __popc(whole) >= __popc(meet) : 8 * __popc(whole) >= 7 * __popc(meet);
+}
+template <int PPL>
+__device__ __forceinline__ bool together_bwd(unsigned meet, unsigned whole) {
+  return PPL == 1 || 4 * __popc(whole) >= 3 * __popc(meet);
 }
 
 // Slot kRing of a warp's entries: support radius -1, accepted by no pixel.
@@ -579,7 +587,7 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
           const unsigned whole = __ballot_sync(kFull, m == kFull);
           if (whole) {
             const unsigned meet = __ballot_sync(kFull, m != 0u);
-            if (together<PPL>(meet, whole)) held = meet;
+            if (together_fwd<PPL>(meet, whole)) held = meet;
           }
         }
         walk.push(mine, !held);
@@ -1000,7 +1008,7 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
       if (whole) {
         const unsigned meet = __ballot_sync(kFull, m != 0u);
         const unsigned w = kTogether<PPL> ? __ballot_sync(kFull, m != 0u && wide) : whole;
-        if (kTogether<PPL> && (PPL == 1 || together<PPL>(meet, whole))) {
+        if (kTogether<PPL> && together_bwd<PPL>(meet, whole)) {
           held = meet;
           mine = 0u;
         } else if (w) {  // (entry 31 comes first)
