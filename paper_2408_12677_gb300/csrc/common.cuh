@@ -122,6 +122,12 @@ __device__ __forceinline__ void adam_apply(float& p, float g, float& m, float& v
   p -= __fdividef(lr * ss * m, sqrt_approx(v) * isb2 + eps);
 }
 
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // 1 / x by the hardware reciprocal (PTX rcp.approx: relative error within
 // 2^-23 for normal x), one instruction instead of the IEEE-rounded
 // division sequence; used where x is a normal number far from overflow.

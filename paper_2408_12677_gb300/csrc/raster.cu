@@ -138,11 +138,11 @@ __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, 
   if (!(R2 > 0.f && f1.x > 0.f && f1.z > 0.f)) return 0u;
   const float Rr = sqrt_approx(R2) * 1.0001f + 1e-4f;
   const float inv0 = rcp_approx(f1.x), inv1 = rcp_approx(f1.z);
-  const float ex0 = Rr * inv0, ey0 = Rr * sqrt_approx(f1.y * f1.y * inv0 * inv0 + inv1 * inv1);
-  const float ex = ex0 + 1e-3f, ey = ey0 + 1e-3f;
+  const float kw = f1.y * inv0, h2 = fmaxf(kw * kw + inv1 * inv1, 1e-30f), rs = rsqrt_approx(h2);
+  const float ex = Rr * inv0 + 1e-3f, ey = Rr * (h2 * rs) + 1e-3f;
   wide = ex * ey > kWide;
   // at height y from its centre the ellipse's x is within kx y +- hx
-  const float u = ex0 * rcp_approx(ey0);
+  const float u = inv0 * rs;
   const float kx = f1.y * u * u, hx = u * Rr * inv1 + 1e-3f + 4e-6f * ex;
   // per row of blocks, the first and last column with centres in that range and
   // in the box (fmaxf and fminf pass a NaN of extreme ratios over: the box alone)
@@ -158,7 +158,7 @@ __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, 
   for (int r = 0; r < M::RH / M::ROWS; ++r) {
     const int c0 = __float2int_ru(fmaxf(lo + r * step, box0)), c1 = __float2int_rd(fminf(hi + r * step, box1));
     const unsigned xm = (kRow >> (M::RW - M::LPG * (c1 - c0 + 1))) << (M::LPG * c0);
-    m |= row0 <= r && r <= row1 && c0 <= c1 ? xm << (M::RW * r) : 0u;
+    m |= !(row0 > r) && !(r > row1) && c0 <= c1 ? xm << (M::RW * r) : 0u;
   }
   return m;
 }
