@@ -12,20 +12,14 @@
 // the size of a small splat.  The backward pass sums a Gaussian's gradient over
 // the group with shuffles and adds it to the global record with vector atomics.
 //
-// Both passes are bound by instruction issue (70% and 66% of cycles issue, the
-// ALU and FMA pipes 41% and 50% busy, DRAM 7%).  With one 8 x 8 block per warp
-// and one list for all 32 lanes, a splat of 4-5 px met 2.95 evaluated pixels
-// per blended one and each (warp, entry) hit paid its list handling and its
-// reduction for 16 blended pixels; lists per group evaluate 1.76 (forward) and
-// 1.96 (backward), and one reduction serves 16 Gaussians: 85 -> 64 us and
-// 168 -> 100 us at 1200 x 680 with 300k Gaussians, 811 -> 654 us and 1759 ->
-// 1110 us for five such views.
-#ifndef BWDP
-#define BWDP 4
-#endif
-#ifndef FWDP
-#define FWDP 4
-#endif
+// Both passes are bound by instruction issue (72% and 70% of cycles issue, the
+// ALU pipe 50% and 42% busy, the FMA pipe 39% and 43%, DRAM 6%; one launch at
+// 1200 x 680).  With one 8 x 8 block per warp and one list for all 32 lanes, a
+// splat of 4-5 px met 2.95 evaluated pixels per blended one and each (warp,
+// entry) hit paid its list handling and its reduction for 16 blended pixels;
+// lists per group evaluate 1.69 (forward), and one reduction serves 16
+// Gaussians: 85 -> 63 us and 168 -> 102 us at 1200 x 680 with 300k Gaussians, an
+// iteration of five such views 1927 -> 1302 us.
 #include <algorithm>
 #include <type_traits>
 
@@ -237,12 +231,11 @@ struct Walk {
     __syncwarp();  // the entries are stored before any lane reads them
     return warp_transpose(m, lane);
   }
-  __device__ __forceinline__ void push(unsigned mine, bool take = true) {  // the staged chunk's entries
+  __device__ __forceinline__ void push(unsigned mine) {  // the staged chunk's entries
     if (DIR > 0) {
       if (mine) met = top + 32 - __clz(mine);
       mine = __brev(mine);
     }
-    if (!take) mine = 0u;
     const int r = top - off;
     cur = r == 0 ? mine : cur;
     w1 = r == 32 ? mine : w1;
@@ -289,32 +282,27 @@ struct Walk {
   }
 };
 
-// Passes with one or two pixels per lane take a chunk by all lanes together where
-// most of its entries that meet the warp's region (meet) meet every block of it
-// (whole): the lanes' lists would be nearly the same, and the backward pass makes
-// one addition to a Gaussian's record per region instead of one per block.  With
-// four or eight pixels an addition the gradients' errors against 64 bits were up
-// to 1.75 times those with 64 (200 x 150, 2000 large splats; 1.03 to 1.07 for a
-// seeded map; means over 24 to 50 maps); now they are 0.95 to 1.05 times, with a
-// spread of 0.03 (200 x 150 to 500 x 400).  With one pixel per lane the backward
-// pass takes every chunk so, two entries at a time, since the few warps wait for
-// each other's exchanges: 97.4 -> 87.8 us an iteration for the former with the
-// ellipse's test of the rows, 150 -> 124 us for 5000 at 320 x 240.  It costs
-// small seeded maps 1 to 4% of an iteration (66 x 38, 896 Gaussians, 55.4 -> 58.4
-// us; 280 x 210, 12000, 66.0 -> 67.8).  With two pixels per lane from three
-// quarters of the entries (seven eighths: errors up to 1.25 at 280 x 210; half: 79
-// instead of 75 us for 20000 seeded ones at 320 x 240), forward from seven
-// eighths.  Not with four, whose additions are of eight pixels in large images
+// Backward passes with one or two pixels per lane take a chunk by all lanes
+// together where most of its entries that meet the warp's region (meet) meet
+// every block of it (whole): the groups' lists would be nearly the same, and
+// there is one addition to a Gaussian's record per region instead of one per
+// block.  With four or eight pixels an addition the gradients' errors against 64
+// bits were up to 1.75 times those with 64 (200 x 150, 2000 large splats; 1.03 to
+// 1.07 for a seeded map; means over 24 to 50 maps); now they are 0.95 to 1.05
+// times, with a spread of 0.03 (200 x 150 to 500 x 400).  With one pixel per lane
+// every chunk is taken so, two entries at a time, since the few warps wait for
+// each other's exchanges: the pass 45 -> 35 us for the former with the ellipse's
+// test of the rows, 64 -> 48 us for 5000 at 320 x 240.  It costs small seeded maps
+// 1 to 4% of an iteration (66 x 38, 896 Gaussians, 55.4 -> 58.4 us).  With two
+// pixels per lane from three quarters of the entries (seven eighths: errors up to
+// 1.25 at 280 x 210; half: 79 instead of 75 us for 20000 seeded ones at 320 x
+// 240).  Not with four, whose additions are of eight pixels in large images
 // (errors as with 64): 294 -> 295 us for 300k Gaussians, 1327 -> 1340 for five
 // views.
 template <int PPL>
 constexpr bool kTogether = PPL <= 2;
 template <int PPL>
-__device__ __forceinline__ bool together_fwd(unsigned meet, unsigned whole) {
-  return PPL == 1 ? 2 * __popc(whole) >= __popc(meet) : 8 * __popc(whole) >= 7 * __popc(meet);
-}
-template <int PPL>
-__device__ __forceinline__ bool together_bwd(unsigned meet, unsigned whole) {
+__device__ __forceinline__ bool together(unsigned meet, unsigned whole) {
   return PPL == 1 || 4 * __popc(whole) >= 3 * __popc(meet);
 }
 
@@ -505,74 +493,12 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
   }
   uint32_t n_blend = 0, n_visit = 0;
 
-  // one entry (each lane its own, or the same one for all), at place idx of the list
-  auto blend = [&](const Entry& en, int idx) {
-    const float4 ea = en.a, eb = en.b, ec = en.c;
-    const float dx = __fsub_rn(plx, ea.x);
-    const float t0 = __fmul_rn(ea.z, dx);
-    float al[2 * NP], in[2 * NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const f2x DY = f2_sub(f2_pack(ply[2 * p], ply[2 * p + 1]), f2_bcast(ea.y));
-      const f2x WQ = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
-      const f2x TQ = f2_mul(WQ, f2_bcast(eb.x));
-      const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ, TQ));
-      const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
-      al[2 * p] = ex2_approx(f2_lo(ARG));
-      al[2 * p + 1] = ex2_approx(f2_hi(ARG));
-      in[2 * p] = one_if_le(f2_lo(Q), eb.w);
-      in[2 * p + 1] = one_if_le(f2_hi(Q), eb.w);
-    }
-    if (eb.y > rp.log2_clamp) {
-#pragma unroll
-      for (int s = 0; s < 2 * NP; ++s) al[s] = fminf(rp.alpha_max, al[s]);
-    }
-    f2x AL[NP], TEST[NP];
-    float low = 1.f;
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      // alpha, exactly 0 (so that T, R, G, B and D stay as they are) outside the support
-      AL[p] = f2_mul(f2_pack(al[2 * p], al[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
-      TEST[p] = f2_mul(T[p], f2_sub(ONE2, AL[p]));
-      low = fminf(low, fminf(f2_lo(TEST[p]), f2_hi(TEST[p])));
-    }
-    if (COUNT) {
-#pragma unroll
-      for (int s = 0; s < PPL; ++s) {
-        n_visit += eb.w > 0.f && ply[s] != kInf ? 1u : 0u;
-        n_blend += in[s] > 0.f && (s & 1 ? f2_hi(TEST[s / 2]) : f2_lo(TEST[s / 2])) >= rp.t_eps ? 1u : 0u;
-      }
-    }
-    if (low < rp.t_eps) {  // a pixel stops in front of this entry
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const bool s0 = f2_lo(TEST[p]) < rp.t_eps, s1 = f2_hi(TEST[p]) < rp.t_eps;
-        AL[p] = f2_pack(s0 ? 0.f : f2_lo(AL[p]), s1 ? 0.f : f2_hi(AL[p]));
-        TEST[p] = f2_pack(s0 ? f2_lo(T[p]) : f2_lo(TEST[p]), s1 ? f2_hi(T[p]) : f2_hi(TEST[p]));
-        ply[2 * p] = s0 ? kInf : ply[2 * p];
-        ply[2 * p + 1] = s1 ? kInf : ply[2 * p + 1];
-        stop[2 * p] = s0 ? idx : stop[2 * p];
-        stop[2 * p + 1] = s1 ? idx : stop[2 * p + 1];
-      }
-    }
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const f2x W = f2_mul(AL[p], T[p]);
-      T[p] = TEST[p];
-      R[p] = f2_fma_s(W, ec.x, R[p]);
-      G[p] = f2_fma_s(W, ec.y, G[p]);
-      B[p] = f2_fma_s(W, ec.z, B[p]);
-      D[p] = f2_fma_s(W, eb.z, D[p]);
-    }
-  };
-
   if (walk.n > 0) {
     walk.begin();
     unsigned gone = 0u;  // 1: every pixel of the lane is done
-    unsigned held = 0u;  // a chunk whose entries all lanes take together
     for (;;) {
       while (__any_sync(kFull, walk.cur == 0u && walk.off < walk.top)) walk.step();
-      const bool can = walk.can_stage() && !held;
+      const bool can = walk.can_stage();
       if (can && __any_sync(kFull, (walk.cur | gone) == 0u)) {  // a lane is dry
         bool out = true;
 #pragma unroll
@@ -582,35 +508,73 @@ __device__ __forceinline__ void fwd_job(const RasterArgs& a, const RasterParams&
         gone = out ? 1u : 0u;
         unsigned m;
         bool wide;
-        const unsigned mine = walk.stage(rp, m, wide);
-        if constexpr (kTogether<PPL>) {
-          const unsigned whole = __ballot_sync(kFull, m == kFull);
-          if (whole) {
-            const unsigned meet = __ballot_sync(kFull, m != 0u);
-            if (together_fwd<PPL>(meet, whole)) held = meet;
-          }
-        }
-        walk.push(mine, !held);
+        walk.push(walk.stage(rp, m, wide));
         if (out) walk.drop();
         continue;
       }
-      int lim = walk.end;
-      if (!held) {
-        lim = walk.limit(can);
-        if (lim == walk.kEnd) break;
-        if (lim == walk.kAgain) continue;
-      } else if (!__any_sync(kFull, walk.cur != 0u)) {
-        const Entry* e = sm.e + ((walk.top - 32) & (kRing - 1));
-        for (; held; held &= held - 1u) {
-          const int j = __ffs(held) - 1;
-          blend(e[j], walk.top - 32 + j);
-        }
-        continue;
-      }
+      const int lim = walk.limit(can);
+      if (lim == walk.kEnd) break;
+      if (lim == walk.kAgain) continue;
       do {
         int idx;
         const Entry& en = sm.e[walk.take(idx)];
-        blend(en, idx);
+        const float4 ea = en.a, eb = en.b, ec = en.c;
+        const float dx = __fsub_rn(plx, ea.x);
+        const float t0 = __fmul_rn(ea.z, dx);
+        float al[2 * NP], in[2 * NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const f2x DY = f2_sub(f2_pack(ply[2 * p], ply[2 * p + 1]), f2_bcast(ea.y));
+          const f2x WQ = f2_fma(f2_bcast(ea.w), f2_bcast(dx), DY);
+          const f2x TQ = f2_mul(WQ, f2_bcast(eb.x));
+          const f2x Q = f2_fma(f2_bcast(t0), f2_bcast(t0), f2_mul(TQ, TQ));
+          const f2x ARG = f2_sub(f2_bcast(eb.y), Q);
+          al[2 * p] = ex2_approx(f2_lo(ARG));
+          al[2 * p + 1] = ex2_approx(f2_hi(ARG));
+          in[2 * p] = one_if_le(f2_lo(Q), eb.w);
+          in[2 * p + 1] = one_if_le(f2_hi(Q), eb.w);
+        }
+        if (eb.y > rp.log2_clamp) {
+#pragma unroll
+          for (int s = 0; s < 2 * NP; ++s) al[s] = fminf(rp.alpha_max, al[s]);
+        }
+        f2x AL[NP], TEST[NP];
+        float low = 1.f;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          // alpha, exactly 0 (so that T, R, G, B and D stay as they are) outside the support
+          AL[p] = f2_mul(f2_pack(al[2 * p], al[2 * p + 1]), f2_pack(in[2 * p], in[2 * p + 1]));
+          TEST[p] = f2_mul(T[p], f2_sub(ONE2, AL[p]));
+          low = fminf(low, fminf(f2_lo(TEST[p]), f2_hi(TEST[p])));
+        }
+        if (COUNT) {
+#pragma unroll
+          for (int s = 0; s < PPL; ++s) {
+            n_visit += eb.w > 0.f && ply[s] != kInf ? 1u : 0u;
+            n_blend += in[s] > 0.f && (s & 1 ? f2_hi(TEST[s / 2]) : f2_lo(TEST[s / 2])) >= rp.t_eps ? 1u : 0u;
+          }
+        }
+        if (low < rp.t_eps) {  // a pixel stops in front of this entry
+#pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const bool s0 = f2_lo(TEST[p]) < rp.t_eps, s1 = f2_hi(TEST[p]) < rp.t_eps;
+            AL[p] = f2_pack(s0 ? 0.f : f2_lo(AL[p]), s1 ? 0.f : f2_hi(AL[p]));
+            TEST[p] = f2_pack(s0 ? f2_lo(T[p]) : f2_lo(TEST[p]), s1 ? f2_hi(T[p]) : f2_hi(TEST[p]));
+            ply[2 * p] = s0 ? kInf : ply[2 * p];
+            ply[2 * p + 1] = s1 ? kInf : ply[2 * p + 1];
+            stop[2 * p] = s0 ? idx : stop[2 * p];
+            stop[2 * p + 1] = s1 ? idx : stop[2 * p + 1];
+          }
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const f2x W = f2_mul(AL[p], T[p]);
+          T[p] = TEST[p];
+          R[p] = f2_fma_s(W, ec.x, R[p]);
+          G[p] = f2_fma_s(W, ec.y, G[p]);
+          B[p] = f2_fma_s(W, ec.z, B[p]);
+          D[p] = f2_fma_s(W, eb.z, D[p]);
+        }
       } while (can ? !__any_sync(kFull, (walk.cur | gone) == 0u) : walk.any_up_to(lim));
     }
     cp_wait_all();
@@ -1008,7 +972,7 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
       if (whole) {
         const unsigned meet = __ballot_sync(kFull, m != 0u);
         const unsigned w = kTogether<PPL> ? __ballot_sync(kFull, m != 0u && wide) : whole;
-        if (kTogether<PPL> && together_bwd<PPL>(meet, whole)) {
+        if (kTogether<PPL> && together<PPL>(meet, whole)) {
           held = meet;
           mine = 0u;
         } else if (w) {  // (entry 31 comes first)
