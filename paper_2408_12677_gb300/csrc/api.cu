@@ -164,7 +164,7 @@ struct gs_ctx {
   int* big_diff = nullptr;        // difference grids of the projection's large rectangles, 0 between passes
                                   // (part of tcount's allocation)
   bool order_tiles = true;  // compute and use the visit order
-  bool persistent = true;   // raster passes as persistent grids pulling (tile, quadrant) jobs
+  bool persistent = true;   // raster passes as persistent grids pulling (tile, region) jobs
   int st_sh = 0;
   TileMap st_map{};
   int64_t st_pix_base[kMaxViews] = {};
@@ -785,7 +785,8 @@ gs_status bin_and_sort(gs_ctx* c, int n, const TileMap& map, cudaStream_t s, boo
                    ensure_buckets(c, T, (uint32_t)entries) == GS_OK &&
                    c->cap_bt * (int64_t)kLenClasses < ((int64_t)1 << 32);
     if (longest > tile_sort_capacity()) {
-      const bool cut = tiles_y && P <= 0xFFFFFFF0ll && P >= kPrefixMean * T;  // (more pairs are refused by the full binning)
+      // (more pairs than that are refused by the full binning)
+      const bool cut = tiles_y && P <= 0xFFFFFFF0ll && P >= kPrefixMean * T;
       if (cut && c->cut_wait > 0) {
         c->cut_wait -= 1;
       } else if (cut) {
@@ -1272,7 +1273,8 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
   const bool buckets = !c->sync && c->bucket_ok && (int64_t)L.tiles <= c->cap_bt;
   // rectangles of more than kHugeTiles tiles go to the difference grids
   bool grids = false;
-  for (int v = 0; v < V; ++v) grids = grids || (!buckets && (int64_t)L.map.tiles_x[v] * L.tiles_y[v] > (int64_t)kHugeTiles);
+  for (int v = 0; v < V && !buckets; ++v)
+    grids = grids || (int64_t)L.map.tiles_x[v] * L.tiles_y[v] > (int64_t)kHugeTiles;
   if (grids) {
     grid_layout(L.map, L.tiles_y, grid_base);
     pa.big_diff = c->big_diff;
@@ -1322,58 +1324,58 @@ gs_status render_fwd_views(gs_ctx* c, const gs_gaussians* g, int32_t V, const gs
                                  c->st_cut ? 0 : c->seen_longest);
 
   for (int attempt = 0;; ++attempt) {
-  RasterArgs ra = raster_args(c, cfg);
-  for (int v = 0; v < V; ++v) {
-    ra.v[v].color = color ? color[v] : nullptr;
-    ra.v[v].depth = depth ? depth[v] : nullptr;
-    ra.v[v].alpha = alpha ? alpha[v] : nullptr;
-  }
-  if (fl) {
-    ra.loss_partials = c->tile_loss;
-    ra.nvalid = c->d_nvalid;
-    ra.w_color = fl->w_color;
+    RasterArgs ra = raster_args(c, cfg);
     for (int v = 0; v < V; ++v) {
-      const int64_t np = (int64_t)cams[v].width * cams[v].height;
-      ra.v[v].trgb = fl->trgb[v];
-      ra.v[v].tdep = fl->tdep[v];
-      ra.v[v].loss_dc = c->dl_img + 4 * L.pix_base[v];
-      ra.v[v].loss_dd = c->dl_img + 4 * L.pix_base[v] + 3 * np;
+      ra.v[v].color = color ? color[v] : nullptr;
+      ra.v[v].depth = depth ? depth[v] : nullptr;
+      ra.v[v].alpha = alpha ? alpha[v] : nullptr;
     }
-  }
-  if (c->st_buckets) {  // visit order from the sort's class lists, recorded for the backward pass
-    ra.order = nullptr;
-    ra.cls_count = c->cls_count;
-    ra.cls_tiles = c->cls_tiles;
-    ra.cls_stride = (uint32_t)c->cap_bt;
-    ra.order_out = c->torder;
-  }
-  ra.zero_work = !c->fwd_work_zero;
-  {
-    StageTimer t(c, GS_STAGE_RASTER_FWD, s);
-    launch_raster_fwd(ra, c->T_final, c->last, c->counting ? c->d_evals : nullptr, s);
-  }
-  c->fwd_work_zero = false;
-  c->launches += 1;
-  GS_CHECK_LAUNCH(c, "raster_fwd");
-  if (!c->st_cut) break;
-  launch_raster_open(ra, c->last, c->pfx_cut, c->pfx_level, c->d_binstats + 4, s);
-  c->launches += 1;
-  GS_CHECK_LAUNCH(c, "raster_open");
-  GS_CUDA(c, cudaMemcpyAsync(c->h_pinned, c->d_binstats + 4, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(c, cudaStreamSynchronize(s));
-  const int64_t open_tiles = (int64_t)c->h_pinned[0];
-  if (open_tiles == 0) break;
-  // some list was cut too short: bin again with longer ones (the third time
-  // the open tiles' in full, which no pixel can exhaust), or all in full
-  if (attempt == 2) return fail(c, GS_ERR_CUDA, "a full list left a pixel open");
-  if (c->counting)
-    GS_CUDA(c, cudaMemcpyAsync(c->d_evals, c->d_evals + 2, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
-  if (fl) GS_CUDA(c, cudaMemsetAsync(c->d_nvalid, 0, kMaxViews * sizeof(uint32_t), s));
-  bool done = false;
-  const bool in_full = attempt == 1 && open_tiles * n_items > kLooks * c->st_pairs;
-  if (in_full) c->cut_wait = kCutWait;
-  else if ((st = bin_prefix(c, n_items, L.map, L.tiles_y, s, attempt + 1, &done)) != GS_OK) return st;
-  if (!done && (st = bin_and_sort_radix(c, n_items, L.map, s, c->pfx_sorted)) != GS_OK) return st;
+    if (fl) {
+      ra.loss_partials = c->tile_loss;
+      ra.nvalid = c->d_nvalid;
+      ra.w_color = fl->w_color;
+      for (int v = 0; v < V; ++v) {
+        const int64_t np = (int64_t)cams[v].width * cams[v].height;
+        ra.v[v].trgb = fl->trgb[v];
+        ra.v[v].tdep = fl->tdep[v];
+        ra.v[v].loss_dc = c->dl_img + 4 * L.pix_base[v];
+        ra.v[v].loss_dd = c->dl_img + 4 * L.pix_base[v] + 3 * np;
+      }
+    }
+    if (c->st_buckets) {  // visit order from the sort's class lists, recorded for the backward pass
+      ra.order = nullptr;
+      ra.cls_count = c->cls_count;
+      ra.cls_tiles = c->cls_tiles;
+      ra.cls_stride = (uint32_t)c->cap_bt;
+      ra.order_out = c->torder;
+    }
+    ra.zero_work = !c->fwd_work_zero;
+    {
+      StageTimer t(c, GS_STAGE_RASTER_FWD, s);
+      launch_raster_fwd(ra, c->T_final, c->last, c->counting ? c->d_evals : nullptr, s);
+    }
+    c->fwd_work_zero = false;
+    c->launches += 1;
+    GS_CHECK_LAUNCH(c, "raster_fwd");
+    if (!c->st_cut) break;
+    launch_raster_open(ra, c->last, c->pfx_cut, c->pfx_level, c->d_binstats + 4, s);
+    c->launches += 1;
+    GS_CHECK_LAUNCH(c, "raster_open");
+    GS_CUDA(c, cudaMemcpyAsync(c->h_pinned, c->d_binstats + 4, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    GS_CUDA(c, cudaStreamSynchronize(s));
+    const int64_t open_tiles = (int64_t)c->h_pinned[0];
+    if (open_tiles == 0) break;
+    // some list was cut too short: bin again with longer ones (the third time
+    // the open tiles' in full, which no pixel can exhaust), or all in full
+    if (attempt == 2) return fail(c, GS_ERR_CUDA, "a full list left a pixel open");
+    if (c->counting)
+      GS_CUDA(c, cudaMemcpyAsync(c->d_evals, c->d_evals + 2, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+    if (fl) GS_CUDA(c, cudaMemsetAsync(c->d_nvalid, 0, kMaxViews * sizeof(uint32_t), s));
+    bool done = false;
+    const bool in_full = attempt == 1 && open_tiles * n_items > kLooks * c->st_pairs;
+    if (in_full) c->cut_wait = kCutWait;
+    else if ((st = bin_prefix(c, n_items, L.map, L.tiles_y, s, attempt + 1, &done)) != GS_OK) return st;
+    if (!done && (st = bin_and_sort_radix(c, n_items, L.map, s, c->pfx_sorted)) != GS_OK) return st;
   }
   c->st_g = *g;
   for (int v = 0; v < V; ++v) {

@@ -19,7 +19,8 @@
 // raises its tile's level, and the binning is repeated: level 1 keeps as many
 // entries as the per-tile sort holds, level 2 all of them.  A level-2 tile's
 // list is gathered by one block that walks the items in depth order, so it
-// needs no sort.
+// needs no sort; where so many tiles are left that this would take longer, all
+// pairs are binned in full.
 #include <algorithm>
 
 #include "common.cuh"

@@ -221,8 +221,6 @@ __device__ __forceinline__ void block_count_tiles(uint32_t* __restrict__ counts,
   __syncthreads();  // s_cnt and s_box are reused by the next view
 }
 
-// One thread per Gaussian: its parameters are read once and projected into
-// every view of the batch (item v * n + i for view v).
 // The SH rows of a projection block in shared memory, copied in 16-byte pieces
 // of the global array whatever the slice's own place within 16 bytes (`shift`
 // floats): piece c holds the slice's floats 4 c - shift .. 4 c - shift + 3.  A
@@ -271,6 +269,8 @@ struct FwdSh {
   }
 };
 
+// One thread per Gaussian: its parameters are read once and projected into
+// every view of the batch (item v * n + i for view v).
 template <int D>
 __global__ void __launch_bounds__(kFwdThreads, 7) project_fwd_kernel(const __grid_constant__ ProjectArgs a,
                                                                   float4* __restrict__ feat,
