@@ -110,12 +110,14 @@ constexpr float kNanOpacity = 64.f;
 // centres of lane l's block.  The box holds every pixel the per-pixel test can
 // accept: q' <= min(qmax, log2 o - log2 alpha_min) is the ellipse
 // (i0 dx)^2 + (i1 (dy - k dx))^2 <= R2, with half-extents sqrt(R2) / i0 and
-// sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2), and per row of blocks only the ellipse's
-// extent over its pixel centres counts: the box of a thin slanted splat holds
-// many times the pixels that it reaches (300k faint needles of 100 px: backward 23
-// -> 4.9 ms, forward 2.3, with one list per warp 13.7 and 12.4; 20000 random
-// splats of up to 20:1 179 -> 150 and 291 -> 236 us; 300k seeded ones as before).  The widening covers float32 rounding
-// of the test and of the hardware square roots and reciprocals.  `wide`: the
+// sqrt(R2) sqrt(k^2 / i0^2 + 1 / i1^2), and in each half of the region's rows
+// only the ellipse's extent over their pixel centres counts: the box of a thin
+// slanted splat holds many times the pixels that it reaches (300k faint needles
+// of 100 px: backward 23 -> 4.9 ms, forward 2.3, with one list per warp 13.7 and
+// 12.4; 20000 random splats of up to 20:1 179 -> 150 and 291 -> 236 us; 300k
+// seeded ones as before; per row of blocks instead of per half: 0.5% slower over
+// 34 maps).  The widening covers float32 rounding of the test and of the hardware
+// square roots and reciprocals.  `wide`: the
 // box has more than 4 kWide pixels.  A NaN opacity (fminf passes it over in R2
 // and here) becomes one that is clamped wherever the splat reaches: the raster
 // loops multiply alpha by 0 outside the support, which a NaN would survive.
@@ -138,22 +140,27 @@ __device__ __forceinline__ unsigned make_entry(float4 f0, float4 f1, float4 f2, 
   // at height y from its centre the ellipse's x is within kx y +- hx
   const float u = inv0 * rs;
   const float kx = f1.y * u * u, hx = u * Rr * inv1 + 1e-3f + 4e-6f * ex;
-  // per row of blocks, the first and last column with centres in that range and
-  // in the box (fmaxf and fminf pass a NaN of extreme ratios over: the box alone)
-  constexpr float BW = M::LPG, BH = M::ROWS, NC = M::RW / M::LPG;
-  constexpr unsigned kRow = M::RW == 32 ? kFull : (1u << M::RW) - 1u;
+  // per half of the region's rows, the first and last column of blocks with
+  // centres in that range and in the box (fmaxf and fminf pass a NaN of extreme
+  // ratios over: the box alone), then the rows that the box meets
+  constexpr int NR = M::RH / M::ROWS, RPH = NR / 2;  // rows of blocks, of a half
+  constexpr float BW = M::LPG, BH = M::ROWS, HH = M::RH / 2, NC = M::RW / M::LPG;
+  constexpr unsigned kRow = (1u << M::RW) - 1u;
   const float rx = mlx - bx, ry = mly - by;
   const float box0 = fmaxf((rx - ex + 0.5f) / BW - 1.f, 0.f), box1 = fminf((rx + ex - 0.5f) / BW, NC - 1.f);
-  const float mid = rx + kx * (0.5f - ry), span = kx * (BH - 1.f), step = kx * (BH / BW);
+  const float mid = rx + kx * (0.5f - ry), span = kx * (HH - 1.f), step = kx * (HH / BW);
   const float lo = (mid + fminf(span, 0.f) - hx + 0.5f) / BW - 1.f, hi = (mid + fmaxf(span, 0.f) + hx - 0.5f) / BW;
-  const float row0 = (ry - ey + 0.5f) / BH - 1.f, row1 = (ry + ey - 0.5f) / BH;
+  const int r0 = __float2int_ru(fmaxf((ry - ey + 0.5f) / BH - 1.f, 0.f));
+  const int r1 = __float2int_rd(fminf((ry + ey - 0.5f) / BH, NR - 1.f));
   unsigned m = 0u;
 #pragma unroll
-  for (int r = 0; r < M::RH / M::ROWS; ++r) {
-    const int c0 = __float2int_ru(fmaxf(lo + r * step, box0)), c1 = __float2int_rd(fminf(hi + r * step, box1));
-    const unsigned xm = (kRow >> (M::RW - M::LPG * (c1 - c0 + 1))) << (M::LPG * c0);
-    m |= !(row0 > r) && !(r > row1) && c0 <= c1 ? xm << (M::RW * r) : 0u;
+  for (int h = 0; h < 2; ++h) {
+    const int c0 = __float2int_ru(fmaxf(lo + h * step, box0)), c1 = __float2int_rd(fminf(hi + h * step, box1));
+    unsigned xm = (kRow >> (M::RW - M::LPG * (c1 - c0 + 1))) << (M::LPG * c0);
+    if (RPH == 2) xm |= xm << M::RW;
+    m |= c0 <= c1 ? xm << (M::RW * RPH * h) : 0u;
   }
+  m = r0 <= r1 ? m & ((kFull >> (32 - M::RW * (r1 - r0 + 1))) << (M::RW * r0)) : 0u;
   return m;
 }
 
