@@ -605,7 +605,7 @@ constexpr uint32_t kPrefixTarget = 256, kPrefixRanks = 32768;
 // faint splats always need (training steps, cut / in full: 1752 x 1168, 1M
 // Gaussians, lists of 1191, opaque 1.88 / 1.35 ms; 1451, a tenth of the image
 // faint 1.95 / 1.64; 920, faint 6.1 / 3.4; 8 views of 640 x 480, 1031, faint 8.7 /
-// 4.8; 1955, opaque 1.83 / 1.75; 2452, opaque 0.98 / about 2.2).
+// 4.8; 1955, opaque 1.83 / 1.75; 2452, opaque 0.97 / 1.98).
 constexpr int64_t kPrefixMean = 2048;
 // A level-2 list costs a look at every item.  Where so many tiles are still open
 // after the second attempt that this takes longer than binning all pairs (kLooks
