@@ -220,10 +220,9 @@ struct Walk {
     g_next = id_at(0);
     fetch(0);
   }
-  // Converts the chunk at `top` and puts the following one into flight;
-  // returns its entries that meet the lane's group (bit i: entry i), in m the
+  // Converts the chunk at `top` and puts the following one into flight: in m the
   // blocks that the lane's entry meets, in wide whether it is wide.
-  __device__ __forceinline__ unsigned stage(const RasterParams& rp, unsigned& m, bool& wide) {
+  __device__ __forceinline__ void convert(const RasterParams& rp, unsigned& m, bool& wide) {
     cp_wait_all();
     Entry e;
     m = 0u;
@@ -236,6 +235,10 @@ struct Walk {
     if (m) sm->e[(top & (kRing - 1)) + lane] = e;
     fetch(top + 32);
     __syncwarp();  // the entries are stored before any lane reads them
+  }
+  // The same; returns the entries that meet the lane's group (bit i: entry i).
+  __device__ __forceinline__ unsigned stage(const RasterParams& rp, unsigned& m, bool& wide) {
+    convert(rp, m, wide);
     return warp_transpose(m, lane);
   }
   __device__ __forceinline__ void push(unsigned mine) {  // the staged chunk's entries
@@ -289,29 +292,24 @@ struct Walk {
   }
 };
 
-// Backward passes with one or two pixels per lane take a chunk by all lanes
-// together where most of its entries that meet the warp's region (meet) meet
-// every block of it (whole): the groups' lists would be nearly the same, and
-// there is one addition to a Gaussian's record per region instead of one per
-// block.  With four or eight pixels an addition the gradients' errors against 64
-// bits were up to 1.75 times those with 64 (200 x 150, 2000 large splats; 1.03 to
-// 1.07 for a seeded map; means over 24 to 50 maps); now they are 0.95 to 1.05
-// times, with a spread of 0.03 (200 x 150 to 500 x 400).  With one pixel per lane
-// every chunk is taken so, two entries at a time, since the few warps wait for
-// each other's exchanges: the pass 45 -> 35 us for the former with the ellipse's
-// test of the rows, 64 -> 48 us for 5000 at 320 x 240.  It costs small seeded maps
-// 1 to 4% of an iteration (66 x 38, 896 Gaussians, 55.4 -> 58.4 us).  With two
-// pixels per lane from three quarters of the entries (seven eighths: errors up to
-// 1.25 at 280 x 210; half: 79 instead of 75 us for 20000 seeded ones at 320 x
-// 240).  Not with four, whose additions are of eight pixels in large images
-// (errors as with 64): 294 -> 295 us for 300k Gaussians, 1327 -> 1340 for five
-// views.
+// Backward passes with one or two pixels per lane take entries by all lanes
+// together, with one addition to a Gaussian's record per region instead of one
+// per block.  With four or eight pixels an addition the gradients' errors against
+// 64 bits were up to 1.75 times those with 64 (200 x 150, 2000 large splats; 1.03
+// to 1.07 for a seeded map; means over 24 to 50 maps); now they are 0.92 to 1.04
+// times, with a spread of 0.03 (64 x 48 to 500 x 400).  With one pixel per lane
+// every chunk is taken so, in a walk without lists, two entries at a time, since
+// the few warps wait for each other's exchanges: the pass 45 -> 33 us for the
+// former (with the ellipse's test), an iteration 98 -> 85; seeded maps 60 -> 58 us
+// (200 x 150) and 54 -> 55 (66 x 38).  With two pixels per lane the chunks in which
+// three quarters of the entries that meet the region meet every block of it, the
+// groups' lists being nearly the same there: 64 -> 48 us for 5000 large splats at
+// 320 x 240 (seven eighths: errors up to 1.25 at 280 x 210; half: 79 instead of 75
+// us an iteration for 20000 seeded ones at 320 x 240).  Not with four, whose
+// additions are of eight pixels in large images (errors as with 64): 294 -> 295 us
+// for 300k Gaussians, 1327 -> 1340 for five views.
 template <int PPL>
 constexpr bool kTogether = PPL <= 2;
-template <int PPL>
-__device__ __forceinline__ bool together(unsigned meet, unsigned whole) {
-  return PPL == 1 || 4 * __popc(whole) >= 3 * __popc(meet);
-}
 
 // Slot kRing of a warp's entries: support radius -1, accepted by no pixel.
 __device__ __forceinline__ void init_warp_smem(WarpSmem& sm) {
@@ -955,13 +953,43 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
     v[3] = v[1] * dx;
     return g2d + 12 * (size_t)__float_as_uint(ec.w);
   };
+  // the entries `bits` of the chunk at `at` by all groups together, every entry on
+  // every block: each Gaussian's sums go over the whole warp and to its record
+  // once, not once per block; two at a time
+  auto walk_all = [&](unsigned bits, int at) {
+    const Entry* e = sm.e + (at & (kRing - 1));
+    const int i0 = walk.chunk(at);
+    while (bits) {
+      const int j = 31 - __clz(bits);
+      bits ^= 1u << j;
+      float v[10];
+      float* rec = sums(e[j], i0 + j, v);
+      if (bits) {
+        const int k = 31 - __clz(bits);
+        bits ^= 1u << k;
+        float u[10];
+        float* rec_u = sums(e[k], i0 + k, u);
+        warp_reduce_add10(v, u, lane, rec, rec_u);
+      } else {
+        warp_reduce_add10(v, lane, rec);
+      }
+    }
+  };
+  if constexpr (PPL == 1) {  // every chunk
+    for (; walk.top < walk.end; walk.top += 32) {
+      unsigned m;
+      bool wide;
+      walk.convert(rp, m, wide);
+      walk_all(__ballot_sync(kFull, m != 0u), walk.top);
+    }
+    cp_wait_all();
+    return;
+  }
   // A chunk taken together, and the entries of another from its first to its last
-  // wide one, are held back until the groups are
-  // done with what comes before, and then walked by all groups together, every
-  // entry on every block: each Gaussian's sums go over the whole warp and to its
-  // record once, not once per block (the nearest splats of a map of large ones
-  // cover the image: 257k additions to one record took 1.30 ms where the pass
-  // now takes 0.13).
+  // wide one, are held back until the groups are done with what comes before, and
+  // then walked by all groups together (the nearest splats of a map of large ones
+  // cover the image: 257k additions to one record took 1.30 ms where the pass now
+  // takes 0.13).
   unsigned held = 0u, rest = 0u;  // these entries; the group's entries of the chunk after them
   bool all = false;               // the groups have them as their own lists (four pixels per lane; a loop over
                                   // them made the pass 1.3 us slower, 106 -> 107.4)
@@ -974,12 +1002,12 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
       unsigned mine = walk.stage(rp, m, wide);
       const int over = walk.chunk(walk.top) + 32 - glast;  // entries behind every pixel of the group
       if (over > 0) mine = over < 32 ? mine & (kFull >> over) : 0u;
-      const unsigned whole = __ballot_sync(kFull, PPL == 1 ? m != 0u : kTogether<PPL> ? m == kFull : m != 0u && wide);
+      const unsigned whole = __ballot_sync(kFull, kTogether<PPL> ? m == kFull : m != 0u && wide);
       rest = 0u;
       if (whole) {
         const unsigned meet = __ballot_sync(kFull, m != 0u);
         const unsigned w = kTogether<PPL> ? __ballot_sync(kFull, m != 0u && wide) : whole;
-        if (kTogether<PPL> && together<PPL>(meet, whole)) {
+        if (kTogether<PPL> && 4 * __popc(whole) >= 3 * __popc(meet)) {
           held = meet;
           mine = 0u;
         } else if (w) {  // (entry 31 comes first)
@@ -999,23 +1027,8 @@ __device__ __forceinline__ void bwd_job(const RasterArgs& a, const RasterParams&
       if (lim == walk.kAgain) continue;
     } else if (!__any_sync(kFull, walk.cur != 0u)) {  // the held entries' turn, or they are done
       if constexpr (kTogether<PPL>) {
-        const Entry* e = sm.e + ((walk.top - 32) & (kRing - 1));
-        const int i0 = walk.chunk(walk.top - 32);
-        while (held) {
-          const int j = 31 - __clz(held);
-          held ^= 1u << j;
-          float v[10];
-          float* rec = sums(e[j], i0 + j, v);
-          if (held) {
-            const int k = 31 - __clz(held);
-            held ^= 1u << k;
-            float u[10];
-            float* rec_u = sums(e[k], i0 + k, u);
-            warp_reduce_add10(v, u, lane, rec, rec_u);
-          } else {
-            warp_reduce_add10(v, lane, rec);
-          }
-        }
+        walk_all(held, walk.top - 32);
+        held = 0u;
         walk.cur = rest;
       } else {
         walk.cur = all ? rest : held;
